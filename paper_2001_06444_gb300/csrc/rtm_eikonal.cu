@@ -10,14 +10,27 @@
 // marching reaches it in one ordered pass, and Gauss-Seidel sweeps in the four
 // diagonal directions reach it by iterating to a fixed point (Zhao 2005).
 //
-// The solver sweeps level by level: in the sweep towards (+z, +x) the nodes
-// with i + j = l depend only on level l - 1 (already updated in this sweep)
-// and on level l + 1 (from the previous sweep), exactly as in the sequential
-// row-by-row sweep, so each level is updated in parallel and the result is
-// that of the sequential sweep (Detrixhe, Gibou and Min 2013).  One CTA solves
-// one (velocity sample, source) problem: its traveltime field lives in shared
-// memory when it fits (about 56 K nodes), else in an L2-resident buffer.
-// Iterations (four sweeps each) stop when one changes no node, or at a cap.
+// Any order of updates in which every node sees each neighbour as the
+// sequential row-by-row sweep does (updated in this sweep, or from the
+// previous one) gives the sequential sweep's result bit for bit.
+//
+// k_eik_rows (every grid whose tile map fits, about 0.7 M nodes): each lane
+// owns R <= 4 consecutive rows, a warp up to 32 R rows, and walks tiles of R x
+// 4 nodes along them, one tile behind the lane of the rows before.  A tile's
+// neighbours above, below and beside come from the lane's registers and from
+// its neighbour lanes by shuffles, so a sweep has no barrier (grids of more
+// than 128 rows take several warps, joined every few tiles), and the next tiles'
+// fields and slowness load while the current one is updated.  Tiles none of
+// whose neighbours changed since their last update are not evaluated again
+// (they could not change), and a problem ends once no tile is left to
+// evaluate, instead of sweeping once more to find that nothing changes.
+//
+// k_eik_sweep (larger grids, and RTM_EIK_TILE): one CTA per problem, tiles on
+// one diagonal in parallel, a barrier per diagonal (Detrixhe, Gibou and Min
+// 2013).
+//
+// Either way the field lives in shared memory or in an L2-resident buffer, and
+// iterations (four sweeps each) stop at the fixed point, or at a cap.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +39,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "rtm_engine.h"
@@ -180,6 +194,408 @@ __global__ void k_eik_slowness(const float *vel, long long n, float *slow) {
     slow[k] = __frcp_rn(vel[k]);
 }
 
+// ------------------------------------------------- row-owning warps --
+
+// Geometry of k_eik_rows for an nz x nx grid: W warps of lanes that own R rows
+// each, NL lanes in all (NLp: rounded up to 8), NC tiles of 4 columns a row.
+struct RowGeo {
+  int R, W, NL, NLp, NC;
+  int PB;            // bytes of a lane's row of the tile map: PB - 1 is 4 x odd, so that lanes
+                     // one tile apart touch different banks in the sweeps of either family
+  int P;             // shared-memory field: floats per row (a multiple of 8: 16-byte accesses
+                     // of lanes R rows and one tile apart touch different banks)
+  long long quads;   // float4 of one skewed copy of the field: (NC + NL - 1) R NLp
+  size_t map_bytes, ring_bytes, field_bytes;  // shared memory: map, warp seams, field
+};
+
+constexpr int kRowGap = 4;    // tiles between the barriers of a CTA of several warps
+constexpr int kRowRing = 16;  // tiles of a seam's ring (> kRowGap + 1 in flight)
+constexpr size_t kRowMap = 64 << 10;  // largest tile map (bytes)
+constexpr int kRowMaxWarps = 12;  // of a CTA: 1536 rows
+constexpr int kRowWarps = 8;  // resident warps an SM needs for shared-memory fields to win
+
+RowGeo row_geo(int nz, int nx) {
+  RowGeo g;
+  g.W = (nz + 127) / 128;
+  g.R = (nz + 32 * g.W - 1) / (32 * g.W);
+  g.NL = (nz + g.R - 1) / g.R;
+  g.W = (g.NL + 31) / 32;
+  g.NLp = (g.NL + 7) / 8 * 8;
+  g.NC = (nx + 3) / 4;
+  g.PB = (g.NC + 7) / 8 * 8 + 5;
+  g.P = (4 * g.NC + 7) / 8 * 8;
+  g.quads = (long long)(g.NC + g.NL - 1) * g.R * g.NLp;
+  g.map_bytes = ((size_t)g.NL * g.PB + 15) / 16 * 16;
+  g.ring_bytes = g.W > 1 ? (size_t)(g.W - 1) * kRowRing * 20 : 0;
+  g.field_bytes = (size_t)g.NL * g.R * g.P * 4;
+  return g;
+}
+
+struct RowArgs {
+  EikArgs e;
+  RowGeo g;
+  const float4 *slow_a, *slow_b;  // [nsample][quads] skewed slowness (+inf outside the grid)
+  float4 *work;                   // off chip: [problems][2][quads] both skewed copies of T
+  int p0, s0;                     // first problem of this launch, first sample of slow_a / slow_b
+};
+
+// The two skewed layouts of a grid's tiles: tile (lane g, column c), row r of
+// the lane at ((c + g) R + r) NLp + g (family A) or ((c + NL-1-g) R + r) NLp + g
+// (family B).  The sweeps (+z, +x) and (-z, -x) hold lanes at one c + g, the
+// other two at one c - g, so each reads whole lines of its family's copy:
+// 4 wavefronts a load instruction instead of 32 from the row-major field.  A
+// changed tile is written to both copies.
+__global__ void k_eik_skew(const float *vel, int nz, int nx, RowGeo g, float4 *slow_a,
+                           float4 *slow_b) {
+  const float *v = vel + (long long)blockIdx.y * nz * nx;
+  float4 *oa = slow_a + blockIdx.y * g.quads, *ob = slow_b + blockIdx.y * g.quads;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < g.quads;
+       q += (long long)gridDim.x * blockDim.x) {
+    const int lane = (int)(q % g.NLp);
+    const long long lr = q / g.NLp;
+    const int r = (int)(lr % g.R), l = (int)(lr / g.R);
+    const int row = lane * g.R + r;
+#pragma unroll
+    for (int fam = 0; fam < 2; ++fam) {
+      const int c = l - (fam ? g.NL - 1 - lane : lane);
+      float s[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const bool in = lane < g.NL && row < nz && c >= 0 && 4 * c + e < nx;
+        s[e] = in ? __frcp_rn(v[(long long)row * nx + 4 * c + e]) : kInf;
+      }
+      (fam ? ob : oa)[q] = make_float4(s[0], s[1], s[2], s[3]);
+    }
+  }
+}
+
+__device__ __forceinline__ float &el(float4 &v, int e) { return reinterpret_cast<float *>(&v)[e]; }
+
+// A problem as its CTA sees it.
+struct RowProblem {
+  const float4 *sa, *sb;  // slowness
+  float4 *ta, *tb;        // off-chip copies of T
+  float *st;              // shared-memory T [NL R][P]
+  unsigned char *map;     // [NL][PB] 1: the tile has to be evaluated
+  float4 *ring;           // [W-1][kRowRing] last rows handed over a seam
+  int *ringf;             // [W-1][kRowRing] and whether they changed
+};
+
+// update() without branches, for a chain of dependent updates: the expressions
+// are the same, so are the bits (the root's argument is at least 1e-30, where
+// the flushing reciprocal square root equals the plain one).  ISO: dz == dx.
+template <bool ISO>
+__device__ __forceinline__ float update_flat(float a, float b, float s, const EikArgs &A) {
+  const float u1 = fminf(a, b), u2 = fmaxf(a, b);
+  float h1 = A.dz, w1 = A.wz, w2 = A.wz;
+  if (!ISO) {
+    const bool vz = a <= b;
+    h1 = vz ? A.dz : A.dx;
+    w1 = vz ? A.wz : A.wx;
+    w2 = vz ? A.wx : A.wz;
+  }
+  const float t1 = u1 + s * h1;
+  const float d = u1 - u2;
+  const float disc = fmaxf(A.wsum * (s * s) - A.wprod * (d * d), 1e-30f);
+  float rs;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(disc));
+  const float two = (w1 * u1 + w2 * u2 + disc * rs) * A.inv_wsum;
+  return t1 <= u2 ? t1 : two;
+}
+
+// What a sweep leaves for the next ones.
+struct RowLeft {
+  bool changed = false;  // a node changed
+  bool map = true;       // tiles are left to evaluate
+  int lo = 0, hi = -1;   // this lane's first and last column with one (one warp only)
+};
+
+// One sweep.  FZ / FX: towards +z / +x.  Order and columns below count in the
+// sweep's direction.  A problem of one warp starts at the first tile left to
+// evaluate and stops behind the last.
+template <int R, bool RES, bool ISO, bool FZ, bool FX>
+__device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, const EikArgs &A,
+                                          RowLeft &B) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = threadIdx.x;
+  const bool own = gl < g.NL;
+  const int NC = g.NC, W = g.W;
+  const int lastlane = min(31, g.NL - 1 - 32 * warp);
+  const int seam_in = FZ ? warp - 1 : warp;        // seam to the warp of the rows before
+  const int seam_out = FZ ? warp : warp - 1;       // ... and after
+  const bool has_in = W > 1 && (FZ ? warp > 0 : warp < W - 1);
+  const bool has_out = W > 1 && (FZ ? warp < W - 1 : warp > 0);
+  const bool first = lane == (FZ ? 0 : lastlane), last = lane == (FZ ? lastlane : 0);
+  const int ko = FZ ? gl : g.NL - 1 - gl;
+  const int start = ko + kRowGap * (FZ ? warp : W - 1 - warp);
+  const int pl = FZ ? max(lane - 1, 0) : min(lane + 1, 31);   // lanes before and after
+  const int sl_ = FZ ? min(lane + 1, 31) : max(lane - 1, 0);
+  constexpr int r0 = FZ ? 0 : R - 1, r1 = FZ ? R - 1 : 0;     // first and last row of a tile
+  constexpr bool FA = FZ == FX;                               // family of this sweep
+  const int steps = NC + g.NL - 1 + kRowGap * (W - 1) + 1;
+  // the first step with a tile to evaluate, and the last one known now
+  int l0 = 0, l1 = steps;
+  if (W == 1) {
+    const bool some = B.hi >= B.lo;
+    l0 = __reduce_min_sync(0xffffffffu, some ? start + (FX ? B.lo : NC - 1 - B.hi) : steps);
+    l1 = __reduce_max_sync(0xffffffffu, some ? start + (FX ? B.hi : NC - 1 - B.lo) : 0);
+  }
+  B.lo = NC;
+  B.hi = -1;
+  const float4 *S = FA ? Q.sa : Q.sb;
+  float4 *T = FA ? Q.ta : Q.tb;
+  const int sk = FA ? gl : g.NL - 1 - gl;
+  const int rowq = R * g.NLp;
+  const float4 inf4 = make_float4(kInf, kInf, kInf, kInf);
+
+  auto cp_of = [&](int c) { return FX ? c : NC - 1 - c; };
+  auto idx = [&](int c) { return (long long)(cp_of(c) + sk) * rowq + gl; };
+  auto load_t = [&](int c, float4 (&t)[R]) {
+    if (own && c >= 0 && c < NC) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        t[r] = RES ? *reinterpret_cast<const float4 *>(Q.st + (size_t)(gl * R + r) * g.P + 4 * cp_of(c))
+                   : T[idx(c) + r * g.NLp];
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) t[r] = inf4;
+    }
+  };
+  auto load_s = [&](int c, float4 (&t)[R]) {
+    if (own && c >= 0 && c < NC) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) t[r] = __ldg(S + idx(c) + r * g.NLp);
+    }
+  };
+  // first row of the lane after the seam at column c (from the previous sweep)
+  auto load_b = [&](int c) {
+    float4 t = inf4;
+    if (last && has_out && c >= 0 && c < NC) {
+      const int g2 = FZ ? gl + 1 : gl - 1;
+      if (RES)
+        t = *reinterpret_cast<const float4 *>(Q.st + (size_t)(g2 * R + r0) * g.P + 4 * cp_of(c));
+      else
+        t = T[((long long)(cp_of(c) + (FA ? g2 : g.NL - 1 - g2)) * R + r0) * g.NLp + g2];
+    }
+    return t;
+  };
+  unsigned char *map = Q.map + (size_t)(own ? gl : 0) * g.PB;
+
+  float4 cur[R], nxt[R], pft[R], sc[R], sn[R], bnx = inf4;
+  float carry[R];      // the row's neighbour behind (updated in this sweep)
+  float4 prev;         // last row of the tile before
+#pragma unroll
+  for (int r = 0; r < R; ++r) sc[r] = sn[r] = inf4;
+  load_t(l0 - 1 - start, cur);
+  load_t(l0 - start, nxt);
+  load_t(l0 + 1 - start, pft);
+  load_s(l0 - start, sn);
+  prev = cur[r1];
+  if (W > 1) bnx = load_b(l0 - start);
+  unsigned mnext = 0;
+  if (own && l0 - start >= 0 && l0 - start < NC) mnext = map[cp_of(l0 - start)];
+  bool nd = false, pend = false, any_ch = false, any_map = false;
+  unsigned chb = 0;  // lanes that changed in the step before
+#pragma unroll 1
+  for (int l = l0; l < steps; ++l) {
+    const int c = l - start;
+    const bool in = own && c >= 0 && c < NC;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      carry[r] = FX ? cur[r].w : cur[r].x;
+      cur[r] = nxt[r];
+      nxt[r] = pft[r];
+      sc[r] = sn[r];
+    }
+    const float4 bcur = bnx;
+    load_t(c + 2, pft);
+    load_s(c + 1, sn);
+    if (W > 1) bnx = load_b(c + 1);
+    bool act = in && (mnext || nd);
+    mnext = 0;
+    if (own && c + 1 >= 0 && c + 1 < NC) mnext = map[cp_of(c + 1)];
+    float4 seam = inf4;
+    if (W > 1 && has_in && first && in) {
+      const int k = seam_in * kRowRing + (c & (kRowRing - 1));
+      seam = Q.ring[k];
+      act = act || Q.ringf[k];
+    }
+    bool ch = false;
+    if (__any_sync(0xffffffffu, act)) {
+      // the tile's neighbours across lanes: the rows before at this column,
+      // updated (that lane was here one step ago), and the rows after, old
+      float4 bef, aft;
+      bef.x = __shfl_sync(0xffffffffu, prev.x, pl);
+      bef.y = __shfl_sync(0xffffffffu, prev.y, pl);
+      bef.z = __shfl_sync(0xffffffffu, prev.z, pl);
+      bef.w = __shfl_sync(0xffffffffu, prev.w, pl);
+      aft.x = __shfl_sync(0xffffffffu, nxt[r0].x, sl_);
+      aft.y = __shfl_sync(0xffffffffu, nxt[r0].y, sl_);
+      aft.z = __shfl_sync(0xffffffffu, nxt[r0].z, sl_);
+      aft.w = __shfl_sync(0xffffffffu, nxt[r0].w, sl_);
+      if (first) bef = seam;
+      if (last) aft = bcur;
+      if (act) {
+#pragma unroll
+        for (int rr = 0; rr < R; ++rr) {
+          const int r = FZ ? rr : R - 1 - rr;
+#pragma unroll
+          for (int cc = 0; cc < 4; ++cc) {
+            const int e = FX ? cc : 3 - cc;
+            const float zb = rr > 0 ? el(cur[FZ ? r - 1 : r + 1], e) : el(bef, e);
+            const float za = rr < R - 1 ? el(cur[FZ ? r + 1 : r - 1], e) : el(aft, e);
+            const float xb = cc > 0 ? el(cur[r], FX ? e - 1 : e + 1) : carry[r];
+            const float xa = cc < 3 ? el(cur[r], FX ? e + 1 : e - 1) : (FX ? nxt[r].x : nxt[r].w);
+            const float v = update_flat<ISO>(fminf(zb, za), fminf(xb, xa), el(sc[r], e), A);
+            ch |= v < el(cur[r], e);
+            el(cur[r], e) = fminf(el(cur[r], e), v);
+          }
+        }
+        if (ch) {
+          if (RES) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+              *reinterpret_cast<float4 *>(Q.st + (size_t)(gl * R + r) * g.P + 4 * cp_of(c)) = cur[r];
+          } else {
+            const long long ia = (long long)(cp_of(c) + gl) * rowq + gl;
+            const long long ib = (long long)(cp_of(c) + g.NL - 1 - gl) * rowq + gl;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              Q.ta[ia + r * g.NLp] = cur[r];
+              Q.tb[ib + r * g.NLp] = cur[r];
+            }
+          }
+        }
+      }
+    }
+    prev = cur[r1];
+    if (W > 1 && has_out && last && in) {  // hand the last row over the seam
+      const int k = seam_out * kRowRing + (c & (kRowRing - 1));
+      Q.ring[k] = cur[r1];
+      Q.ringf[k] = ch;
+    }
+    // what this step's changes leave to evaluate: the lane before changed its
+    // next column (evaluated in this sweep), this lane's next column
+    // likewise; the column behind is final for this sweep
+    const unsigned chm = __ballot_sync(0xffffffffu, ch);
+    const bool ch_b = !first && ((chm >> pl) & 1u), ch_a = !last && ((chm >> sl_) & 1u);
+    nd = ch || ch_b;
+    const bool left = pend || ch || ch_a;
+    if (own && c >= 1 && c <= NC) {
+      const int cp = cp_of(c - 1);
+      map[cp] = left;
+      any_map |= left;
+      if (left) {
+        B.lo = min(B.lo, cp);
+        B.hi = max(B.hi, cp);
+      }
+    }
+    if (W > 1 && has_in && first && ch) {  // the rows before passed this column already
+      Q.map[(size_t)(FZ ? gl - 1 : gl + 1) * g.PB + cp_of(c)] = 1;
+      any_map = true;
+    }
+    pend = ch;
+    any_ch |= ch;
+    if (W > 1) {
+      if ((l & (kRowGap - 1)) == kRowGap - 1) __syncthreads();
+    } else if (l > l1 && !(chm | chb)) {
+      break;
+    }
+    chb = chm;
+  }
+  if (W > 1) {
+    B.changed |= __syncthreads_or(any_ch) != 0;
+    B.map = __syncthreads_or(any_map) != 0;
+  } else {
+    __syncwarp();
+    B.changed |= __any_sync(0xffffffffu, any_ch) != 0;
+    B.map = __any_sync(0xffffffffu, any_map) != 0;
+  }
+}
+
+template <int R, bool RES, bool ISO>
+__global__ void __launch_bounds__(32 * kRowMaxWarps) k_eik_rows(const __grid_constant__ RowArgs A) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  const RowGeo &g = A.g;
+  const EikArgs &E = A.e;
+  const int p = A.p0 + blockIdx.x, sample = p / E.nsrc, src = p % E.nsrc;
+  const int tid = threadIdx.x, nth = blockDim.x;
+  RowProblem Q;
+  Q.map = s_raw;
+  Q.ring = reinterpret_cast<float4 *>(s_raw + g.map_bytes);
+  Q.ringf = reinterpret_cast<int *>(Q.ring + (g.W - 1) * kRowRing);
+  Q.st = reinterpret_cast<float *>(s_raw + g.map_bytes + (g.ring_bytes + 15) / 16 * 16);
+  Q.sa = A.slow_a + (sample - A.s0) * g.quads;
+  Q.sb = A.slow_b + (sample - A.s0) * g.quads;
+  Q.ta = RES ? nullptr : A.work + (long long)blockIdx.x * 2 * g.quads;
+  Q.tb = RES ? nullptr : Q.ta + g.quads;
+  const float4 inf4 = make_float4(kInf, kInf, kInf, kInf);
+  for (int k = tid; k < (int)(g.map_bytes / 4); k += nth) reinterpret_cast<unsigned *>(Q.map)[k] = 0;
+  if (RES) {
+    float4 *t = reinterpret_cast<float4 *>(Q.st);
+    for (int k = tid; k < (int)(g.field_bytes / 16); k += nth) t[k] = inf4;
+  } else {
+    for (long long k = tid; k < 2 * g.quads; k += nth) Q.ta[k] = inf4;
+  }
+  __syncthreads();
+  const int iz = E.src[2 * src], ix = E.src[2 * src + 1];
+  const int gs = iz / R, rs = iz - gs * R, cs = ix >> 2;
+  auto qa = [&](int lane, int r, int c) { return ((long long)(c + lane) * R + r) * g.NLp + lane; };
+  auto qb = [&](int lane, int r, int c) {
+    return ((long long)(c + g.NL - 1 - lane) * R + r) * g.NLp + lane;
+  };
+  if (tid == 0) {
+    if (RES) {
+      Q.st[(size_t)iz * g.P + ix] = 0.0f;
+    } else {
+      reinterpret_cast<float *>(Q.ta + qa(gs, rs, cs))[ix & 3] = 0.0f;
+      reinterpret_cast<float *>(Q.tb + qb(gs, rs, cs))[ix & 3] = 0.0f;
+    }
+    Q.map[(size_t)gs * g.PB + cs] = 1;
+    if (gs > 0) Q.map[(size_t)(gs - 1) * g.PB + cs] = 1;
+    if (gs + 1 < g.NL) Q.map[(size_t)(gs + 1) * g.PB + cs] = 1;
+    if (cs > 0) Q.map[(size_t)gs * g.PB + cs - 1] = 1;
+    if (cs + 1 < g.NC) Q.map[(size_t)gs * g.PB + cs + 1] = 1;
+  }
+  __syncthreads();
+  // the four diagonal directions: (+z, +x), (+z, -x), (-z, -x), (-z, +x); an
+  // iteration that changes nothing ends the solve, and an empty map means
+  // that the rest of this iteration and the next one change nothing
+  RowLeft B;
+  if (tid < g.NL) {
+    B.lo = tid == gs ? max(cs - 1, 0) : cs;
+    B.hi = tid == gs ? min(cs + 1, g.NC - 1) : (abs(tid - gs) == 1 ? cs : -1);
+  }
+  int it = 0;
+  bool converged = false;
+  for (; it < E.max_iter; ++it) {
+    B.changed = false;
+    if (B.map) row_sweep<R, RES, ISO, true, true>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, true, false>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, false, false>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, false, true>(Q, g, E, B);
+    if (!B.changed) {
+      converged = true;
+      break;
+    }
+  }
+  if (tid == 0) E.iters[p] = converged ? it + 1 : -1;
+  __syncthreads();
+  auto value = [&](int i, int j) {
+    if (RES) return Q.st[(size_t)i * g.P + j];
+    const int lane = i / R;
+    return reinterpret_cast<const float *>(Q.ta + qa(lane, i - lane * R, j >> 2))[j & 3];
+  };
+  if (E.times) {
+    float *out = E.times + (long long)p * E.nrec;
+    for (int r = tid; r < E.nrec; r += nth) out[r] = value(E.rec[2 * r], E.rec[2 * r + 1]);
+  }
+  if (E.fields) {
+    float *out = E.fields + (long long)p * E.nz * E.nx;
+    for (int i = 0; i < E.nz; ++i)
+      for (int j = tid; j < E.nx; j += nth) out[(long long)i * E.nx + j] = value(i, j);
+  }
+}
+
 }  // namespace
 
 namespace rtm {
@@ -192,12 +608,9 @@ size_t eik_resident_limit() {
   return (size_t)std::max(0, optin - 1024);
 }
 
-cudaError_t launch_eikonal(const float *slow, int nsample, int nz, int nx, double dz, double dx,
-                           int nsrc, const int *src, int nrec, const int *rec, int max_iter,
-                           float *times, float *fields, int *iters, bool resident,
-                           cudaStream_t st) {
+static EikArgs eik_args(int nz, int nx, double dz, double dx, int nsrc, const int *src, int nrec,
+                        const int *rec, int max_iter, float *times, float *fields, int *iters) {
   EikArgs A{};
-  A.slow = slow;
   A.nz = nz;
   A.nx = nx;
   A.nsrc = nsrc;
@@ -215,6 +628,103 @@ cudaError_t launch_eikonal(const float *slow, int nsample, int nz, int nx, doubl
   A.fields = fields;
   A.max_iter = max_iter;
   A.iters = iters;
+  return A;
+}
+
+// The row-owning solver over all problems.  vel: device.  `work` and `slow`
+// hold one group of samples (or, for a sample of many sources, a part of its
+// problems) at a time: RowPlan.
+struct RowPlan {
+  RowGeo g;
+  bool resident = false;
+  size_t smem = 0;
+  int group = 1;         // samples whose skewed slowness is held at once
+  long long chunk = 1;   // problems of one launch
+  size_t slow_bytes = 0, work_bytes = 0;
+};
+
+// Off-chip fields and slowness stay within about this much scratch.
+constexpr size_t kRowScratch = size_t(2) << 30;
+
+// False: the grid's tile map is too large (k_eik_sweep solves it).
+static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
+                     size_t smem_cta, size_t smem_sm) {
+  if ((long long)((nz + 3) / 4) * ((nx + 3) / 4) > (long long)kRowMap) return false;
+  p.g = row_geo(nz, nx);
+  const RowGeo &g = p.g;
+  if (g.W > kRowMaxWarps || g.map_bytes > kRowMap) return false;
+  const size_t base = g.map_bytes + (g.ring_bytes + 15) / 16 * 16;
+  const long long problems = (long long)nsample * nsrc;
+  p.resident = false;
+  if (!(flags & RTM_EIK_OFFCHIP) && base + g.field_bytes <= smem_cta) {
+    const long long per_sm =
+        std::min<long long>(32 / g.W, (long long)(smem_sm / (base + g.field_bytes + 1024)));
+    p.resident = (flags & RTM_EIK_SHARED) || problems <= per_sm * sms || per_sm * g.W >= kRowWarps;
+  }
+  p.smem = base + (p.resident ? g.field_bytes : 0);
+  const size_t per = 2 * (size_t)g.quads * sizeof(float4);  // both copies
+  const size_t per_sample = per + (p.resident ? 0 : per * nsrc);
+  p.group = (int)std::max<size_t>(1, std::min<size_t>(nsample, kRowScratch / per_sample));
+  p.chunk = (long long)p.group * nsrc;
+  if (!p.resident)
+    p.chunk = std::max<long long>(1, std::min<long long>(p.chunk, (long long)(kRowScratch / per)));
+  p.slow_bytes = per * p.group;
+  p.work_bytes = p.resident ? 16 : per * (size_t)p.chunk;
+  return true;
+}
+
+static cudaError_t launch_eik_rows(const RowPlan &P, const float *vel, int nsample,
+                                   const EikArgs &E, float4 *slow, float4 *work, cudaStream_t st) {
+  RowArgs A{};
+  A.e = E;
+  A.g = P.g;
+  A.slow_a = slow;
+  A.slow_b = slow + (long long)P.group * P.g.quads;
+  A.work = work;
+  auto run = [&](auto kernel, unsigned n) -> cudaError_t {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)P.smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<n, 32 * P.g.W, P.smem, st>>>(A);
+    return cudaGetLastError();
+  };
+  const bool iso = E.dz == E.dx;
+  auto go = [&](auto rows, unsigned n) -> cudaError_t {
+    constexpr int R = decltype(rows)::value;
+    if (P.resident) return iso ? run(k_eik_rows<R, true, true>, n) : run(k_eik_rows<R, true, false>, n);
+    return iso ? run(k_eik_rows<R, false, true>, n) : run(k_eik_rows<R, false, false>, n);
+  };
+  for (int s0 = 0; s0 < nsample; s0 += P.group) {
+    const int ns = std::min(P.group, nsample - s0);
+    const unsigned bx = (unsigned)std::min<long long>((P.g.quads + 255) / 256, 1024);
+    for (int y0 = 0; y0 < ns; y0 += 65535) {
+      const long long at = (long long)y0 * P.g.quads;
+      k_eik_skew<<<dim3(bx, std::min(65535, ns - y0)), 256, 0, st>>>(
+          vel + (long long)(s0 + y0) * E.nz * E.nx, E.nz, E.nx, P.g, slow + at,
+          slow + (long long)P.group * P.g.quads + at);
+    }
+    A.s0 = s0;
+    const long long p1 = (long long)(s0 + ns) * E.nsrc;
+    for (long long p0 = (long long)s0 * E.nsrc; p0 < p1; p0 += P.chunk) {
+      A.p0 = (int)p0;
+      const unsigned n = (unsigned)std::min(P.chunk, p1 - p0);
+      cudaError_t e = cudaErrorInvalidValue;
+      switch (P.g.R) {
+        case 1: e = go(std::integral_constant<int, 1>(), n); break;
+        case 2: e = go(std::integral_constant<int, 2>(), n); break;
+        case 3: e = go(std::integral_constant<int, 3>(), n); break;
+        case 4: e = go(std::integral_constant<int, 4>(), n); break;
+      }
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaGetLastError();
+}
+
+static cudaError_t launch_eikonal(EikArgs A, const float *slow, int nsample, bool resident,
+                                  cudaStream_t st) {
+  A.slow = slow;
+  const int nz = A.nz, nx = A.nx, nsrc = A.nsrc;
   const long long problems = (long long)nsample * nsrc;
   if (problems > 0x7fffffffll) return cudaErrorInvalidValue;
   // tile shape: 2 x 2 (a short chain of dependent updates per thread, half
@@ -250,7 +760,7 @@ cudaError_t launch_eikonal(const float *slow, int nsample, int nz, int nx, doubl
   }
 }
 
-cudaError_t launch_eik_slowness(const float *vel, long long n, float *slow, cudaStream_t st) {
+static cudaError_t launch_eik_slowness(const float *vel, long long n, float *slow, cudaStream_t st) {
   const long long blocks = std::min<long long>((n + 255) / 256, 152 * 32);
   k_eik_slowness<<<(unsigned)std::max<long long>(1, blocks), 256, 0, st>>>(vel, n, slow);
   return cudaGetLastError();
@@ -295,7 +805,7 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   cudaStream_t st = (cudaStream_t)stream;
   const long long N = (long long)nz * nx, problems = (long long)nsample * nsrc;
   const size_t vbytes = (size_t)nsample * N * 4;
-  DevBuf dvel, dslow, dtab, dtimes, dfields, diters, drng;
+  DevBuf dvel, dslow, dwork, dtab, dtimes, dfields, diters, drng;
   const float *v = vel;
   if (!is_device_ptr(vel)) {
     EIK_CU(dvel.alloc(ctx, vbytes, st));
@@ -314,8 +824,6 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
     if (out[2])
       return fail(ctx, RTM_ERR_ARG, "%u velocity values are non-positive or not finite", out[2]);
   }
-  EIK_CU(dslow.alloc(ctx, vbytes, st));
-  EIK_CU(launch_eik_slowness(v, (long long)nsample * N, dslow.as<float>(), st));
   std::vector<int> tab(2 * (size_t)(nsrc + nrec));
   for (int k = 0; k < nsrc; ++k) {
     tab[2 * k] = src_iz[k];
@@ -327,8 +835,13 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   }
   EIK_CU(dtab.alloc(ctx, tab.size() * 4, st));
   EIK_CU(cudaMemcpyAsync(dtab.p, tab.data(), tab.size() * 4, cudaMemcpyHostToDevice, st));
-  int sms = 0;
+  int sms = 0, smem_cta = 0, smem_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  cudaDeviceGetAttribute(&smem_cta, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
+  RowPlan plan;
+  const bool rows = !getenv("RTM_EIK_TILE") && row_plan(plan, nz, nx, nsample, nsrc, flags, sms,
+                                                        (size_t)smem_cta, (size_t)smem_sm);
   const bool fits = (size_t)N * 4 <= eik_resident_limit();
   const bool resident = fits && !(flags & RTM_EIK_OFFCHIP) &&
                         ((flags & RTM_EIK_SHARED) || problems <= (long long)sms);
@@ -339,11 +852,18 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
     dt = dtimes.as<float>();
   }
   float *df = fields;
-  if ((fields && !is_device_ptr(fields)) || (!fields && !resident)) {
+  if ((fields && !is_device_ptr(fields)) || (!fields && !rows && !resident)) {
     EIK_CU(dfields.alloc(ctx, fbytes, st));  // output staging, or the off-chip work fields
     df = dfields.as<float>();
   }
   EIK_CU(diters.alloc(ctx, (size_t)problems * 4, st));
+  if (rows) {
+    EIK_CU(dslow.alloc(ctx, plan.slow_bytes, st));
+    EIK_CU(dwork.alloc(ctx, plan.work_bytes, st));
+  } else {
+    EIK_CU(dslow.alloc(ctx, vbytes, st));
+    EIK_CU(launch_eik_slowness(v, (long long)nsample * N, dslow.as<float>(), st));
+  }
   struct Timer {  // the solver's device time (profiling), released on every path
     cudaEvent_t a = nullptr, b = nullptr;
     ~Timer() {
@@ -354,9 +874,12 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   if (ctx->prof && cudaEventCreate(&tm.a) == cudaSuccess && cudaEventCreate(&tm.b) == cudaSuccess)
     cudaEventRecord(tm.a, st);
   const cudaEvent_t e0 = tm.b ? tm.a : nullptr, e1 = tm.b;
-  EIK_CU(launch_eikonal(dslow.as<float>(), nsample, nz, nx, dz, dx, nsrc, dtab.as<int>(), nrec,
-                        dtab.as<int>() + 2 * nsrc, max_iter, dt, df, diters.as<int>(), resident,
-                        st));
+  const EikArgs E = eik_args(nz, nx, dz, dx, nsrc, dtab.as<int>(), nrec, dtab.as<int>() + 2 * nsrc,
+                             max_iter, dt, df, diters.as<int>());
+  if (rows)
+    EIK_CU(launch_eik_rows(plan, v, nsample, E, dslow.as<float4>(), dwork.as<float4>(), st));
+  else
+    EIK_CU(launch_eikonal(E, dslow.as<float>(), nsample, resident, st));
   if (e1) cudaEventRecord(e1, st);
   std::vector<int> it((size_t)problems);
   EIK_CU(cudaMemcpyAsync(it.data(), diters.p, (size_t)problems * 4, cudaMemcpyDeviceToHost, st));
