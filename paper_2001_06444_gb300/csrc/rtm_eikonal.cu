@@ -197,38 +197,54 @@ __global__ void k_eik_slowness(const float *vel, long long n, float *slow) {
 // ------------------------------------------------- row-owning warps --
 
 // Geometry of k_eik_rows for an nz x nx grid: W warps of lanes that own R rows
-// each, NL lanes in all (NLp: rounded up to 8), NC tiles of 4 columns a row.
+// each, NL lanes in all, NC tiles of 4 columns a row.  Every array is padded so
+// that a lane ahead of or behind its own tiles reads in bounds (and +inf one
+// tile beside the grid), which saves the loop all range checks of its loads.
 struct RowGeo {
-  int R, W, NL, NLp, NC;
+  int R, W, NL, NC;
   int PB;            // bytes of a lane's row of the tile map: PB - 1 is 4 x odd, so that lanes
                      // one tile apart touch different banks in the sweeps of either family
-  int P;             // shared-memory field: floats per row (a multiple of 8: 16-byte accesses
-                     // of lanes R rows and one tile apart touch different banks)
-  long long quads;   // float4 of one skewed copy of the field: (NC + NL - 1) R NLp
-  size_t map_bytes, ring_bytes, field_bytes;  // shared memory: map, warp seams, field
+  int P;             // shared-memory field: floats per row, one tile of +inf on either side (a
+                     // multiple of 8: 16-byte accesses of lanes R rows and one tile apart touch
+                     // different banks)
+  int pad;           // rows of the skewed copies before the first tile
+  int rowq;          // float4 of one row of a skewed copy: R x 32 W
+  int quads;         // ... and of one copy
+  int map_bytes, ring_bytes, field_bytes;  // shared memory: map, warp seams, field
+  int map0, field0;  // offsets of tile (0, 0) within the map (bytes) and the field (floats)
 };
 
 constexpr int kRowGap = 4;    // tiles between the barriers of a CTA of several warps
 constexpr int kRowRing = 16;  // tiles of a seam's ring (> kRowGap + 1 in flight)
-constexpr size_t kRowMap = 64 << 10;  // largest tile map (bytes)
-constexpr int kRowMaxWarps = 12;  // of a CTA: 1536 rows
+constexpr int kRowMap = 64 << 10;  // largest tile map (bytes)
+constexpr int kRowMaxWarps = 12;   // of a CTA: 1536 rows
 constexpr int kRowWarps = 8;  // resident warps an SM needs for shared-memory fields to win
 
-RowGeo row_geo(int nz, int nx) {
-  RowGeo g;
+// False: too large (k_eik_sweep solves it).
+bool row_geo(int nz, int nx, RowGeo &g) {
+  if ((long long)((nz + 3) / 4) * ((nx + 3) / 4) > kRowMap) return false;
   g.W = (nz + 127) / 128;
   g.R = (nz + 32 * g.W - 1) / (32 * g.W);
   g.NL = (nz + g.R - 1) / g.R;
   g.W = (g.NL + 31) / 32;
-  g.NLp = (g.NL + 7) / 8 * 8;
   g.NC = (nx + 3) / 4;
+  if (g.W > kRowMaxWarps) return false;
+  const int lanes = 32 * g.W, slack = lanes + kRowGap * g.W + 4;  // tiles a lane runs past its row
   g.PB = (g.NC + 7) / 8 * 8 + 5;
-  g.P = (4 * g.NC + 7) / 8 * 8;
-  g.quads = (long long)(g.NC + g.NL - 1) * g.R * g.NLp;
-  g.map_bytes = ((size_t)g.NL * g.PB + 15) / 16 * 16;
-  g.ring_bytes = g.W > 1 ? (size_t)(g.W - 1) * kRowRing * 20 : 0;
-  g.field_bytes = (size_t)g.NL * g.R * g.P * 4;
-  return g;
+  g.P = (4 * (g.NC + 2) + 7) / 8 * 8;
+  g.pad = kRowGap * (g.W - 1) + 4;
+  g.rowq = g.R * lanes;
+  const long long quads = (long long)(g.NC + lanes - 1 + 2 * g.pad) * g.rowq;
+  const long long map = (long long)lanes * g.PB + 2 * slack;
+  const long long field = 4ll * ((long long)lanes * g.R * g.P + 8 * slack + 8);
+  if (map > kRowMap || quads > (1 << 28) || field > (1ll << 30)) return false;
+  g.quads = (int)quads;
+  g.map0 = slack;
+  g.map_bytes = (int)((map + 15) / 16 * 16);
+  g.ring_bytes = ((g.W - 1) * kRowRing * 20 + 15) / 16 * 16;
+  g.field0 = 4 * slack + 4;
+  g.field_bytes = (int)((field + 15) / 16 * 16);
+  return true;
 }
 
 struct RowArgs {
@@ -240,20 +256,18 @@ struct RowArgs {
 };
 
 // The two skewed layouts of a grid's tiles: tile (lane g, column c), row r of
-// the lane at ((c + g) R + r) NLp + g (family A) or ((c + NL-1-g) R + r) NLp + g
-// (family B).  The sweeps (+z, +x) and (-z, -x) hold lanes at one c + g, the
-// other two at one c - g, so each reads whole lines of its family's copy:
-// 4 wavefronts a load instruction instead of 32 from the row-major field.  A
-// changed tile is written to both copies.
+// the lane at (pad + c + g) rowq + 32 W r + g (family A) or (pad + c + NL-1-g)
+// rowq + 32 W r + g (family B).  The sweeps (+z, +x) and (-z, -x) hold lanes at
+// one c + g, the other two at one c - g, so each reads whole lines of its
+// family's copy: 4 wavefronts a load instruction instead of 32 from the
+// row-major field.  A changed tile is written to both copies.
 __global__ void k_eik_skew(const float *vel, int nz, int nx, RowGeo g, float4 *slow_a,
                            float4 *slow_b) {
   const float *v = vel + (long long)blockIdx.y * nz * nx;
-  float4 *oa = slow_a + blockIdx.y * g.quads, *ob = slow_b + blockIdx.y * g.quads;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < g.quads;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int lane = (int)(q % g.NLp);
-    const long long lr = q / g.NLp;
-    const int r = (int)(lr % g.R), l = (int)(lr / g.R);
+  float4 *oa = slow_a + (long long)blockIdx.y * g.quads, *ob = slow_b + (long long)blockIdx.y * g.quads;
+  const int lanes = 32 * g.W;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.quads; q += gridDim.x * blockDim.x) {
+    const int lane = q % lanes, lr = q / lanes, r = lr % g.R, l = lr / g.R - g.pad;
     const int row = lane * g.R + r;
 #pragma unroll
     for (int fam = 0; fam < 2; ++fam) {
@@ -271,7 +285,7 @@ __global__ void k_eik_skew(const float *vel, int nz, int nx, RowGeo g, float4 *s
 
 __device__ __forceinline__ float &el(float4 &v, int e) { return reinterpret_cast<float *>(&v)[e]; }
 
-// A problem as its CTA sees it.
+// A problem as its CTA sees it; positions count from tile (0, 0).
 struct RowProblem {
   const float4 *sa, *sb;  // slowness
   float4 *ta, *tb;        // off-chip copies of T
@@ -311,94 +325,82 @@ struct RowLeft {
 };
 
 // One sweep.  FZ / FX: towards +z / +x.  Order and columns below count in the
-// sweep's direction.  A problem of one warp starts at the first tile left to
-// evaluate and stops behind the last.
-template <int R, bool RES, bool ISO, bool FZ, bool FX>
+// sweep's direction.  A problem of one warp (W1) starts at the first tile left
+// to evaluate and stops behind the last.
+template <int R, bool RES, bool ISO, bool W1, bool FZ, bool FX>
 __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, const EikArgs &A,
                                           RowLeft &B) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = W1 ? 0 : threadIdx.x >> 5, gl = threadIdx.x;
   const bool own = gl < g.NL;
-  const int NC = g.NC, W = g.W;
+  const int NC = own ? g.NC : 0, W = W1 ? 1 : g.W, lanes = 32 * W;
   const int lastlane = min(31, g.NL - 1 - 32 * warp);
   const int seam_in = FZ ? warp - 1 : warp;        // seam to the warp of the rows before
   const int seam_out = FZ ? warp : warp - 1;       // ... and after
-  const bool has_in = W > 1 && (FZ ? warp > 0 : warp < W - 1);
-  const bool has_out = W > 1 && (FZ ? warp < W - 1 : warp > 0);
+  const bool has_in = !W1 && (FZ ? warp > 0 : warp < W - 1);
+  const bool has_out = !W1 && (FZ ? warp < W - 1 : warp > 0);
   const bool first = lane == (FZ ? 0 : lastlane), last = lane == (FZ ? lastlane : 0);
   const int ko = FZ ? gl : g.NL - 1 - gl;
   const int start = ko + kRowGap * (FZ ? warp : W - 1 - warp);
-  const int pl = FZ ? max(lane - 1, 0) : min(lane + 1, 31);   // lanes before and after
-  const int sl_ = FZ ? min(lane + 1, 31) : max(lane - 1, 0);
+  const int lb = FZ ? max(lane - 1, 0) : min(lane + 1, 31);   // lanes before and after
+  const int la = FZ ? min(lane + 1, 31) : max(lane - 1, 0);
   constexpr int r0 = FZ ? 0 : R - 1, r1 = FZ ? R - 1 : 0;     // first and last row of a tile
   constexpr bool FA = FZ == FX;                               // family of this sweep
-  const int steps = NC + g.NL - 1 + kRowGap * (W - 1) + 1;
+  constexpr int dir = FX ? 1 : -1;
+  const int steps = g.NC + g.NL - 1 + kRowGap * (W - 1) + 1;
   // the first step with a tile to evaluate, and the last one known now
   int l0 = 0, l1 = steps;
-  if (W == 1) {
+  if (W1) {
     const bool some = B.hi >= B.lo;
     l0 = __reduce_min_sync(0xffffffffu, some ? start + (FX ? B.lo : NC - 1 - B.hi) : steps);
     l1 = __reduce_max_sync(0xffffffffu, some ? start + (FX ? B.hi : NC - 1 - B.lo) : 0);
   }
-  B.lo = NC;
+  B.lo = g.NC;
   B.hi = -1;
-  const float4 *S = FA ? Q.sa : Q.sb;
-  float4 *T = FA ? Q.ta : Q.tb;
-  const int sk = FA ? gl : g.NL - 1 - gl;
-  const int rowq = R * g.NLp;
+  // this lane's positions at column c0 = l0 - start, advanced tile by tile
+  int c = l0 - start;
+  const int cp0 = FX ? c : g.NC - 1 - c;
+  const int q0 = (cp0 + (FA ? gl : g.NL - 1 - gl)) * g.rowq + gl;
+  const int dq = dir * g.rowq;
+  const float4 *S = (FA ? Q.sa : Q.sb) + q0;
+  const float4 *T = RES ? nullptr : (FA ? Q.ta : Q.tb) + q0;
+  float4 *To = RES ? nullptr : (FA ? Q.tb : Q.ta) + (cp0 + (FA ? g.NL - 1 - gl : gl)) * g.rowq + gl;
+  float *F = RES ? Q.st + gl * R * g.P + 4 * cp0 : nullptr;
+  unsigned char *M = Q.map + gl * g.PB + cp0;
+  // (the seam's rows after: the lane after the last one, same column)
+  const int g2 = FZ ? gl + 1 : gl - 1;
+  const int qb = (cp0 + (FA ? g2 : g.NL - 1 - g2)) * g.rowq + r0 * lanes + g2;
+  const float4 *Tb = RES ? nullptr : (FA ? Q.ta : Q.tb) + qb;
+  const float *Fb = RES ? Q.st + (g2 * R + r0) * g.P + 4 * cp0 : nullptr;
+  auto load_t = [&](int ahead, float4 (&t)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      t[r] = RES ? *reinterpret_cast<const float4 *>(F + r * g.P + 4 * dir * ahead)
+                 : T[ahead * dq + r * lanes];
+  };
+  auto load_s = [&](int ahead, float4 (&t)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) t[r] = __ldg(S + ahead * dq + r * lanes);
+  };
   const float4 inf4 = make_float4(kInf, kInf, kInf, kInf);
+  auto load_b = [&](int ahead) {
+    if (W1 || !has_out || !last) return inf4;
+    return RES ? *reinterpret_cast<const float4 *>(Fb + 4 * dir * ahead) : Tb[ahead * dq];
+  };
 
-  auto cp_of = [&](int c) { return FX ? c : NC - 1 - c; };
-  auto idx = [&](int c) { return (long long)(cp_of(c) + sk) * rowq + gl; };
-  auto load_t = [&](int c, float4 (&t)[R]) {
-    if (own && c >= 0 && c < NC) {
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        t[r] = RES ? *reinterpret_cast<const float4 *>(Q.st + (size_t)(gl * R + r) * g.P + 4 * cp_of(c))
-                   : T[idx(c) + r * g.NLp];
-    } else {
-#pragma unroll
-      for (int r = 0; r < R; ++r) t[r] = inf4;
-    }
-  };
-  auto load_s = [&](int c, float4 (&t)[R]) {
-    if (own && c >= 0 && c < NC) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) t[r] = __ldg(S + idx(c) + r * g.NLp);
-    }
-  };
-  // first row of the lane after the seam at column c (from the previous sweep)
-  auto load_b = [&](int c) {
-    float4 t = inf4;
-    if (last && has_out && c >= 0 && c < NC) {
-      const int g2 = FZ ? gl + 1 : gl - 1;
-      if (RES)
-        t = *reinterpret_cast<const float4 *>(Q.st + (size_t)(g2 * R + r0) * g.P + 4 * cp_of(c));
-      else
-        t = T[((long long)(cp_of(c) + (FA ? g2 : g.NL - 1 - g2)) * R + r0) * g.NLp + g2];
-    }
-    return t;
-  };
-  unsigned char *map = Q.map + (size_t)(own ? gl : 0) * g.PB;
-
-  float4 cur[R], nxt[R], pft[R], sc[R], sn[R], bnx = inf4;
-  float carry[R];      // the row's neighbour behind (updated in this sweep)
-  float4 prev;         // last row of the tile before
-#pragma unroll
-  for (int r = 0; r < R; ++r) sc[r] = sn[r] = inf4;
-  load_t(l0 - 1 - start, cur);
-  load_t(l0 - start, nxt);
-  load_t(l0 + 1 - start, pft);
-  load_s(l0 - start, sn);
-  prev = cur[r1];
-  if (W > 1) bnx = load_b(l0 - start);
-  unsigned mnext = 0;
-  if (own && l0 - start >= 0 && l0 - start < NC) mnext = map[cp_of(l0 - start)];
-  bool nd = false, pend = false, any_ch = false, any_map = false;
+  float4 cur[R], nxt[R], pft[R], sc[R], sn[R], bnx, prev;
+  load_t(-1, cur);
+  load_t(0, nxt);
+  load_t(1, pft);
+  load_s(0, sn);
+  bnx = load_b(0);
+  prev = cur[r1];  // last row of the tile before
+  unsigned mnext = M[0];
+  bool ch = false, nd = false, any_ch = false, any_map = false;
   unsigned chb = 0;  // lanes that changed in the step before
 #pragma unroll 1
   for (int l = l0; l < steps; ++l) {
-    const int c = l - start;
-    const bool in = own && c >= 0 && c < NC;
+    const bool in = (unsigned)c < (unsigned)NC;
+    float carry[R];  // each row's neighbour behind (updated in this sweep)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       carry[r] = FX ? cur[r].w : cur[r].x;
@@ -406,32 +408,32 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
       nxt[r] = pft[r];
       sc[r] = sn[r];
     }
+    load_t(2, pft);
+    load_s(1, sn);
     const float4 bcur = bnx;
-    load_t(c + 2, pft);
-    load_s(c + 1, sn);
-    if (W > 1) bnx = load_b(c + 1);
+    if (!W1) bnx = load_b(1);
     bool act = in && (mnext || nd);
-    mnext = 0;
-    if (own && c + 1 >= 0 && c + 1 < NC) mnext = map[cp_of(c + 1)];
+    mnext = M[dir];
     float4 seam = inf4;
-    if (W > 1 && has_in && first && in) {
+    if (!W1 && has_in && first && in) {
       const int k = seam_in * kRowRing + (c & (kRowRing - 1));
       seam = Q.ring[k];
       act = act || Q.ringf[k];
     }
-    bool ch = false;
+    const bool pend = ch;
+    ch = false;
     if (__any_sync(0xffffffffu, act)) {
       // the tile's neighbours across lanes: the rows before at this column,
       // updated (that lane was here one step ago), and the rows after, old
       float4 bef, aft;
-      bef.x = __shfl_sync(0xffffffffu, prev.x, pl);
-      bef.y = __shfl_sync(0xffffffffu, prev.y, pl);
-      bef.z = __shfl_sync(0xffffffffu, prev.z, pl);
-      bef.w = __shfl_sync(0xffffffffu, prev.w, pl);
-      aft.x = __shfl_sync(0xffffffffu, nxt[r0].x, sl_);
-      aft.y = __shfl_sync(0xffffffffu, nxt[r0].y, sl_);
-      aft.z = __shfl_sync(0xffffffffu, nxt[r0].z, sl_);
-      aft.w = __shfl_sync(0xffffffffu, nxt[r0].w, sl_);
+      bef.x = __shfl_sync(0xffffffffu, prev.x, lb);
+      bef.y = __shfl_sync(0xffffffffu, prev.y, lb);
+      bef.z = __shfl_sync(0xffffffffu, prev.z, lb);
+      bef.w = __shfl_sync(0xffffffffu, prev.w, lb);
+      aft.x = __shfl_sync(0xffffffffu, nxt[r0].x, la);
+      aft.y = __shfl_sync(0xffffffffu, nxt[r0].y, la);
+      aft.z = __shfl_sync(0xffffffffu, nxt[r0].z, la);
+      aft.w = __shfl_sync(0xffffffffu, nxt[r0].w, la);
       if (first) bef = seam;
       if (last) aft = bcur;
       if (act) {
@@ -451,24 +453,20 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
           }
         }
         if (ch) {
-          if (RES) {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-              *reinterpret_cast<float4 *>(Q.st + (size_t)(gl * R + r) * g.P + 4 * cp_of(c)) = cur[r];
-          } else {
-            const long long ia = (long long)(cp_of(c) + gl) * rowq + gl;
-            const long long ib = (long long)(cp_of(c) + g.NL - 1 - gl) * rowq + gl;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-              Q.ta[ia + r * g.NLp] = cur[r];
-              Q.tb[ib + r * g.NLp] = cur[r];
+          for (int r = 0; r < R; ++r) {
+            if (RES) {
+              *reinterpret_cast<float4 *>(F + r * g.P) = cur[r];
+            } else {
+              const_cast<float4 *>(T)[r * lanes] = cur[r];
+              To[r * lanes] = cur[r];
             }
           }
         }
       }
     }
     prev = cur[r1];
-    if (W > 1 && has_out && last && in) {  // hand the last row over the seam
+    if (!W1 && has_out && last && in) {  // hand the last row over the seam
       const int k = seam_out * kRowRing + (c & (kRowRing - 1));
       Q.ring[k] = cur[r1];
       Q.ringf[k] = ch;
@@ -477,32 +475,42 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
     // next column (evaluated in this sweep), this lane's next column
     // likewise; the column behind is final for this sweep
     const unsigned chm = __ballot_sync(0xffffffffu, ch);
-    const bool ch_b = !first && ((chm >> pl) & 1u), ch_a = !last && ((chm >> sl_) & 1u);
+    const bool ch_b = !first && ((chm >> lb) & 1u), ch_a = !last && ((chm >> la) & 1u);
     nd = ch || ch_b;
-    const bool left = pend || ch || ch_a;
-    if (own && c >= 1 && c <= NC) {
-      const int cp = cp_of(c - 1);
-      map[cp] = left;
+    if ((unsigned)(c - 1) < (unsigned)NC) {
+      const bool left = pend || ch || ch_a;
+      M[-dir] = left;
       any_map |= left;
-      if (left) {
+      if (W1 && left) {
+        const int cp = FX ? c - 1 : NC - c;
         B.lo = min(B.lo, cp);
         B.hi = max(B.hi, cp);
       }
     }
-    if (W > 1 && has_in && first && ch) {  // the rows before passed this column already
-      Q.map[(size_t)(FZ ? gl - 1 : gl + 1) * g.PB + cp_of(c)] = 1;
+    if (!W1 && has_in && first && ch) {  // the rows before passed this column already
+      Q.map[(FZ ? gl - 1 : gl + 1) * g.PB + (FX ? c : NC - 1 - c)] = 1;
       any_map = true;
     }
-    pend = ch;
     any_ch |= ch;
-    if (W > 1) {
+    if (!W1) {
       if ((l & (kRowGap - 1)) == kRowGap - 1) __syncthreads();
     } else if (l > l1 && !(chm | chb)) {
       break;
     }
     chb = chm;
+    ++c;
+    S += dq;
+    M += dir;
+    if (RES) {
+      F += 4 * dir;
+      Fb += 4 * dir;
+    } else {
+      T += dq;
+      To += dq;
+      Tb += dq;
+    }
   }
-  if (W > 1) {
+  if (!W1) {
     B.changed |= __syncthreads_or(any_ch) != 0;
     B.map = __syncthreads_or(any_map) != 0;
   } else {
@@ -512,67 +520,63 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
   }
 }
 
-template <int R, bool RES, bool ISO>
-__global__ void __launch_bounds__(32 * kRowMaxWarps) k_eik_rows(const __grid_constant__ RowArgs A) {
+template <int R, bool RES, bool ISO, bool W1>
+__global__ void __launch_bounds__(W1 ? 32 : 32 * kRowMaxWarps) k_eik_rows(const __grid_constant__ RowArgs A) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   const RowGeo &g = A.g;
   const EikArgs &E = A.e;
   const int p = A.p0 + blockIdx.x, sample = p / E.nsrc, src = p % E.nsrc;
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = threadIdx.x, nth = blockDim.x, lanes = 32 * g.W;
+  const float4 inf4 = make_float4(kInf, kInf, kInf, kInf);
   RowProblem Q;
-  Q.map = s_raw;
+  Q.map = s_raw + g.map0;
   Q.ring = reinterpret_cast<float4 *>(s_raw + g.map_bytes);
   Q.ringf = reinterpret_cast<int *>(Q.ring + (g.W - 1) * kRowRing);
-  Q.st = reinterpret_cast<float *>(s_raw + g.map_bytes + (g.ring_bytes + 15) / 16 * 16);
-  Q.sa = A.slow_a + (sample - A.s0) * g.quads;
-  Q.sb = A.slow_b + (sample - A.s0) * g.quads;
-  Q.ta = RES ? nullptr : A.work + (long long)blockIdx.x * 2 * g.quads;
+  float *field = reinterpret_cast<float *>(s_raw + g.map_bytes + g.ring_bytes);
+  Q.st = field + g.field0;
+  const long long s0 = (long long)(sample - A.s0) * g.quads + g.pad * g.rowq;
+  Q.sa = A.slow_a + s0;
+  Q.sb = A.slow_b + s0;
+  float4 *work = RES ? nullptr : A.work + (long long)blockIdx.x * 2 * g.quads;
+  Q.ta = RES ? nullptr : work + g.pad * g.rowq;
   Q.tb = RES ? nullptr : Q.ta + g.quads;
-  const float4 inf4 = make_float4(kInf, kInf, kInf, kInf);
-  for (int k = tid; k < (int)(g.map_bytes / 4); k += nth) reinterpret_cast<unsigned *>(Q.map)[k] = 0;
+  for (int k = tid; k < g.map_bytes / 4; k += nth) reinterpret_cast<unsigned *>(s_raw)[k] = 0;
   if (RES) {
-    float4 *t = reinterpret_cast<float4 *>(Q.st);
-    for (int k = tid; k < (int)(g.field_bytes / 16); k += nth) t[k] = inf4;
+    for (int k = tid; k < g.field_bytes / 16; k += nth) reinterpret_cast<float4 *>(field)[k] = inf4;
   } else {
-    for (long long k = tid; k < 2 * g.quads; k += nth) Q.ta[k] = inf4;
+    for (int k = tid; k < 2 * g.quads; k += nth) work[k] = inf4;
   }
   __syncthreads();
   const int iz = E.src[2 * src], ix = E.src[2 * src + 1];
   const int gs = iz / R, rs = iz - gs * R, cs = ix >> 2;
-  auto qa = [&](int lane, int r, int c) { return ((long long)(c + lane) * R + r) * g.NLp + lane; };
-  auto qb = [&](int lane, int r, int c) {
-    return ((long long)(c + g.NL - 1 - lane) * R + r) * g.NLp + lane;
-  };
   if (tid == 0) {
     if (RES) {
-      Q.st[(size_t)iz * g.P + ix] = 0.0f;
+      Q.st[iz * g.P + ix] = 0.0f;
     } else {
-      reinterpret_cast<float *>(Q.ta + qa(gs, rs, cs))[ix & 3] = 0.0f;
-      reinterpret_cast<float *>(Q.tb + qb(gs, rs, cs))[ix & 3] = 0.0f;
+      reinterpret_cast<float *>(Q.ta + (cs + gs) * g.rowq + rs * lanes + gs)[ix & 3] = 0.0f;
+      reinterpret_cast<float *>(Q.tb + (cs + g.NL - 1 - gs) * g.rowq + rs * lanes + gs)[ix & 3] = 0.0f;
     }
-    Q.map[(size_t)gs * g.PB + cs] = 1;
-    if (gs > 0) Q.map[(size_t)(gs - 1) * g.PB + cs] = 1;
-    if (gs + 1 < g.NL) Q.map[(size_t)(gs + 1) * g.PB + cs] = 1;
-    if (cs > 0) Q.map[(size_t)gs * g.PB + cs - 1] = 1;
-    if (cs + 1 < g.NC) Q.map[(size_t)gs * g.PB + cs + 1] = 1;
+    Q.map[gs * g.PB + cs] = 1;
+    if (gs > 0) Q.map[(gs - 1) * g.PB + cs] = 1;
+    if (gs + 1 < g.NL) Q.map[(gs + 1) * g.PB + cs] = 1;
+    if (cs > 0) Q.map[gs * g.PB + cs - 1] = 1;
+    if (cs + 1 < g.NC) Q.map[gs * g.PB + cs + 1] = 1;
   }
   __syncthreads();
   // the four diagonal directions: (+z, +x), (+z, -x), (-z, -x), (-z, +x); an
   // iteration that changes nothing ends the solve, and an empty map means
   // that the rest of this iteration and the next one change nothing
   RowLeft B;
-  if (tid < g.NL) {
-    B.lo = tid == gs ? max(cs - 1, 0) : cs;
-    B.hi = tid == gs ? min(cs + 1, g.NC - 1) : (abs(tid - gs) == 1 ? cs : -1);
-  }
+  B.lo = tid == gs ? max(cs - 1, 0) : cs;
+  B.hi = tid == gs ? min(cs + 1, g.NC - 1) : (abs(tid - gs) == 1 && tid < g.NL ? cs : -1);
   int it = 0;
   bool converged = false;
   for (; it < E.max_iter; ++it) {
     B.changed = false;
-    if (B.map) row_sweep<R, RES, ISO, true, true>(Q, g, E, B);
-    if (B.map) row_sweep<R, RES, ISO, true, false>(Q, g, E, B);
-    if (B.map) row_sweep<R, RES, ISO, false, false>(Q, g, E, B);
-    if (B.map) row_sweep<R, RES, ISO, false, true>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, W1, true, true>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, W1, true, false>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, W1, false, false>(Q, g, E, B);
+    if (B.map) row_sweep<R, RES, ISO, W1, false, true>(Q, g, E, B);
     if (!B.changed) {
       converged = true;
       break;
@@ -581,9 +585,10 @@ __global__ void __launch_bounds__(32 * kRowMaxWarps) k_eik_rows(const __grid_con
   if (tid == 0) E.iters[p] = converged ? it + 1 : -1;
   __syncthreads();
   auto value = [&](int i, int j) {
-    if (RES) return Q.st[(size_t)i * g.P + j];
+    if (RES) return Q.st[i * g.P + j];
     const int lane = i / R;
-    return reinterpret_cast<const float *>(Q.ta + qa(lane, i - lane * R, j >> 2))[j & 3];
+    return reinterpret_cast<const float *>(Q.ta + ((j >> 2) + lane) * g.rowq + (i - lane * R) * lanes +
+                                           lane)[j & 3];
   };
   if (E.times) {
     float *out = E.times + (long long)p * E.nrec;
@@ -637,7 +642,7 @@ static EikArgs eik_args(int nz, int nx, double dz, double dx, int nsrc, const in
 struct RowPlan {
   RowGeo g;
   bool resident = false;
-  size_t smem = 0;
+  int smem = 0;
   int group = 1;         // samples whose skewed slowness is held at once
   long long chunk = 1;   // problems of one launch
   size_t slow_bytes = 0, work_bytes = 0;
@@ -646,19 +651,15 @@ struct RowPlan {
 // Off-chip fields and slowness stay within about this much scratch.
 constexpr size_t kRowScratch = size_t(2) << 30;
 
-// False: the grid's tile map is too large (k_eik_sweep solves it).
 static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
-                     size_t smem_cta, size_t smem_sm) {
-  if ((long long)((nz + 3) / 4) * ((nx + 3) / 4) > (long long)kRowMap) return false;
-  p.g = row_geo(nz, nx);
+                     int smem_cta, int smem_sm) {
+  if (!row_geo(nz, nx, p.g)) return false;
   const RowGeo &g = p.g;
-  if (g.W > kRowMaxWarps || g.map_bytes > kRowMap) return false;
-  const size_t base = g.map_bytes + (g.ring_bytes + 15) / 16 * 16;
+  const int base = g.map_bytes + g.ring_bytes;
   const long long problems = (long long)nsample * nsrc;
   p.resident = false;
   if (!(flags & RTM_EIK_OFFCHIP) && base + g.field_bytes <= smem_cta) {
-    const long long per_sm =
-        std::min<long long>(32 / g.W, (long long)(smem_sm / (base + g.field_bytes + 1024)));
+    const long long per_sm = std::min(32 / g.W, smem_sm / (base + g.field_bytes + 1024));
     p.resident = (flags & RTM_EIK_SHARED) || problems <= per_sm * sms || per_sm * g.W >= kRowWarps;
   }
   p.smem = base + (p.resident ? g.field_bytes : 0);
@@ -679,11 +680,11 @@ static cudaError_t launch_eik_rows(const RowPlan &P, const float *vel, int nsamp
   A.e = E;
   A.g = P.g;
   A.slow_a = slow;
-  A.slow_b = slow + (long long)P.group * P.g.quads;
+  A.slow_b = slow + (size_t)P.group * P.g.quads;
   A.work = work;
   auto run = [&](auto kernel, unsigned n) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)P.smem);
+                                         P.smem);
     if (e != cudaSuccess) return e;
     kernel<<<n, 32 * P.g.W, P.smem, st>>>(A);
     return cudaGetLastError();
@@ -691,12 +692,18 @@ static cudaError_t launch_eik_rows(const RowPlan &P, const float *vel, int nsamp
   const bool iso = E.dz == E.dx;
   auto go = [&](auto rows, unsigned n) -> cudaError_t {
     constexpr int R = decltype(rows)::value;
-    if (P.resident) return iso ? run(k_eik_rows<R, true, true>, n) : run(k_eik_rows<R, true, false>, n);
-    return iso ? run(k_eik_rows<R, false, true>, n) : run(k_eik_rows<R, false, false>, n);
+    auto one = [&](auto res, auto same) -> cudaError_t {
+      constexpr bool RES = decltype(res)::value, ISO = decltype(same)::value;
+      return P.g.W == 1 ? run(k_eik_rows<R, RES, ISO, true>, n) : run(k_eik_rows<R, RES, ISO, false>, n);
+    };
+    const std::true_type yes;
+    const std::false_type no;
+    if (P.resident) return iso ? one(yes, yes) : one(yes, no);
+    return iso ? one(no, yes) : one(no, no);
   };
   for (int s0 = 0; s0 < nsample; s0 += P.group) {
     const int ns = std::min(P.group, nsample - s0);
-    const unsigned bx = (unsigned)std::min<long long>((P.g.quads + 255) / 256, 1024);
+    const unsigned bx = (unsigned)std::min((P.g.quads + 255) / 256, 1024);
     for (int y0 = 0; y0 < ns; y0 += 65535) {
       const long long at = (long long)y0 * P.g.quads;
       k_eik_skew<<<dim3(bx, std::min(65535, ns - y0)), 256, 0, st>>>(
@@ -841,7 +848,7 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
   RowPlan plan;
   const bool rows = !getenv("RTM_EIK_TILE") && row_plan(plan, nz, nx, nsample, nsrc, flags, sms,
-                                                        (size_t)smem_cta, (size_t)smem_sm);
+                                                        smem_cta, smem_sm);
   const bool fits = (size_t)N * 4 <= eik_resident_limit();
   const bool resident = fits && !(flags & RTM_EIK_OFFCHIP) &&
                         ((flags & RTM_EIK_SHARED) || problems <= (long long)sms);
