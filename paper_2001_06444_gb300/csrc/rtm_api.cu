@@ -450,7 +450,68 @@ struct Common {
   long long n_rent = 0, n_rext = 0, n_rcen = 0;  // receiver-table entries (debug index checks)
   DevBuf c_all, gx, gz, src_rc, rptr, rent, rext_ptr, rext_ent, rcen_ptr, rcen_ent, wav, items, err;
   CUtensorMap mc;
+  ResPlan res;       // phases with the grid on chip (C = 0: not)
+  DevBuf res_ent;    // ... and their receivers, sorted by row and strip
+  int res_max_ent = 0;
 };
+
+// How B items' phases run with the grid on chip (k_resident), or C = 0 if the
+// tile kernels are the faster form or the grid does not fit.
+// Measured on a GB300 (600-step phases, FP32 and FP16 snapshots every 4 steps):
+//   a resident step takes 0.55 us + 0.1 us per strip of 4 points that a
+//   scheduler's threads own (rows x threads / 128), + 0.3 us backward with more
+//   than 4 rows a thread: 201 x 101 in 16 blocks 1.0-1.1 us, in 4 blocks 2.3-2.9
+//   us, 401 x 111 in 16 blocks 1.7 us; clusters beyond those that run at once
+//   take further rounds;
+//   a tile-kernel step takes 3.4 us, from 60 tiles (120 x 24) on about 3.0 us +
+//   6 ns a tile: 32 items of 201 x 101 6.5-7.8 us, 24 of 401 x 111 7.5-8.1 us.
+// Both sides at the line: 64 items of 201 x 101 4.8 us against 9.5, 24 of 401 x
+// 111 6.8 against 7.5 (forward), 8 of 851 x 176 do not fit.
+// RTM_RESIDENT=C or C,R forces a cluster size (and rows a thread), 0 none.
+static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, int *max_ent) {
+  const char *env = std::getenv("RTM_RESIDENT");
+  int fc = 0, fr = 0;
+  if (env) std::sscanf(env, "%d,%d", &fc, &fr);
+  if (env && fc <= 0) return ResPlan{};
+  const double tiles = (double)B * g.ntx2 * ((g.NZ + 23) / 24);
+  double best_t = fc > 0 ? 1e300 : std::max(3.4, 3.0 + 0.006 * tiles);
+  ResPlan best, p;
+  for (int C : {16, 8, 4, 2, 1}) {
+    if (fc > 0 && C != fc) continue;
+    if (!resident_shape(g, C, fr, p)) continue;
+    const int ents = resident_max_ent(p, ent);
+    if (!resident_fits(p, ents)) continue;
+    const int n = resident_clusters(p, ents);
+    if (n < 1) continue;
+    const double t = ((B + n - 1) / n) *
+                     (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0));
+    if (t < best_t) {
+      best_t = t;
+      best = p;
+      *max_ent = ents;
+    }
+  }
+  return best;
+}
+
+// Chooses the resident form for B items in flight and uploads its receiver table.
+static int setup_resident(rtm_ctx *ctx, Common &C, const rtm_acq &acq, int B, cudaStream_t st) {
+  const Geo &g = C.g;
+  const int NS = (g.X0 + g.NX + 3) / 4;
+  std::vector<int2> ent(acq.nrec);
+  for (int r = 0; r < acq.nrec; ++r) {
+    const int row = acq.rec_iz[r] + g.nb, col = acq.rec_ix[r] + g.CP;
+    ent[r] = make_int2(row * NS + col / 4, 4 * r + col % 4);
+  }
+  std::stable_sort(ent.begin(), ent.end(), [](const int2 &a, const int2 &b) { return a.x < b.x; });
+  C.res = resident_plan(g, B, ent, &C.res_max_ent);
+  if (!C.res.C) return RTM_OK;
+  if (ent.empty()) ent.push_back(make_int2(0x7fffffff, 0));
+  CU(C.res_ent.alloc(ctx, ent.size() * sizeof(int2), st));
+  // (a pageable copy is staged before the call returns)
+  CU(cudaMemcpyAsync(C.res_ent.p, ent.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+  return RTM_OK;
+}
 
 // Receiver lists of the two-step tiles: every tile whose extended region
 // (tile plus a 4-point ring) holds the receiver, and the one tile whose centre
@@ -647,6 +708,38 @@ static void fill_args2(Step2Args &A2, const StepArgs &A, const Common &C) {
   A2.len.rent = C.n_rext;
 }
 
+static void fill_args_res(ResArgs &R, const StepArgs &A, const Common &C) {
+  std::memset(&R, 0, sizeof(R));
+  R.g = A.g;
+  R.k = A.k;
+  R.gx = A.gx;
+  R.gz = A.gz;
+  R.c_all = A.c_all;
+  R.item_sample = A.item_sample;
+  R.item_shot = A.item_shot;
+  R.src_row = A.src_row;
+  R.src_col = A.src_col;
+  R.wav = A.wav;
+  R.src_scale = A.src_scale;
+  R.ent = C.res_ent.as<int2>();
+  R.nent = A.nrec;
+  R.max_ent = C.res_max_ent;
+  R.nrec = A.nrec;
+  R.nt = A.nt;
+  R.seis = A.seis;
+  R.rec_out = A.rec_out;
+  R.snap = A.snap;
+  R.snap_dtype = A.snap_dtype;
+  R.nsnap = A.nsnap;
+  R.smax = A.smax;
+  R.num = A.num;
+  R.den = A.den;
+  R.dmax = A.dmax;
+  R.refl = A.refl;
+  R.err = A.err;
+  R.len = A.len;
+}
+
 // Test hook: if injections are pending, take one and raise this call's flag.
 static int maybe_inject_timeout(rtm_ctx *ctx, const Common &C, cudaStream_t st) {
   int n = ctx->inject_timeouts.load();
@@ -745,13 +838,15 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
                       cfg.l2_ahead, cfg.pdl);
   }
   if (!rc) rc = maybe_inject_timeout(ctx, C, st);
-  if (rc) return rc;
-  trace_mark("tables and model set up");
-  const Geo &g = C.g;
-  const int nsnap = gr.nt / op.isnap;
   const long long nitems = (long long)nsample * acq.nshot;
   if (B > nitems) B = (int)nitems;
   if (B < 1) B = 1;
+  if (!rc && cfg.resident) rc = setup_resident(ctx, C, acq, B, st);
+  if (rc) return rc;
+  trace_mark("tables and model set up");
+  const Geo &g = C.g;
+  const bool res = C.res.C > 0;
+  const int nsnap = gr.nt / op.isnap;
   // items in (sample, shot) order
   std::vector<int> items(2 * nitems);
   for (long long q = 0; q < nitems; ++q) {
@@ -867,18 +962,47 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   // Forward steps n0 .. n1-1 on Fs.  store: keep S^k, k in K and n0 < k <= n1,
   // in slot k/isnap - 1 - kbase.  save: copy the state into checkpoint n/cpC
   // before every step n that is a multiple of cpC.
+  auto save_state = [&](Fields &Fs, int n) -> int {
+    const size_t bytes = (size_t)nb * g.plane * 4;
+    float *dst = cps.as<float>() + (size_t)(n / cpC) * 2 * B * g.plane;
+    CU(cudaMemcpyAsync(dst, Fs.v[Fs.cv].p, bytes, cudaMemcpyDeviceToDevice, st));
+    CU(cudaMemcpyAsync(dst + (size_t)B * g.plane, Fs.d[Fs.cd].p, bytes, cudaMemcpyDeviceToDevice,
+                       st));
+    return RTM_OK;
+  };
+  // A phase of `count` steps with the grid on chip.  Outside checkpoint mode a
+  // phase starts at rest and nobody reads its end state.
+  auto resident = [&](int mode, Fields &Fs, int k_first, int count, int kbase, bool store) -> int {
+    ResArgs R;
+    fill_args_res(R, A, C);
+    R.v = Fs.v[Fs.cv].as<float>();
+    R.d = Fs.d[Fs.cd].as<float>();
+    R.load_state = R.store_state = cpC != 0;
+    R.k_first = k_first;
+    R.count = count;
+    R.isnap = isnap;
+    R.kbase = kbase;
+    R.store = store;
+    R.dmax_flag = mode == MODE_BWD && k_first >= isnap && k_first - count < isnap;
+    CU(launch_resident(mode, C.res, R, nb, st));
+    ++step_launches;
+    return RTM_OK;
+  };
   auto fwd_range = [&](Fields &Fs, int n0, int n1, int kbase, bool store, bool save) -> int {
     int r2;
+    if (res) {
+      for (int n = n0; n < n1;) {
+        if (save && n % cpC == 0 && (r2 = save_state(Fs, n))) return r2;
+        const int e = save ? std::min(n1, (n / cpC + 1) * cpC) : n1;
+        if ((r2 = resident(MODE_FWD, Fs, n, e - n, kbase, store))) return r2;
+        n = e;
+      }
+      return RTM_OK;
+    }
     auto idx = [&](int k) { return k / isnap - 1 - kbase; };
     bool stored = true;  // the range's input field is not the range's to store
     for (int n = n0; n < n1;) {
-      if (save && n % cpC == 0) {
-        const size_t bytes = (size_t)nb * g.plane * 4;
-        float *dst = cps.as<float>() + (size_t)(n / cpC) * 2 * B * g.plane;
-        CU(cudaMemcpyAsync(dst, Fs.v[Fs.cv].p, bytes, cudaMemcpyDeviceToDevice, st));
-        CU(cudaMemcpyAsync(dst + (size_t)B * g.plane, Fs.d[Fs.cd].p, bytes,
-                           cudaMemcpyDeviceToDevice, st));
-      }
+      if (save && n % cpC == 0 && (r2 = save_state(Fs, n))) return r2;
       if (two && n + 2 <= n1 && (!half || isnap % 2 == 0)) {
         Step2RT r;
         r.t1 = n;
@@ -921,6 +1045,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   // is imaged once, in the same order, so images do not change.
   auto bwd_range = [&](Fields &Ws, int k1, int k0, int kbase) -> int {
     int r2;
+    if (res) return resident(MODE_BWD, Ws, k1, k1 - k0, kbase, false);
     auto idx = [&](int k) { return k / isnap - 1 - kbase; };
     auto single = [&](int k) -> int {  // w^k from w^{k+1}; images w^k
       StepRT r{};
@@ -993,6 +1118,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
         A.len.rec_out = A2.len.rec_out = (nitems - q0) * (long long)nt * acq.nrec;
         if ((rc = mark())) return rc;
         rc = run_phase(ctx, graph, st, [&]() -> int {
+          if (res) return resident(MODE_BORN, F, 0, nt, 0, false);
           auto slot = [&](int k) { return inK(k) ? k / isnap - 1 : -1; };
           for (int n = 0; n < nt;) {
             int r2;
@@ -1119,8 +1245,10 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
   }
   CU(C.items.alloc(ctx, items.size() * 4, st));
   CU(cudaMemcpyAsync(C.items.p, items.data(), items.size() * 4, cudaMemcpyHostToDevice, st));
+  if (ctx->defaults.resident && (rc = setup_resident(ctx, C, acq, B, st))) return rc;
+  const bool res = C.res.C > 0;
   Fields F;
-  if ((rc = alloc_fields(ctx, F, g, B, st, sk))) return rc;
+  if (!res && (rc = alloc_fields(ctx, F, g, B, st, sk))) return rc;
   StepArgs A;
   fill_args(A, C, gr, acq);
   A.len.items = B;
@@ -1128,11 +1256,19 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
   long long launches = 0;
   for (int q0 = 0; q0 < ns; q0 += B) {
     const int nb = std::min(B, ns - q0);
-    if ((rc = zero_fields(ctx, F, g, nb, st))) return rc;
+    if (!res && (rc = zero_fields(ctx, F, g, nb, st))) return rc;
     A.item_sample = C.items.as<int>() + q0;
     A.item_shot = C.items.as<int>() + ns + q0;
     A.rec_out = seis_d + (size_t)q0 * gr.nt * acq.nrec;
     A.len.rec_out = (long long)(ns - q0) * gr.nt * acq.nrec;
+    if (res) {  // the whole modelling in one launch
+      ResArgs R;
+      fill_args_res(R, A, C);
+      R.count = gr.nt;
+      CU(launch_resident(MODE_MODEL, C.res, R, nb, st));
+      ++launches;
+      continue;
+    }
     Step2Args A2;
     fill_args2(A2, A, C);
     for (int n = 0; n < gr.nt;) {
@@ -1293,6 +1429,9 @@ int rtm_ctx_create(rtm_ctx **out, int device, size_t hbm_budget_bytes) {
   const char *sk = std::getenv("RTM_STEP_KERNEL");
   const int k = sk ? std::atoi(sk) : 0;
   ctx->defaults.step_kernel = (k >= 1 && k <= 4) ? k : 2;
+  // (a chosen kernel runs every phase; RTM_RESIDENT=0 keeps phases off chip)
+  const char *rs = std::getenv("RTM_RESIDENT");
+  ctx->defaults.resident = !sk && !(rs && rs[0] == '0');
   const char *tz = std::getenv("RTM_TILE_Z");
   const int z = tz ? std::atoi(tz) : 24;
   ctx->defaults.tile_z = ((z == 16 && k == 3) || (z == 32 && k == 4)) ? z : 24;
@@ -1394,6 +1533,7 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
         c.tile_z = kd[1];
         c.l2_ahead = kd[2];
         c.graph = graph;
+        c.resident = ctx->defaults.resident;
         c.max_items = items >= nitems ? 0 : (int)items;
         bool dup = false;
         for (auto &o : cand)

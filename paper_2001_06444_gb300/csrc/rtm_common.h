@@ -170,6 +170,39 @@ struct Step2RT {
                        // 0 = no prefetch
 };
 
+// Arguments of one phase of B items with the grid on chip (k_resident).
+struct ResArgs {
+  Geo g;
+  Coef k;
+  const float *gx, *gz;
+  const float *c_all;
+  const int *item_sample, *item_shot;
+  float *v, *d;              // [B][plane] state read before and written after the phase
+  int load_state, store_state;  // (0: starts at rest; 0: nobody reads the end state)
+  const int *src_row, *src_col;
+  const float *wav;
+  float src_scale;
+  const int2 *ent;           // receivers {padded row * NS + strip, 4 receiver + column in the strip}
+  int nent, max_ent;         // entries, most of one block
+  int nrec, nt;
+  const float *seis;
+  float *rec_out;
+  void *snap;
+  int snap_dtype, nsnap;
+  unsigned *smax;
+  float *num, *den;
+  unsigned *dmax;
+  const float *refl;
+  int *err;
+  DbgLen len;
+  int k_first, count;        // BWD: k = k_first, k_first - 1, ..; else updates n = k_first, ..
+  int isnap, kbase;          // imaging interval (0: none); slot of S^k is k / isnap - 1 - kbase
+  int store;                 // FWD: keep the snapshots
+  int dmax_flag;             // BWD: the phase images k == isnap: reduce max(den)
+  unsigned C;                // (set by the launcher) blocks of a cluster, rows of a block, strips
+  int H, NS;
+};
+
 enum { MODE_FWD = 0, MODE_MODEL = 1, MODE_BWD = 2, MODE_BORN = 3 };
 
 }  // namespace rtm

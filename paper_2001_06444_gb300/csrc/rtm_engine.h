@@ -31,6 +31,7 @@ struct RunConfig {
   int l2_ahead = 0;     // step_kernel 2: each block prefetches a later block's tile into L2
   int image_input = 0;  // two-step backward launches image their input field where they can
   int pdl = 0;          // step_kernel 4: programmatic dependent launches (griddepcontrol)
+  int resident = 1;     // run phases with the grid on chip where that is faster (resident_plan)
 };
 // Shape key of the autotuner cache.
 struct TuneKey {

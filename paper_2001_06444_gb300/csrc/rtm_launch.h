@@ -3,6 +3,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "rtm_common.h"
 
 namespace rtm {
@@ -36,6 +38,18 @@ cudaError_t launch_step2a(int mode, int tile_z, const CUtensorMap &mv, const CUt
 size_t step2a_smem_bytes(int tile_z);
 // bounded-wait self-test: raises *flag after waiting `ns` for bytes that never arrive
 cudaError_t launch_wait_probe(int *flag, unsigned long long ns, cudaStream_t st);
+// whole phases with the grid on chip, one cluster of blocks per item
+// (rtm_resident.cu): C blocks of H rows; a thread owns R rows x 4 columns
+constexpr int kResRows = 6;
+struct ResPlan {
+  int C = 0, H = 0, R = 0, G = 0, NS = 0, threads = 0;
+};
+// The shape with C blocks (R = 0: the fewest rows a thread that fit); false if it does not fit.
+bool resident_shape(const Geo &g, int C, int R, ResPlan &p);
+int resident_max_ent(const ResPlan &p, const std::vector<int2> &ent);
+bool resident_fits(const ResPlan &p, int max_ent);
+int resident_clusters(const ResPlan &p, int max_ent);
+cudaError_t launch_resident(int mode, const ResPlan &p, ResArgs A, int B, cudaStream_t st);
 int step2_tile_x();
 int step2_tile_z();
 int step2_ext();

@@ -161,36 +161,53 @@ __device__ __forceinline__ void block_max_atomic(float v, unsigned *dst, float *
 // Returns d^{n+1} (before injection); v^{n+1} = v^n + d^{n+1}.  Lanes are
 // processed in pairs (0,1) and (2,3); each lane rounds as the scalar form of
 // the single-step kernel.
-template <bool SPONGE, bool ISO>
-__device__ __forceinline__ float4 update4(const float4 *zc, const float4 &xl, const float4 &xr,
-                                          const float4 &dv, const float4 &cv, const Coef &k,
-                                          float gzr, const float *gxs) {
+template <bool ISO>
+__device__ __forceinline__ void laplacian4(const float4 *zc, const float4 &xl, const float4 &xr,
+                                           const Coef &k, float2 (&lap)[2]) {
   const float4 xc = zc[4];
   const float v[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w, xr.x, xr.y, xr.z, xr.w};
-  float out[4];
 #pragma unroll
   for (int l = 0; l < 4; l += 2) {
     const float2 ce = make_float2(v[4 + l], v[5 + l]);
-    float2 lap = make_float2(0.f, 0.f);
+    float2 a = make_float2(0.f, 0.f);
 #pragma unroll
     for (int m = 4; m >= 1; --m) {
-      const float2 xm = make_float2(v[4 + l - m], v[5 + l - m]);
-      const float2 xp = make_float2(v[4 + l + m], v[5 + l + m]);
+      // columns an odd distance away straddle register pairs: added one by one,
+      // which costs fewer instructions than moving them into pairs
+      const float2 xs =
+          (m & 1) ? make_float2(__fadd_rn(v[4 + l - m], v[4 + l + m]), __fadd_rn(v[5 + l - m], v[5 + l + m]))
+                  : __fadd2_rn(make_float2(v[4 + l - m], v[5 + l - m]), make_float2(v[4 + l + m], v[5 + l + m]));
       const float2 zm = l == 0 ? make_float2(zc[4 - m].x, zc[4 - m].y)
                                : make_float2(zc[4 - m].z, zc[4 - m].w);
       const float2 zp = l == 0 ? make_float2(zc[4 + m].x, zc[4 + m].y)
                                : make_float2(zc[4 + m].z, zc[4 + m].w);
       if (ISO) {
-        const float2 s = __fadd2_rn(__fadd2_rn(xm, xp), __fadd2_rn(zm, zp));
+        const float2 s = __fadd2_rn(xs, __fadd2_rn(zm, zp));
         const float2 t = __ffma2_rn(ce, make_float2(-4.f, -4.f), s);
-        lap = __ffma2_rn(make_float2(k.ax[m - 1], k.ax[m - 1]), t, lap);
+        a = __ffma2_rn(make_float2(k.ax[m - 1], k.ax[m - 1]), t, a);
       } else {
-        const float2 tx = __ffma2_rn(ce, make_float2(-2.f, -2.f), __fadd2_rn(xm, xp));
-        lap = __ffma2_rn(make_float2(k.ax[m - 1], k.ax[m - 1]), tx, lap);
+        const float2 tx = __ffma2_rn(ce, make_float2(-2.f, -2.f), xs);
+        a = __ffma2_rn(make_float2(k.ax[m - 1], k.ax[m - 1]), tx, a);
         const float2 tz = __ffma2_rn(ce, make_float2(-2.f, -2.f), __fadd2_rn(zm, zp));
-        lap = __ffma2_rn(make_float2(k.az[m - 1], k.az[m - 1]), tz, lap);
+        a = __ffma2_rn(make_float2(k.az[m - 1], k.az[m - 1]), tz, a);
       }
     }
+    lap[l / 2] = a;
+  }
+}
+
+template <bool SPONGE, bool ISO>
+__device__ __forceinline__ float4 update4(const float4 *zc, const float4 &xl, const float4 &xr,
+                                          const float4 &dv, const float4 &cv, const Coef &k,
+                                          float gzr, const float *gxs) {
+  const float4 xc = zc[4];
+  float2 laps[2];
+  laplacian4<ISO>(zc, xl, xr, k, laps);
+  float out[4];
+#pragma unroll
+  for (int l = 0; l < 4; l += 2) {
+    const float2 ce = l == 0 ? make_float2(xc.x, xc.y) : make_float2(xc.z, xc.w);
+    const float2 lap = laps[l / 2];
     const float2 c = l == 0 ? make_float2(cv.x, cv.y) : make_float2(cv.z, cv.w);
     const float2 p = l == 0 ? make_float2(dv.x, dv.y) : make_float2(dv.z, dv.w);
     const float2 nd = __ffma2_rn(c, lap, p);
