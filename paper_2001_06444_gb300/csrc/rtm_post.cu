@@ -87,20 +87,152 @@ __global__ void k_filter(const float *stack_all, const float *comp_all, int nz, 
   out[(long long)smp * nz * nx + (long long)i * nx + j] = r;
 }
 
-// Per-pixel statistics over n images: FP64 two-pass mean and standard
-// deviation (divisor n-1), then a bitonic sort of each pixel's column in
-// shared memory for the 5% / 95% quantiles (linear interpolation at
-// h = (n-1) p).  A block stages PB pixels x npad values, pixel-fastest so
+// Per-pixel statistics over n images: mean and standard deviation (divisor
+// n-1) in FP64, and the 5% / 95% quantiles (linear interpolation at h = (n-1)
+// p).  A block stages PB pixels x n values in shared memory, pixel-fastest, so
 // global loads are coalesced and shared accesses are conflict-free.
+//
+// Two forms.  The general one sums in FP64, two passes, and sorts each pixel's
+// column (bitonic).  It is bound by FP64 arithmetic, which this device runs at
+// about 1/64 of the FP32 rate (5 FP64 operations a value), and by the sort:
+// 0.70 ms for 64 x 597,051.  The other (n <= kFastN, every value of the block
+// finite) takes one pixel per thread and no FP64 operation per value:
+//   - each value becomes an integer X on a grid 2^55 below the pixel's largest
+//     power of two (exact unless the value is 2^31 times smaller than the
+//     largest), so sum X is exact in 64 bits;
+//   - with M the rounded mean of the X, sum (X - M)^2 is exact in three 64-bit
+//     sums of products of 28-bit digits, and sum (X - mean)^2 = sum (X - M)^2 -
+//     R^2 / n with R = sum X - n M: no cancellation, at most one rounding each
+//     in FP64 per pixel;
+//   - the quantiles need the few smallest and largest values only: sorted lists
+//     of L in registers, 2 L minima and maxima a value.
+constexpr int kFastN = 128;
+
+// Quantile p of the sorted column from its two order statistics: separately
+// rounded multiply and add (no FMA contraction), so the FP64 value, and hence
+// its float rounding, is the textbook formula's.
+__device__ __forceinline__ float interpolate(float xl, float xh, double f) {
+  return (float)__dadd_rn((double)xl, __dmul_rn(f, __dsub_rn((double)xh, (double)xl)));
+}
+
+// The float with bits b as an integer on the grid 2^(emax - 181).
+__device__ __forceinline__ long long grid_value(unsigned b, int emax) {
+  const int e = (b >> 23) & 0xff;
+  const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | (e ? 0x800000u : 0u)) << 31;
+  const long long x = (long long)(m >> min(emax - max(e, 1), 63));
+  return (int)b < 0 ? -x : x;
+}
+
+// a / n correctly rounded from inv = 1 / n rounded (Markstein's correction)
+__device__ __forceinline__ double div_by(double a, double n, double inv) {
+  const double q = a * inv;
+  return __fma_rn(__fma_rn(-q, n, a), inv, q);
+}
+
+template <int L>
+__device__ __forceinline__ void fast_stats(const float *col, int n, int PB, int emax, double inv_n,
+                                           double inv_n1, int lo5, int lo95, double f5, double f95,
+                                           double &mean, double &sd, float &q5, float &q95) {
+  float lowest[L], highest[L];  // sorted: lowest[0] the smallest, highest[0] the largest
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    lowest[i] = INFINITY;
+    highest[i] = -INFINITY;
+  }
+  long long sum = 0;
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    const float v = col[k * PB];
+    sum += grid_value(__float_as_uint(v), emax);
+    float a = v, b = v;
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      const float c = fminf(lowest[i], a), d = fmaxf(highest[i], b);
+      if (i + 1 < L) {
+        a = fmaxf(lowest[i], a);
+        b = fminf(highest[i], b);
+      }
+      lowest[i] = c;
+      highest[i] = d;
+    }
+  }
+  const double scale = __hiloint2double((emax - 181 + 1023) << 20, 0);  // of the grid
+  const double mu = div_by((double)sum, (double)n, inv_n);
+  mean = mu * scale;
+  const long long M = __double2ll_rn(mu);
+  unsigned long long s00 = 0, s10 = 0, s11 = 0;
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    const long long d = grid_value(__float_as_uint(col[k * PB]), emax) - M;
+    const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
+    const unsigned a0 = (unsigned)a & 0xfffffffu, a1 = (unsigned)(a >> 28);
+    s00 += (unsigned long long)a0 * a0;
+    s10 += (unsigned long long)a1 * a0;
+    s11 += (unsigned long long)a1 * a1;
+  }
+  // (s10 < 2^63 and s11 <= 2^63 for n <= 128)
+  double q = __fma_rn((double)s11, 72057594037927936.0,
+                      __fma_rn((double)s10, 536870912.0, (double)s00));
+  const double R = (double)(sum - n * M);
+  q = __fma_rn(-R, R * inv_n, q);
+  sd = n > 1 ? sqrt(div_by(q, (double)(n - 1), inv_n1)) * scale : 0.0;
+  float a = lowest[0], b = lowest[0], c = highest[0], d = highest[0];
+  const int hi5 = min(lo5 + 1, n - 1), hi95 = min(lo95 + 1, n - 1);
+#pragma unroll
+  for (int i = 1; i < L; ++i) {
+    a = lo5 == i ? lowest[i] : a;
+    b = hi5 == i ? lowest[i] : b;
+    c = n - 1 - lo95 == i ? highest[i] : c;
+    d = n - 1 - hi95 == i ? highest[i] : d;
+  }
+  q5 = interpolate(a, b, f5);
+  q95 = interpolate(c, d, f95);
+}
+
+// L: length of the fast form's lists (0: the general form only)
+template <int L>
 __global__ void k_ens_stats(const float *images, int n, int npad, int PB, long long npix,
                             double *mean, double *std_, float *q05, float *q95) {
   extern __shared__ float sv[];  // [npad][PB]
   const long long p0 = (long long)blockIdx.x * PB;
-  for (int idx = threadIdx.x; idx < npad * PB; idx += blockDim.x) {
-    const int k = idx / PB, p = idx - k * PB;
-    float x = INFINITY;
-    if (k < n) x = (p0 + p < npix) ? images[(long long)k * npix + p0 + p] : 0.f;
-    sv[idx] = x;
+  // (rounded products: h - lo must not contract into one rounding)
+  const double h5 = __dmul_rn((double)(n - 1), 0.05), h95 = __dmul_rn((double)(n - 1), 0.95);
+  const int lo5 = (int)floor(h5), lo95 = (int)floor(h95);
+  if (L > 0) {
+    // one pixel per thread (blockDim.x >= PB)
+    const int p = threadIdx.x;
+    const bool in = p < PB && p0 + p < npix;
+    unsigned top = 0;  // largest magnitude's bits
+    if (p < PB) {
+      const float *src = images + p0 + p;
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) {
+        const float v = in ? __ldcs(src + (long long)k * npix) : 0.f;
+        sv[k * PB + p] = v;
+        top = max(top, __float_as_uint(v) & 0x7fffffffu);
+      }
+    }
+    if (!__syncthreads_or(top >= 0x7f800000u)) {  // all finite
+      if (!in) return;
+      double m, s;
+      float a, b;
+      fast_stats<L == 0 ? 1 : L>(sv + p, n, PB, max((int)(top >> 23), 1), 1.0 / n,
+                                 n > 1 ? 1.0 / (n - 1) : 0.0, lo5, lo95, h5 - lo5, h95 - lo95, m, s,
+                                 a, b);
+      mean[p0 + p] = m;
+      std_[p0 + p] = s;
+      q05[p0 + p] = a;
+      q95[p0 + p] = b;
+      return;
+    }
+    for (int idx = n * PB + threadIdx.x; idx < npad * PB; idx += blockDim.x) sv[idx] = INFINITY;
+  } else {
+    for (int idx = threadIdx.x; idx < npad * PB; idx += blockDim.x) {
+      const int k = idx / PB, p = idx - k * PB;
+      float x = INFINITY;
+      if (k < n) x = (p0 + p < npix) ? images[(long long)k * npix + p0 + p] : 0.f;
+      sv[idx] = x;
+    }
   }
   __syncthreads();
   double mu[2] = {0.0, 0.0}, sd[2] = {0.0, 0.0};
@@ -139,20 +271,8 @@ __global__ void k_ens_stats(const float *images, int n, int npad, int PB, long l
     if (pix >= npix) continue;
     mean[pix] = mu[t];
     std_[pix] = sd[t];
-    const double ps[2] = {0.05, 0.95};
-    float qo[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const double h = (double)(n - 1) * ps[u];
-      const int lo = (int)floor(h);
-      const int hi = min(lo + 1, n - 1);
-      const double xl = sv[lo * PB + p], xh = sv[hi * PB + p];
-      // separately rounded multiply and add (no FMA contraction), so the
-      // FP64 value, and hence its float rounding, is the textbook formula's
-      qo[u] = (float)__dadd_rn(xl, __dmul_rn(h - lo, __dsub_rn(xh, xl)));
-    }
-    q05[pix] = qo[0];
-    q95[pix] = qo[1];
+    q05[pix] = interpolate(sv[lo5 * PB + p], sv[min(lo5 + 1, n - 1) * PB + p], h5 - lo5);
+    q95[pix] = interpolate(sv[lo95 * PB + p], sv[min(lo95 + 1, n - 1) * PB + p], h95 - lo95);
   }
 }
 
@@ -161,12 +281,24 @@ __global__ void k_init_range(unsigned long long *mm) {
   mm[1] = 0x7FF0000000000000ull;  // +inf: min
 }
 
-__global__ void k_std_range(const double *std_, long long npix, unsigned long long *mm) {
+// Extremes of the map: one pair of atomics per block (a pair per warp on the
+// same two words took longer than the read).
+constexpr int kRangeThreads = 256, kRangeLoads = 4;
+__global__ void __launch_bounds__(kRangeThreads) k_std_range(const double *std_, long long npix,
+                                                             unsigned long long *mm) {
+  __shared__ double s_mx[kRangeThreads / 32], s_mn[kRangeThreads / 32];
   double mx = 0.0, mn = INFINITY;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < npix;
-       e += (long long)gridDim.x * blockDim.x) {
-    mx = fmax(mx, std_[e]);
-    mn = fmin(mn, std_[e]);
+  const long long stride = (long long)gridDim.x * kRangeThreads;
+  for (long long e = blockIdx.x * (long long)kRangeThreads + threadIdx.x; e < npix;
+       e += kRangeLoads * stride) {
+    double x[kRangeLoads];
+#pragma unroll
+    for (int k = 0; k < kRangeLoads; ++k) x[k] = std_[e + k * stride < npix ? e + k * stride : e];
+#pragma unroll
+    for (int k = 0; k < kRangeLoads; ++k) {
+      mx = fmax(mx, x[k]);
+      mn = fmin(mn, x[k]);
+    }
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
@@ -174,6 +306,15 @@ __global__ void k_std_range(const double *std_, long long npix, unsigned long lo
     mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
   }
   if ((threadIdx.x & 31) == 0) {
+    s_mx[threadIdx.x >> 5] = mx;
+    s_mn[threadIdx.x >> 5] = mn;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kRangeThreads / 32; ++w) {
+      mx = fmax(mx, s_mx[w]);
+      mn = fmin(mn, s_mn[w]);
+    }
     atomicMax(&mm[0], (unsigned long long)__double_as_longlong(mx));
     atomicMin(&mm[1], (unsigned long long)__double_as_longlong(mn));
   }
@@ -223,15 +364,23 @@ cudaError_t launch_ens_stats(const float *images, int n, long long npix, double 
   if (PB > 256) PB = 256;
   if (PB < 1) PB = 1;
   const size_t smem = (size_t)PB * npad * sizeof(float);
-  if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_ens_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   const long long blocks = (npix + PB - 1) / PB;
-  k_ens_stats<<<(unsigned)blocks, 256, smem, st>>>(images, n, npad, PB, npix, mean, std_, q05,
-                                                   q95);
-  return cudaGetLastError();
+  auto go = [&](auto kernel, int threads) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      cudaError_t e =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    kernel<<<(unsigned)blocks, threads, smem, st>>>(images, n, npad, PB, npix, mean, std_, q05, q95);
+    return cudaGetLastError();
+  };
+  // the fast form's lists hold the order statistics up to floor(0.05 (n-1)) + 1
+  // from either end: 3 for n <= 40, 5 for n <= 80, 8 for n <= 140
+  const int threads = (PB + 31) / 32 * 32;
+  if (n <= 40) return go(k_ens_stats<3>, threads);
+  if (n <= 80) return go(k_ens_stats<5>, threads);
+  if (n <= kFastN) return go(k_ens_stats<8>, threads);
+  return go(k_ens_stats<0>, 256);
 }
 
 cudaError_t launch_unc_maps(const double *mean, const double *std_, long long npix,
@@ -239,8 +388,9 @@ cudaError_t launch_unc_maps(const double *mean, const double *std_, long long np
                             cudaStream_t st) {
   k_init_range<<<1, 1, 0, st>>>(scratch);
   long long blocks = (npix + 255) / 256;
-  const unsigned rb = (unsigned)(blocks > 2048 ? 2048 : (blocks < 1 ? 1 : blocks));
-  k_std_range<<<rb, 256, 0, st>>>(std_, npix, scratch);
+  long long rb = (npix + kRangeThreads * kRangeLoads - 1) / (kRangeThreads * kRangeLoads);
+  if (rb > 4 * 152) rb = 4 * 152;
+  k_std_range<<<(unsigned)(rb < 1 ? 1 : rb), kRangeThreads, 0, st>>>(std_, npix, scratch);
   k_unc_maps<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(mean, std_, npix, scratch,
                                                                   conf, ratio);
   return cudaGetLastError();
