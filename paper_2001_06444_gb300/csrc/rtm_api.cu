@@ -459,14 +459,15 @@ struct Common {
 // tile kernels are the faster form or the grid does not fit.
 // Measured on a GB300 (600-step phases, FP32 and FP16 snapshots every 4 steps):
 //   a resident step takes 0.55 us + 0.1 us per strip of 4 points that a
-//   scheduler's threads own (rows x threads / 128), + 0.3 us backward with more
-//   than 4 rows a thread: 201 x 101 in 16 blocks 1.0-1.1 us, in 4 blocks 2.3-2.9
-//   us, 401 x 111 in 16 blocks 1.7 us; clusters beyond those that run at once
-//   take further rounds;
+//   scheduler's threads own (rows x threads / 128), + 0.15 us with more than 4
+//   rows a thread, + 0.4 us with more than 384 threads: 201 x 101 in 16 blocks
+//   1.0-1.2 us, in 4 blocks 2.3-2.9 us, 401 x 111 in 16 blocks 1.7 us, 501 x 181
+//   2.9-3.7 us; clusters beyond those that run at once take further rounds;
 //   a tile-kernel step takes 3.4 us, from 60 tiles (120 x 24) on about 3.0 us +
 //   6 ns a tile: 32 items of 201 x 101 6.5-7.8 us, 24 of 401 x 111 7.5-8.1 us.
-// Both sides at the line: 64 items of 201 x 101 4.8 us against 9.5, 24 of 401 x
-// 111 6.8 against 7.5 (forward), 8 of 851 x 176 do not fit.
+// Both sides near the line: 64 items of 201 x 101 4.8-6.4 us against 9.5-11.2,
+// one item of 501 x 181 3.0-3.7 against 3.4-4.1, 24 of 401 x 111 6.8-8.4 against
+// 7.5-8.1; 851 x 176 does not fit.
 // RTM_RESIDENT=C or C,R forces a cluster size (and rows a thread), 0 none.
 static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, int *max_ent) {
   const char *env = std::getenv("RTM_RESIDENT");
@@ -484,7 +485,8 @@ static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, 
     const int n = resident_clusters(p, ents);
     if (n < 1) continue;
     const double t = ((B + n - 1) / n) *
-                     (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0));
+                     (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0) +
+                      (p.threads > 384 ? 0.4 : 0.0));
     if (t < best_t) {
       best_t = t;
       best = p;

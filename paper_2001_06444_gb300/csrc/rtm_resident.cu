@@ -39,7 +39,7 @@ namespace {
 
 using namespace s2;
 
-constexpr int kResThreads = 384;  // of a block at most: 168 registers a thread
+constexpr int kResThreads[2] = {384, 512};  // of a block at most: two builds
 constexpr int kResCluster = 16;   // blocks of a cluster at most
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -156,9 +156,11 @@ __device__ __forceinline__ float4 update4_pre(const float4 *zc, const float4 &xl
 // What stays in registers depends on R: up to 3 rows a thread keep the sponge's
 // products (PRE), up to 4 keep num, den and the next snapshot (HOLD); beyond,
 // the sponge is evaluated from its factors and num and den go through L2 at
-// imaging steps.
-template <int MODE, int R>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_constant__ ResArgs A) {
+// imaging steps.  T: threads at most, 384 (168 registers each) or, for grids that
+// do not fit them, 512 (128 registers, some of them spilled: a 32-item phase of
+// 201 x 101 in 4 blocks takes 2.9-3.7 us a step with 512 threads, 2.6-3.2 with 384).
+template <int MODE, int R, int T>
+__global__ void __launch_bounds__(T, 1) k_resident(const __grid_constant__ ResArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool PRE = R <= 3, HOLD = R <= 4;
   constexpr bool SRC = MODE == MODE_FWD || MODE == MODE_MODEL, BWD = MODE == MODE_BWD;
@@ -244,17 +246,18 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int x = PRE ? r : 0;
-    gc[r] = d[r] = g2[x] = gq[x] = gm[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    d[r] = g2[x] = gq[x] = gm[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r < nr) {
       const long long o = (long long)(row0 + lr0 + r) * g.P + col;
-      gc[r] = __ldg(reinterpret_cast<const float4 *>(cc + o));
+      c = __ldg(reinterpret_cast<const float4 *>(cc + o));
       if (A.load_state) d[r] = *reinterpret_cast<const float4 *>(gd + o);
       if (PRE) {
         const float gz = A.gz[row0 + lr0 + r];
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
           const float gg = __fmul_rn(gz, A.gx[col + l]);
-          el4(gc[r], l) = __fmul_rn(gg, lane4(gc[r], l));
+          el4(c, l) = __fmul_rn(gg, lane4(c, l));
           if (gg == 1.f) {
             el4(gm[x], l) = 1.f;
           } else {
@@ -264,6 +267,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
         }
       }
     }
+    gc[r] = c;
   }
   // a warp clear of the sponge takes the interior formula
   const bool edge = nr > 0 && (row0 + lr0 < g.nb || row0 + lr0 + R > g.NZ - g.nb ||
@@ -360,9 +364,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (RTM_IN((long long)(i0 + r) * g.nx + min(j0 + 3, g.nx - 1), A.len.refl, A.err)) {
       const float *m = A.refl + (long long)(i0 + r) * g.nx + j0;
+      const float4 c = gc[r];
 #pragma unroll
       for (int l = 0; l < 4; ++l)
-        if (j0 + l < g.nx) el4(x, l) = __fmul_rn(lane4(gc[r], l), __ldg(m + l));
+        if (j0 + l < g.nx) el4(x, l) = __fmul_rn(lane4(c, l), __ldg(m + l));
     }
     return x;
   };
@@ -449,29 +454,35 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     if (IMG && img) snap_scale(A.snap_dtype, Smax, Ss, Sinv);
     float mx = 0.f;
     const long long soff = ((long long)b * A.nsnap + sidx) * g.pplane + pix0;
-    float4 nv[R];
-    auto rows = [&](auto sp, auto iso) {
+    // The rows in chunks of RC: within a chunk straight-line code, so that its
+    // rows' chains overlap; more rows at once would not leave the registers.
+    constexpr int RC = R <= 4 ? R : (R + 1) / 2;
+    float4 nvr[R <= 4 ? R : 1];  // v^{n+1} (more rows: read back from vout)
+    auto chunk = [&](auto sp, auto iso, auto first) {
       constexpr bool SP = decltype(sp)::value, ISO = decltype(iso)::value;
-      const float *w = vin + lr0 * PV + 4 + col;
-      float4 zc[R + 8], xl[R], xr[R];
+      constexpr int RA = decltype(first)::value, N = R - RA < RC ? R - RA : RC;
+      const float *w = vin + (lr0 + RA) * PV + 4 + col;
+      float4 zc[N + 8], xl[N], xr[N], nv[N];
 #pragma unroll
-      for (int z = 0; z < R + 8; ++z) zc[z] = *reinterpret_cast<const float4 *>(w + z * PV);
+      for (int z = 0; z < N + 8; ++z) zc[z] = *reinterpret_cast<const float4 *>(w + z * PV);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        xl[r] = *reinterpret_cast<const float4 *>(w + (r + 4) * PV - 4);
-        xr[r] = *reinterpret_cast<const float4 *>(w + (r + 4) * PV + 4);
+      for (int i = 0; i < N; ++i) {
+        xl[i] = *reinterpret_cast<const float4 *>(w + (i + 4) * PV - 4);
+        xr[i] = *reinterpret_cast<const float4 *>(w + (i + 4) * PV + 4);
       }
-      // (one block of straight-line code: the rows' chains overlap)
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+      for (int i = 0; i < N; ++i) {
+        const int r = RA + i;
         if constexpr (PRE)
-          d[r] = update4_pre<SP, ISO>(&zc[r], xl[r], xr[r], d[r], gc[r], g2[r], gq[r], gm[r], A.k);
+          d[r] = update4_pre<SP, ISO>(&zc[i], xl[i], xr[i], d[r], gc[r], g2[r], gq[r], gm[r], A.k);
         else
-          d[r] = update4<SP, ISO>(&zc[r], xl[r], xr[r], d[r], gc[r], A.k, SP ? s_gz[lr0 + r] : 1.f,
+          d[r] = update4<SP, ISO>(&zc[i], xl[i], xr[i], d[r], gc[r], A.k, SP ? s_gz[lr0 + r] : 1.f,
                                   s_gx + col);
+      }
       if (BORN && img) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
+        for (int i = 0; i < N; ++i) {
+          const int r = RA + i;
           if (((pmask >> r) & 1u) &&
               (KEEP || RTM_IN(soff + (long long)r * g.SX + 3, A.len.snap, A.err))) {
             const float4 S = snap_value4(KEEP ? Sp[KEEP ? r : 0] : snap_raw4(A.snap, soff + r * g.SX, A.snap_dtype),
@@ -486,31 +497,55 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
       }
       if ((SRC || BWD) && special) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
+        for (int i = 0; i < N; ++i) {
+          const int r = RA + i;
           if (SRC && r == src_r)
             set4(d[r], src_l, fmaf(lane4(gc[r], src_l), wav * A.src_scale, lane4(d[r], src_l)));
           if (BWD && ((rmask >> r) & 1u)) {
             const float *dat = s_dat + p * A.max_ent;
+            const float4 c = gc[r];
             if (rfast) {
-              d[r].x = __fadd_rn(d[r].x, __fmul_rn(gc[r].x, dat[rstart]));
-              d[r].y = __fadd_rn(d[r].y, __fmul_rn(gc[r].y, dat[rstart + 1]));
-              d[r].z = __fadd_rn(d[r].z, __fmul_rn(gc[r].z, dat[rstart + 2]));
-              d[r].w = __fadd_rn(d[r].w, __fmul_rn(gc[r].w, dat[rstart + 3]));
+              d[r].x = __fadd_rn(d[r].x, __fmul_rn(c.x, dat[rstart]));
+              d[r].y = __fadd_rn(d[r].y, __fmul_rn(c.y, dat[rstart + 1]));
+              d[r].z = __fadd_rn(d[r].z, __fmul_rn(c.z, dat[rstart + 2]));
+              d[r].w = __fadd_rn(d[r].w, __fmul_rn(c.w, dat[rstart + 3]));
             } else {
               const int e = r == rfirst ? rstart : first_ent(r), key = s_ent[e].x;
               for (int x = e; x < ne && s_ent[x].x == key; ++x) {
                 const int l = s_ent[x].y & 3;
-                set4(d[r], l, __fadd_rn(lane4(d[r], l), __fmul_rn(lane4(gc[r], l), dat[x])));
+                set4(d[r], l, __fadd_rn(lane4(d[r], l), __fmul_rn(lane4(c, l), dat[x])));
               }
             }
           }
         }
       }
+      // the rows that border a neighbour go out first
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const float4 ce = zc[r + 4];
-        nv[r] = make_float4(ce.x + d[r].x, ce.y + d[r].y, ce.z + d[r].z, ce.w + d[r].w);
+      for (int i = 0; i < N; ++i) {
+        const int r = RA + i;
+        const float4 ce = zc[i + 4];
+        nv[i] = make_float4(ce.x + d[r].x, ce.y + d[r].y, ce.z + d[r].z, ce.w + d[r].w);
+        if (R <= 4) nvr[R <= 4 ? r : 0] = nv[i];
       }
+      if (border && more) {
+        const unsigned ro = (unsigned)((p ^ 1) * plane_v + (lr0 + 4) * PV + 4 + col);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const int r = RA + i;
+          if (r < nr && has_next && lr0 + r >= H - 4)
+            st_async4(v_next + (ro + (r - H) * PV) * 4, b_next + 8 * (p ^ 1), nv[i]);
+          if (r < nr && has_prev && lr0 + r < 4)
+            st_async4(v_prev + (ro + (r + H) * PV) * 4, b_prev + 8 * (p ^ 1), nv[i]);
+        }
+      }
+      float *wo = vout + (lr0 + RA + 4) * PV + 4 + col;
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (RA + i < nr) *reinterpret_cast<float4 *>(wo + i * PV) = nv[i];
+    };
+    auto rows = [&](auto sp, auto iso) {
+      chunk(sp, iso, std::integral_constant<int, 0>());
+      if constexpr (RC < R) chunk(sp, iso, std::integral_constant<int, RC>());
     };
     if (nr > 0) {
       const std::true_type yes;
@@ -523,23 +558,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
         else rows(no, no);
       }
     }
-    // the rows that border a neighbour go out first
-    if (border && more) {
-      const unsigned ro = (unsigned)((p ^ 1) * plane_v + (lr0 + 4) * PV + 4 + col);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (r < nr && has_next && lr0 + r >= H - 4)
-          st_async4(v_next + (ro + (r - H) * PV) * 4, b_next + 8 * (p ^ 1), nv[r]);
-        if (r < nr && has_prev && lr0 + r < 4)
-          st_async4(v_prev + (ro + (r + H) * PV) * 4, b_prev + 8 * (p ^ 1), nv[r]);
-      }
-    }
-    if (nr > 0) {
-      float *wo = vout + (lr0 + 4) * PV + 4 + col;
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (r < nr) *reinterpret_cast<float4 *>(wo + r * PV) = nv[r];
-    }
+    auto value = [&](int r) {  // v^{n+1} of this thread's row r
+      return R <= 4 ? nvr[R <= 4 ? r : 0]
+                    : *reinterpret_cast<const float4 *>(vout + (lr0 + r + 4) * PV + 4 + col);
+    };
     if (REC && special) {
       const long long o = ((long long)b * A.nt + t) * A.nrec;
 #pragma unroll
@@ -548,16 +570,17 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
         if (rfast) {
           if (RTM_IN(o + rfirst_rec + 3, A.len.rec_out, A.err)) {
             float *out = A.rec_out + o + rfirst_rec;
-            out[0] = nv[r].x;
-            out[1] = nv[r].y;
-            out[2] = nv[r].z;
-            out[3] = nv[r].w;
+            const float4 x = value(r);
+            out[0] = x.x;
+            out[1] = x.y;
+            out[2] = x.z;
+            out[3] = x.w;
           }
         } else {
           const int e = r == rfirst ? rstart : first_ent(r), key = s_ent[e].x;
           for (int x = e; x < ne && s_ent[x].x == key; ++x)
             if (RTM_IN(o + (s_ent[x].y >> 2), A.len.rec_out, A.err))
-              A.rec_out[o + (s_ent[x].y >> 2)] = lane4(nv[r], s_ent[x].y & 3);
+              A.rec_out[o + (s_ent[x].y >> 2)] = lane4(value(r), s_ent[x].y & 3);
         }
       }
     }
@@ -565,8 +588,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if (!((pmask >> r) & 1u)) continue;
+        float4 x = value(r);
         if (A.snap_dtype == 0) {
-          float4 x = nv[r];
           if (j0 + 1 >= g.nx) x.y = 0.f;
           if (j0 + 2 >= g.nx) x.z = 0.f;
           if (j0 + 3 >= g.nx) x.w = 0.f;
@@ -575,14 +598,14 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
         } else {
 #pragma unroll
           for (int l = 0; l < 4; ++l)
-            if (j0 + l < g.nx) mx = fmaxf(mx, fabsf(lane4(nv[r], l)));
+            if (j0 + l < g.nx) mx = fmaxf(mx, fabsf(lane4(x, l)));
         }
       }
     }
     if (KEEP && BWD && img) {
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        image_add(snap_value4(Sp[KEEP ? r : 0], A.snap_dtype, Ss), nv[r], num[KB > 1 ? r : 0],
+        image_add(snap_value4(Sp[KEEP ? r : 0], A.snap_dtype, Ss), value(r), num[KB > 1 ? r : 0],
                   den[KB > 1 ? r : 0]);
     }
     if (!KEEP && BWD && img) {  // num and den through L2, two rows' loads in flight at once
@@ -600,7 +623,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
 #pragma unroll
         for (int y = 0; y < 2; ++y)
           if (r2 + y < R && ((pmask >> (r2 + y)) & 1u) && ok_img(r2 + y, soff)) {
-            image_add(snap_value4(raw[y], A.snap_dtype, Ss), nv[r2 + y < R ? r2 + y : 0], nu[y], de[y]);
+            image_add(snap_value4(raw[y], A.snap_dtype, Ss), value(r2 + y), nu[y], de[y]);
             *reinterpret_cast<float4 *>(A.num + pbase + (r2 + y) * g.SX) = nu[y];
             *reinterpret_cast<float4 *>(A.den + pbase + (r2 + y) * g.SX) = de[y];
             if (k == isnap) dm = fmaxf(dm, fmaxf(fmaxf(de[y].x, de[y].y), fmaxf(de[y].z, de[y].w)));
@@ -686,16 +709,16 @@ size_t res_smem(const ResPlan &p, int max_ent) {
 constexpr size_t kResSmem = 226 << 10;
 
 template <class F>
-cudaError_t with_kernel(int mode, int R, F f) {
-#define RTM_RES_ROWS(M)                          \
-  switch (R) {                                   \
-    case 1: return f(k_resident<M, 1>);          \
-    case 2: return f(k_resident<M, 2>);          \
-    case 3: return f(k_resident<M, 3>);          \
-    case 4: return f(k_resident<M, 4>);          \
-    case 5: return f(k_resident<M, 5>);          \
-    case 6: return f(k_resident<M, 6>);          \
-  }                                              \
+cudaError_t with_kernel(int mode, const ResPlan &p, F f) {
+#define RTM_RES_ROWS(M)                                                             \
+  switch (p.R) {                                                                     \
+    case 1: return f(k_resident<M, 1, 384>);                                         \
+    case 2: return f(k_resident<M, 2, 384>);                                         \
+    case 3: return f(k_resident<M, 3, 384>);                                         \
+    case 4: return f(k_resident<M, 4, 384>);                                         \
+    case 5: return p.threads <= 384 ? f(k_resident<M, 5, 384>) : f(k_resident<M, 5, 512>); \
+    case 6: return p.threads <= 384 ? f(k_resident<M, 6, 384>) : f(k_resident<M, 6, 512>); \
+  }                                                                                  \
   break;
   switch (mode) {
     case MODE_FWD: RTM_RES_ROWS(MODE_FWD)
@@ -738,12 +761,17 @@ bool resident_shape(const Geo &g, int C, int R, ResPlan &p) {
   p.NS = (g.X0 + g.NX + 3) / 4;
   p.H = (g.NZ + C - 1) / C;
   if (C > 1 && p.H < HALO) return false;  // a halo spans one neighbour
-  for (p.R = R > 0 ? R : 1; p.R <= kResRows; ++p.R) {
-    p.G = (p.H + p.R - 1) / p.R;
-    if (p.NS * p.G <= kResThreads) break;
-    if (R > 0) return false;
+  // the fewest rows a thread that fit 384 threads, else (5 rows and more) 512
+  bool fits = false;
+  for (int t : kResThreads) {
+    for (p.R = R > 0 ? R : (t > 384 ? 5 : 1); !fits && p.R <= (R > 0 ? R : kResRows); ++p.R) {
+      p.G = (p.H + p.R - 1) / p.R;
+      fits = p.NS * p.G <= t && (t <= 384 || p.R >= 5);
+      if (fits) break;
+    }
+    if (fits) break;
   }
-  if (p.R > kResRows) return false;
+  if (!fits) return false;
   p.threads = (p.NS * p.G + 31) / 32 * 32;
   return res_smem(p, 0) <= kResSmem;
 }
@@ -774,7 +802,7 @@ int resident_clusters(const ResPlan &p, int max_ent) {
   int n = 0;
   Launch l(p, p.C, (smem + 1023) & ~(size_t)1023, nullptr);
   // (the backward kernel: the one that takes the most registers)
-  const cudaError_t e = with_kernel(MODE_BWD, p.R, [&](auto kernel) {
+  const cudaError_t e = with_kernel(MODE_BWD, p, [&](auto kernel) {
     cudaError_t r = allow(kernel);
     return r == cudaSuccess ? cudaOccupancyMaxActiveClusters(&n, kernel, &l.cfg) : r;
   });
@@ -796,7 +824,7 @@ cudaError_t launch_resident(int mode, const ResPlan &p, ResArgs A, int B, cudaSt
   const size_t smem = res_smem(p, A.max_ent);
   if (smem > kResSmem) return cudaErrorInvalidValue;
   Launch l(p, B * p.C, smem, st);
-  return with_kernel(mode, p.R, [&](auto kernel) {
+  return with_kernel(mode, p, [&](auto kernel) {
     const cudaError_t e = allow(kernel);
     return e == cudaSuccess ? cudaLaunchKernelEx(&l.cfg, kernel, A) : e;
   });

@@ -79,6 +79,7 @@ def _survey(nx, nz, nb, dx, dz, nt, receivers):
     (90, 47, 20, 12.0, 101, "reversed", ("16,1", "16,4", "4,3", "2,6")),
     (5, 69, 0, 10.0, 57, "scattered", ("16,1", "8,2", "2,5")),
     (201, 101, 20, 10.0, 90, "row", ("16", "8", "4")),
+    (470, 90, 20, 10.0, 40, "row", ("8,5", "8,6", "16,4")),
 ])
 def test_resident_phases_equal_single_steps(nx, nz, nb, dz, nt, receivers, shapes):
     s = _survey(nx, nz, nb, 10.0, dz, nt, receivers)
