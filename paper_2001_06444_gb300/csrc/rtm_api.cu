@@ -455,6 +455,10 @@ struct Common {
   int res_max_ent = 0;
 };
 
+static double tile_step_us(double n, int tile_z);
+static double tiles_of(const Geo &g, int B, int tile_z);
+static int best_tile(const Geo &g, int B);
+
 // How B items' phases run with the grid on chip (k_resident), or C = 0 if the
 // tile kernels are the faster form or the grid does not fit.
 // Measured on a GB300 (600-step phases, FP32 and FP16 snapshots every 4 steps):
@@ -463,19 +467,18 @@ struct Common {
 //   rows a thread, + 0.4 us with more than 384 threads: 201 x 101 in 16 blocks
 //   1.0-1.2 us, in 4 blocks 2.3-2.9 us, 401 x 111 in 16 blocks 1.7 us, 501 x 181
 //   2.9-3.7 us; clusters beyond those that run at once take further rounds;
-//   a tile-kernel step takes 3.4 us, from 60 tiles (120 x 24) on about 3.0 us +
-//   6 ns a tile: 32 items of 201 x 101 6.5-7.8 us, 24 of 401 x 111 7.5-8.1 us.
-// Both sides near the line: 64 items of 201 x 101 4.8-6.4 us against 9.5-11.2,
-// one item of 501 x 181 3.0-3.7 against 3.4-4.1, 24 of 401 x 111 6.8-8.4 against
-// 7.5-8.1; 851 x 176 does not fit.
+//   a tile-kernel step as tile_step_us.
+// Both sides near the line: 64 items of 201 x 101 4.8-6.4 us against 7.7, 7 of
+// 501 x 181 3.0-3.8 against 4.7, one of them 3.0-3.6 against 2.6; 851 x 176 does
+// not fit.
 // RTM_RESIDENT=C or C,R forces a cluster size (and rows a thread), 0 none.
 static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, int *max_ent) {
   const char *env = std::getenv("RTM_RESIDENT");
   int fc = 0, fr = 0;
   if (env) std::sscanf(env, "%d,%d", &fc, &fr);
   if (env && fc <= 0) return ResPlan{};
-  const double tiles = (double)B * g.ntx2 * ((g.NZ + 23) / 24);
-  double best_t = fc > 0 ? 1e300 : std::max(3.4, 3.0 + 0.006 * tiles);
+  const int tz = best_tile(g, B);
+  double best_t = fc > 0 ? 1e300 : tile_step_us(tiles_of(g, B, tz), tz);
   ResPlan best, p;
   for (int C : {16, 8, 4, 2, 1}) {
     if (fc > 0 && C != fc) continue;
@@ -494,6 +497,50 @@ static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, 
     }
   }
   return best;
+}
+
+// Estimated time of a two-step launch's step (us) over n tiles of tile_z rows
+// with kernel 4 as a programmatic dependent of the launch before, fitted to 11
+// workloads from 201 x 101 x 1 to 1701 x 351 x 48 (migration and modelling):
+// up to 152 tiles one block an SM, its latency; up to 456 one wave of 3 blocks an
+// SM; beyond, throughput.  Measured against the two-step kernel 2 that ran
+// before (us a step): 1 item of 851 x 176 2.6 against 3.7 (16 rows), 4 of them
+// 3.7 against 4.8 (16), 8 of them 5.4 against 7.0 (32), 1701 x 351 x 4 8.5
+// against 9.2 (32), 2401 x 601 x 1 5.3 against 7.0 (32).
+static double tile_step_us(double n, int tile_z) {
+  switch (tile_z) {
+    case 16: return n <= 152 ? 2.55 : n <= 456 ? 2.55 + 0.0037 * (n - 152) : 1.6 + 0.0050 * n;
+    case 24:
+      return n <= 152   ? 2.85
+             : n <= 456 ? std::min(5.3, 2.85 + 0.0105 * (n - 152))
+                        : std::max(5.3, 2.35 + 0.0062 * n);
+    default: return n <= 152 ? 3.3 : n <= 456 ? 3.85 + 0.005 * (n - 152) : 2.7 + 0.0076 * n;
+  }
+}
+
+static double tiles_of(const Geo &g, int B, int tile_z) {
+  return (double)B * g.ntx2 * ((g.NZ + tile_z - 1) / tile_z);
+}
+
+static int best_tile(const Geo &g, int B) {
+  int best = 24;
+  for (int z : {16, 32})
+    if (tile_step_us(tiles_of(g, B, z), z) < tile_step_us(tiles_of(g, B, best), best)) best = z;
+  return best;
+}
+
+// The launch configuration of B items in flight where it is left to the
+// library.  Programmatic dependent launches gain while a launch's start and end
+// are a good part of it (see tile_step_us); a launch of more tiles than about
+// 6000 (13 waves) only loses block slots to the blocks that wait for it (48
+// items of 1701 x 351, modelling: 66.0 us a step against 63.1 without).
+static RunConfig resolve_config(RunConfig c, const Geo &g, int B) {
+  if (c.step_kernel == 0) {
+    c.step_kernel = 4;
+    c.tile_z = best_tile(g, B);
+  }
+  if (c.pdl < 0) c.pdl = c.step_kernel == 4 && tiles_of(g, B, c.tile_z) <= 6000;
+  return c;
 }
 
 // Chooses the resident form for B items in flight and uploads its receiver table.
@@ -552,12 +599,12 @@ static void step2_receiver_lists(const Geo &g, const rtm_acq &acq, std::vector<i
 
 // Upload the per-call tables shared by all items.
 static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_acq &acq,
-                        int nsample, const float *vel_d, cudaStream_t st, int step_kernel,
-                        int tile_z, int l2_ahead, int pdl) {
-  C.g = make_geo(gr, step_kernel >= 3 ? tile_z : 24);
+                        int nsample, const float *vel_d, cudaStream_t st, const RunConfig &cfg) {
+  const int step_kernel = cfg.step_kernel;
+  C.g = make_geo(gr, step_kernel >= 3 ? cfg.tile_z : 24);
   C.kernel = step_kernel;
-  C.l2_ahead = l2_ahead;
-  C.pdl = pdl;
+  C.l2_ahead = cfg.l2_ahead;
+  C.pdl = cfg.pdl;
   C.k = make_coef(gr);
   C.nsample = nsample;
   const Geo &g = C.g;
@@ -775,8 +822,7 @@ static int step2(rtm_ctx *ctx, int mode, Step2Args &A2, const Common &C, Fields 
   Step2RT r = rt;
   r.reverse = F.n2 & 1;
   r.ahead = C.l2_ahead;
-  // (programmatic dependent launches are built for the migration's phases)
-  r.pdl = C.kernel == 4 && C.pdl && (mode == MODE_FWD || mode == MODE_BWD);
+  r.pdl = C.kernel == 4 && C.pdl;
   if (C.kernel == 3)
     CU(launch_step2p(mode, C.g.tz2, F.mv[F.cv], F.md[F.cd], C.mc, A2, r, nb, st));
   else if (C.kernel == 4)
@@ -830,19 +876,19 @@ static int run_phase(rtm_ctx *ctx, bool graph, cudaStream_t st, F issue) {
 
 int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *vel_d,
                    const rtm_acq &acq, const float *seis_d, const rtm_opts &op, float *img_d,
-                   int B, cudaStream_t st, const RunConfig &cfg, const float *born_refl,
+                   int B, cudaStream_t st, const RunConfig &wanted, const float *born_refl,
                    float *born_out, LateCopy *late, int flag_slot) {
   Common C;
   int rc;
-  {
-    PhaseRange ph("setup");
-    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg.step_kernel, cfg.tile_z,
-                      cfg.l2_ahead, cfg.pdl);
-  }
-  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   const long long nitems = (long long)nsample * acq.nshot;
   if (B > nitems) B = (int)nitems;
   if (B < 1) B = 1;
+  const RunConfig cfg = resolve_config(wanted, make_geo(gr), B);
+  {
+    PhaseRange ph("setup");
+    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg);
+  }
+  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   if (!rc && cfg.resident) rc = setup_resident(ctx, C, acq, B, st);
   if (rc) return rc;
   trace_mark("tables and model set up");
@@ -1231,15 +1277,15 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
 static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
                         const rtm_acq &acq, int s0, int ns, float *seis_d, int B,
                         cudaStream_t st, int flag_slot) {
-  const int sk = ctx->defaults.step_kernel;
+  if (B > ns) B = ns;
+  if (B < 1) B = 1;
+  const RunConfig cfg = resolve_config(ctx->defaults, make_geo(gr), B);
+  const int sk = cfg.step_kernel;
   Common C;
-  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, sk, ctx->defaults.tile_z,
-                        ctx->defaults.l2_ahead, ctx->defaults.pdl);
+  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, cfg);
   if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   if (rc) return rc;
   const Geo &g = C.g;
-  if (B > ns) B = ns;
-  if (B < 1) B = 1;
   std::vector<int> items(2 * (size_t)ns);
   for (int q = 0; q < ns; ++q) {
     items[q] = 0;
@@ -1423,28 +1469,30 @@ int rtm_ctx_create(rtm_ctx **out, int device, size_t hbm_budget_bytes) {
     ctx->h_flags[2 * i] = ctx->h_flags[2 * i + 1] = 0;
     ctx->free_flags.push_back(i);
   }
-  // RTM_STEP_KERNEL picks the context's default propagation kernel: 1 the
-  // single-step kernel, 2 (default) the two-step kernel with one tile per
-  // block (RTM_L2_AHEAD=1 turns on its L2 prefetch of later tiles), 3 the
-  // persistent two-step kernel (RTM_TILE_Z=16 for 16-row tiles), 4 the
-  // two-step kernel with v^{n+1} over v^n (RTM_TILE_Z=32 for 32-row tiles)
+  // RTM_STEP_KERNEL picks the context's default propagation kernel (unset: the
+  // library chooses kernel 4 and its tile by the launch's size): 1 the
+  // single-step kernel, 2 the two-step kernel with one tile per block
+  // (RTM_L2_AHEAD=1 turns on its L2 prefetch of later tiles), 3 the persistent
+  // two-step kernel (RTM_TILE_Z=16 for 16-row tiles), 4 the two-step kernel with
+  // v^{n+1} over v^n (RTM_TILE_Z=16 or 32 for tiles of 16 or 32 rows)
   const char *sk = std::getenv("RTM_STEP_KERNEL");
+  const char *la = std::getenv("RTM_L2_AHEAD");
+  ctx->defaults.l2_ahead = (la && la[0] == '1') ? 1 : 0;
   const int k = sk ? std::atoi(sk) : 0;
-  ctx->defaults.step_kernel = (k >= 1 && k <= 4) ? k : 2;
+  ctx->defaults.step_kernel = (k >= 1 && k <= 4) ? k : (sk || ctx->defaults.l2_ahead) ? 2 : 0;
   // (a chosen kernel runs every phase; RTM_RESIDENT=0 keeps phases off chip)
   const char *rs = std::getenv("RTM_RESIDENT");
   ctx->defaults.resident = !sk && !(rs && rs[0] == '0');
   const char *tz = std::getenv("RTM_TILE_Z");
   const int z = tz ? std::atoi(tz) : 24;
-  ctx->defaults.tile_z = ((z == 16 && k == 3) || (z == 32 && k == 4)) ? z : 24;
-  const char *la = std::getenv("RTM_L2_AHEAD");
-  ctx->defaults.l2_ahead = (la && la[0] == '1') ? 1 : 0;
+  ctx->defaults.tile_z = ((z == 16 && k >= 3) || (z == 32 && k == 4)) ? z : 24;
   // RTM_IMAGE_INPUT=1: backward launches image their input field where they can
   const char *ii = std::getenv("RTM_IMAGE_INPUT");
   ctx->defaults.image_input = (ii && ii[0] == '1') ? 1 : 0;
-  // RTM_PDL=1: the kernel-4 launches are programmatic dependents of the previous one
+  // RTM_PDL=1 / 0: the kernel-4 launches are / are not programmatic dependents of
+  // the previous one (unset: by the launch's size)
   const char *pd = std::getenv("RTM_PDL");
-  ctx->defaults.pdl = (pd && pd[0] == '1') ? 1 : 0;
+  ctx->defaults.pdl = pd ? (pd[0] == '1') : -1;
   // RTM_GRAPHS=1 captures each phase of a batch in a CUDA graph by default
   const char *gr = std::getenv("RTM_GRAPHS");
   ctx->defaults.graph = (gr && gr[0] == '1') ? 1 : 0;

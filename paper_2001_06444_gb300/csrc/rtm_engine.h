@@ -21,16 +21,18 @@ struct rtm_server;
 namespace rtm {
 // How a migration is launched (all choices give bit-identical results).
 struct RunConfig {
-  int step_kernel = 2;  // 2: two-step kernel, one tile per block, where possible;
+  int step_kernel = 0;  // 0: chosen with its tile by the launch's size (resolve_config);
+                        // 2: two-step kernel, one tile per block, where possible;
                         // 3: persistent two-step kernel with a copy ring;
                         // 4: two-step kernel, one tile per block, v^{n+1} over v^n;
                         // 1: single-step only
   int max_items = 0;    // cap on items in flight (0 = memory budget)
   int graph = 0;        // 1: capture each phase of a batch in a CUDA graph
-  int tile_z = 24;      // centre rows of a two-step tile (16 with kernel 3, 32 with kernel 4)
+  int tile_z = 24;      // centre rows of a two-step tile (16 with kernels 3 and 4, 32 with kernel 4)
   int l2_ahead = 0;     // step_kernel 2: each block prefetches a later block's tile into L2
   int image_input = 0;  // two-step backward launches image their input field where they can
-  int pdl = 0;          // step_kernel 4: programmatic dependent launches (griddepcontrol)
+  int pdl = -1;         // step_kernel 4: programmatic dependent launches (griddepcontrol);
+                        // -1: chosen by the launch's size
   int resident = 1;     // run phases with the grid on chip where that is faster (resident_plan)
 };
 // Shape key of the autotuner cache.

@@ -736,21 +736,19 @@ size_t step2p_smem_bytes(int tile_z) {
 }
 
 size_t step2a_smem_bytes(int tile_z) {
-  return (tile_z == 32 ? sizeof(Smem1<5>) : sizeof(Smem1<4>)) + 128;
+  return (tile_z == 32 ? sizeof(Smem1<5>) : tile_z == 16 ? sizeof(Smem1<3>) : sizeof(Smem1<4>)) + 128;
 }
 
 cudaError_t launch_step2a(int mode, int tile_z, const CUtensorMap &mv, const CUtensorMap &md,
                           const CUtensorMap &mc, const Step2Args &A, const Step2RT &rt, int B,
                           cudaStream_t st) {
-  if (tile_z != 24 && tile_z != 32) return cudaErrorInvalidValue;
+  if (tile_z != 16 && tile_z != 24 && tile_z != 32) return cudaErrorInvalidValue;
   const long long ntl = (long long)B * A.g.ntx2 * A.g.ntz2;
   if (ntl < 1 || ntl > 0x7fffffffLL) return cudaErrorInvalidValue;
-  // the input-field imaging and programmatic-dependent instances exist for the
-  // backward and forward migration phases only
+  // the input-field imaging instances exist for the backward phase only
   const bool in_img = rt.img_in_idx >= 0 || rt.dmax_flag == 3;
   if (in_img && mode != MODE_BWD) return cudaErrorInvalidValue;
-  if (rt.pdl && mode != MODE_BWD && mode != MODE_FWD) return cudaErrorInvalidValue;
-  static std::atomic<bool> attr_set[32];
+  static std::atomic<bool> attr_set[48];
   const size_t smem = step2a_smem_bytes(tile_z);
   dim3 block(32, NTH / 32);
   auto launch = [&](auto kernel, int slot) -> cudaError_t {
@@ -778,28 +776,27 @@ cudaError_t launch_step2a(int mode, int tile_z, const CUtensorMap &mv, const CUt
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, mv, md, mc, A, rt, (int)ntl);
   };
-  // slot = 16 * (tile_z == 32) + 4 * mode + VAR
+  // slot = 16 * (0: 24 rows, 1: 32, 2: 16) + 4 * mode + VAR
   const int var = (in_img ? 1 : 0) | (rt.pdl ? 2 : 0);
-  const int slot = (tile_z == 32 ? 16 : 0) + 4 * mode + var;
-#define RTM_S2A(M, R, V) launch(k_step2a<M, R, V>, (R == 5 ? 16 : 0) + 4 * M + V)
+  const int slot = (tile_z == 32 ? 16 : tile_z == 16 ? 32 : 0) + 4 * mode + var;
+#define RTM_S2A(M, R, V) launch(k_step2a<M, R, V>, (R == 5 ? 16 : R == 3 ? 32 : 0) + 4 * M + V)
+#define RTM_S2A_ALL(BASE, R)                             \
+  case BASE + 0: return RTM_S2A(MODE_FWD, R, 0);         \
+  case BASE + 2: return RTM_S2A(MODE_FWD, R, 2);         \
+  case BASE + 4: return RTM_S2A(MODE_MODEL, R, 0);       \
+  case BASE + 6: return RTM_S2A(MODE_MODEL, R, 2);       \
+  case BASE + 8: return RTM_S2A(MODE_BWD, R, 0);         \
+  case BASE + 9: return RTM_S2A(MODE_BWD, R, 1);         \
+  case BASE + 10: return RTM_S2A(MODE_BWD, R, 2);        \
+  case BASE + 11: return RTM_S2A(MODE_BWD, R, 3);        \
+  case BASE + 12: return RTM_S2A(MODE_BORN, R, 0);       \
+  case BASE + 14: return RTM_S2A(MODE_BORN, R, 2);
   switch (slot) {
-    case 0: return RTM_S2A(MODE_FWD, 4, 0);
-    case 2: return RTM_S2A(MODE_FWD, 4, 2);
-    case 4: return RTM_S2A(MODE_MODEL, 4, 0);
-    case 8: return RTM_S2A(MODE_BWD, 4, 0);
-    case 9: return RTM_S2A(MODE_BWD, 4, 1);
-    case 10: return RTM_S2A(MODE_BWD, 4, 2);
-    case 11: return RTM_S2A(MODE_BWD, 4, 3);
-    case 12: return RTM_S2A(MODE_BORN, 4, 0);
-    case 16: return RTM_S2A(MODE_FWD, 5, 0);
-    case 18: return RTM_S2A(MODE_FWD, 5, 2);
-    case 20: return RTM_S2A(MODE_MODEL, 5, 0);
-    case 24: return RTM_S2A(MODE_BWD, 5, 0);
-    case 25: return RTM_S2A(MODE_BWD, 5, 1);
-    case 26: return RTM_S2A(MODE_BWD, 5, 2);
-    case 27: return RTM_S2A(MODE_BWD, 5, 3);
-    case 28: return RTM_S2A(MODE_BORN, 5, 0);
+    RTM_S2A_ALL(0, 4)
+    RTM_S2A_ALL(16, 5)
+    RTM_S2A_ALL(32, 3)
   }
+#undef RTM_S2A_ALL
 #undef RTM_S2A
   return cudaErrorInvalidValue;
 }
