@@ -36,11 +36,12 @@
 // Decoding, per group of arrays, in two passes with no device-side waiting:
 //   1. the walk: one thread per chunk (a CTA's chunks ordered by size first)
 //      finds the bit offset and the cost class (events, members) of every
-//      block; the CTA lists its blocks that are not all zero in class order
-//      (a segment of the decode's list) and writes its all-zero blocks to
-//      the output, row by row;
-//   2. the decode: a CTA per segment, one block per thread in list order,
-//      so that the lanes of a warp run the same loops for as many trips.
+//      block; the CTA lists its blocks that are not all zero in class order,
+//      window by window (1024 consecutive blocks);
+//   2. the decode: a CTA per window, one block per thread in list order, so
+//      that the lanes of a warp run the same loops for as many trips; the
+//      window's values come together in shared memory and are written row by
+//      row.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -68,10 +69,13 @@ constexpr int kWalk = 128;               // decoder's walk: chunks per CTA, one 
 constexpr int kWalkKeys = 64;            // size classes the walk orders chunks by
 constexpr int kSeg = kWalk * kChunk;     // blocks of a walk CTA: a segment of the decode's list
 constexpr int kClasses = 256;            // decode cost classes (0: all-zero blocks)
-constexpr int kDec = 256;                // decoder: threads per CTA, one block per thread
+constexpr int kWin = 1024;               // blocks of a decode window
+constexpr int kSegWins = kSeg / kWin;    // windows of a segment
+constexpr int kDec = 512;                // decoder: threads per CTA, one block per thread
+constexpr int kOutPitch = 4 * kWin + 8;  // floats of a window's row in shared memory
 constexpr u64 kGroupBlocks = 1ull << 24; // list entries per group of arrays
-static_assert(kClasses % kWalk == 0 && kWalk % 32 == 0 && kWalk >= 64,
-              "class counts spread evenly over the walk threads");
+static_assert(kSegWins == kWalk / 32 && kClasses % 32 == 0 && kSeg % kWin == 0,
+              "a warp of the walk scans the class counts of one window");
 static_assert(kSeg <= (1 << 13), "a segment's block index takes 13 bits of a list entry");
 constexpr int kHeader = 64;
 constexpr u32 kMagic = 0x5A4D5452u;
@@ -120,9 +124,9 @@ struct DecArgs {
   u32 arr0;       // first array of this group (error reports)
   u32 count;      // arrays in this group
   u32 nseg;       // segments (kWalk chunks, kSeg blocks) per array
-  u32 *list;      // [count][nseg][kSeg] per segment: its blocks not all zero, in class
-                  // order: index in the segment << 15 | bit offset in the chunk
-  u32 *segcount;  // [count][nseg] entries of each segment's list
+  u32 *list;      // [count][nseg][kSegWins][kWin] per window: its blocks not all zero, in
+                  // class order: index in the segment << 15 | bit offset in the chunk
+  u32 *wincount;  // [count][nseg][kSegWins] entries of each window's list
 };
 
 // kmin for every block exponent of a tolerance: the largest k in [1, 30]
@@ -665,104 +669,88 @@ __device__ __forceinline__ bool significance(R &rd, int kmin, unsigned char *sfx
   return true;
 }
 
-// The walk of one chunk: the bit offset of each of its first nblk blocks
-// that is not all zero into offs, and its cost class (1 + 16 min(events, 14)
-// + min(members, 15): the trip counts of the decode's two loops) into cls;
-// both arrays come zeroed, and class 0 marks an all-zero block.  Every
-// iteration consumes one token: a run of all-zero blocks, a block's head, or
-// one event of its significance section (failed group tests, the successful
-// one, the scan, the coefficient found).  Every member of the prefix
-// carries w bits and a sign, w the plane above kmin of the next coefficient
-// found, so the refinement section is skipped in one step with the token
-// that ends the significance section.  The lanes of a warp, each on its own
-// chunk, move one token per iteration whatever their blocks look like, and
-// a warp takes as many iterations as its longest chunk has tokens.  Returns
-// false on a malformed chunk.
+// The walk of one chunk: the bit offset of each of its first nblk blocks that
+// is not all zero into offs, and its cost class (1 + 16 min(events, 14) +
+// min(members, 15): the trip counts of the decode's two loops) into cls; both
+// arrays come zeroed, and class 0 marks an all-zero block.  Per trip of the
+// outer loop a lane skips a run of all-zero blocks and walks one block, event
+// by event (failed group tests, the successful one, the scan, the coefficient
+// found), so that the lanes of a warp, whose chunks are of similar size, run
+// the short event loop together; one token of any kind per trip made every
+// trip run the code of all kinds (96 instructions a token).  Every member of
+// the prefix carries w bits and a sign, w the plane above kmin of the next
+// coefficient found, so the refinement section is skipped in one step.
+// Returns false on a malformed chunk.
 template <bool LL>
 __device__ bool walk_chunk(GReader &rd, u32 nblk, const unsigned char *ktab, unsigned short *offs,
                            unsigned char *cls) {
   constexpr int Ktop = LL ? 32 : 30;
-  int phase = 0;  // 0 a block's head, 1 an event, 3 a scan past the window
-  int k = 0, kmin = 0, n = 0, g = 0, ne = 0;
-  u32 blk = 0, refine = 0;
-  bool ok = true;
-  while (blk < nblk && ok) {
-    const u32 v = rd.peek();
-    u32 adv = 0;
-    bool event = false;  // an event ends in this token: coefficient n + g at plane k
-    bool done = false;   // the significance section ends with this token
-    if (phase == 0) {
-      if (!(v & 1u)) {  // a run of all-zero blocks (one flag bit each)
-        adv = (u32)min(v ? __ffs(v) - 1 : 32, (int)(nblk - blk));
-        blk += adv;
-      } else {
-        offs[blk] = (unsigned short)rd.pos;  // < 2^16: a chunk holds at most 640 words
-        if (LL) {
-          adv = 1;
-        } else {
-          const int eb = (int)((v >> 1) & 511u);
-          ok = eb < kTab;
-          kmin = ok ? ktab[eb] : 0;
-          adv = 10;
-        }
-        phase = 1;
-        k = Ktop;
-        n = 0;
-        ne = 0;
-        refine = 0;
+  u32 blk = 0;
+  while (true) {
+    while (true) {  // all-zero blocks, one flag bit each
+      const u32 v = rd.peek();
+      const int run = min(v ? __ffs(v) - 1 : 32, (int)(nblk - blk));
+      blk += (u32)run;
+      if (run < 32 || blk >= nblk) {
+        rd.skip(run);
+        break;
       }
-    } else if (phase == 1) {
+      rd.skip(32);
+    }
+    if (blk >= nblk) return true;
+    offs[blk] = (unsigned short)rd.pos;  // < 2^16: a chunk holds at most 640 words
+    int kmin = 0;
+    if (LL) {
+      rd.skip(1);
+    } else {
+      const int eb = (int)((rd.peek() >> 1) & 511u);
+      if (eb >= kTab) return false;
+      kmin = ktab[eb];
+      rd.skip(10);
+    }
+    int k = Ktop, n = 0, ne = 0;
+    u32 refine = 0;
+    while (n < 16) {
+      const u32 v = rd.peek();
       const int lim = k - kmin + 1;
       const int z = v ? __ffs(v) - 1 : 32;
-      if (z >= lim) {  // every remaining plane fails
-        adv = (u32)lim;
-        done = true;
-      } else if (z == 32) {  // (lossless) 32 failed tests, planes left
-        adv = 32;
-        k -= 32;
-      } else {
-        k -= z;
+      int g;
+      if (z < lim && z < 32) {
         const u32 v2 = z < 31 ? v >> (z + 1) : 0u;  // 31 - z valid bits
         g = v2 ? __ffs(v2) - 1 : 32;
         if (g < 31 - z) {
-          adv = (u32)(z + g + 2);
-          event = true;
+          rd.skip(z + g + 2);
         } else {  // the scan goes on past the window
-          adv = 32;
-          g = 31 - z;
-          phase = 3;
+          rd.skip(z + 1);
+          g = zeros(rd, 16 - n);
+          if (g < 16 - n) rd.skip(1);
         }
-        ok = g < 16 - n;
+        k -= z;
+      } else {
+        if (z >= lim) {  // every remaining plane fails
+          rd.skip(lim);
+          break;
+        }
+        rd.skip(32);  // (lossless) 32 failed tests, planes left
+        k -= 32;
+        continue;
       }
-    } else {
-      const int zz = v ? __ffs(v) - 1 : 32;
-      g += zz;
-      ok = zz < 32 && g < 16 - n;
-      adv = (u32)(zz + 1);
-      event = true;
-      phase = 1;
-    }
-    if (event && ok) {  // members n .. n + g enter the prefix at plane k
+      if (g >= 16 - n) return false;
+      // members n .. n + g enter the prefix at plane k
       refine += (u32)(g + 1) * (u32)(k - kmin + 1);
       n += g + 1;
       ++ne;
-      done = n == 16;
     }
-    if (done && ok) {
-      cls[blk] = (unsigned char)(1 + min(ne, 14) * 16 + min(n, 15));
-      adv += refine;
-      phase = 0;
-      ++blk;
-    }
-    rd.advance(adv);
+    cls[blk] = (unsigned char)(1 + min(ne, 14) * 16 + min(n, 15));
+    ++blk;
+    rd.advance(refine);
   }
-  return ok;
 }
 
 // Decode one block into x (the decode).  Returns false on a malformed block.
 template <bool LL, class R>
 __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
-                                             unsigned char *sfx, int *qs, int sstride,
+                                             unsigned char *sfx, int sstride, int *qs,
                                              float (&x)[16]) {
   if (!getbits(rd, 1)) {
 #pragma unroll
@@ -781,17 +769,15 @@ __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
   // refinement: magnitudes and signs, in coding order, each at the midpoint
   // of its kept interval.  Fixed accuracy takes a rolled loop over the
   // members (one trip per member, so lanes with as many members stay in
-  // step), the coefficients through this thread's shared-memory slots qs[j *
-  // sstride], j in block order; lossless keeps the unrolled register form
-  // (its 64-bit slots would cost occupancy).
+  // step), the coefficients through the block's place in the window's shared
+  // memory, qs[(j / 4) kOutPitch + j % 4], j in block order (it comes zeroed);
+  // lossless keeps the unrolled register form (64-bit coefficients).
   using S = typename std::conditional<LL, long long, int>::type;
   S q[16];
   long long qw[16];
   const u64 half = kmin > 0 ? (1ull << (kmin - 1)) : 0ull;
   const int n = found ? 32 - __clz(found) : 0;  // members: up to the last coefficient found
   if constexpr (!LL) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) qs[j * sstride] = 0;
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int w = sfx[(i + __ffs(found >> i) - 1) * sstride] - kmin;  // 0 .. 30
@@ -800,13 +786,19 @@ __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
       if ((found >> i) & 1u) t |= 1ull << w;
       if (t) {
         const long long v = (long long)((t << kmin) + half);
-        qs[perm_rt(i) * sstride] = (int)((fs >> w) ? -v : v);
+        const int j = perm_rt(i);
+        qs[(j >> 2) * kOutPitch + (j & 3)] = (int)((fs >> w) ? -v : v);
       }
     }
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      q[j] = (S)qs[j * sstride];
-      qw[j] = (long long)qs[j * sstride];
+    for (int r = 0; r < 4; ++r) {
+      const int4 t = *reinterpret_cast<const int4 *>(qs + r * kOutPitch);
+      const int u[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {
+        q[4 * r + l] = (S)u[l];
+        qw[4 * r + l] = (long long)u[l];
+      }
     }
   } else {
 #pragma unroll
@@ -925,9 +917,9 @@ __device__ __forceinline__ int walk_key(u32 nw) {
 // shared memory), so that a warp walks chunks of similar length: the walk
 // moves one token per iteration and a warp takes as many iterations as its
 // longest chunk.  The bit offsets and cost classes of the blocks stay in
-// shared memory; the CTA then writes the segment's list (its blocks that are
-// not all zero, ordered by class with a second counting sort) and its count,
-// and writes the all-zero blocks to the output.  One kernel per mode; each
+// shared memory; the CTA then writes its windows' lists (the blocks that are
+// not all zero, ordered by class with a second counting sort per window) and
+// their counts.  One kernel per mode; each
 // skips the other mode's streams, and the fixed-accuracy one reports bad
 // headers.
 template <bool LL>
@@ -935,16 +927,14 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
   __shared__ unsigned short s_offs[kWalk][kChunk + 1];
   __shared__ unsigned char s_cls[kWalk][kChunk + 4];
   __shared__ unsigned char s_kmin[kTab];
-  __shared__ int s_cnt[kClasses];
+  __shared__ int s_cnt[kSegWins * kClasses];
   __shared__ unsigned short s_order[kWalk];
-  __shared__ int s_wsum[kWalk / 32];
-  __shared__ u32 s_nnz;
   __shared__ int s_ok;
   const u32 arr = blockIdx.y;
   const int tid = threadIdx.x;
   const unsigned char *slot = a.in + (u64)arr * a.stride;
   if (tid == 0) s_ok = header_ok(a, slot);
-  for (int i = tid; i < kClasses; i += kWalk) s_cnt[i] = 0;
+  for (int i = tid; i < kSegWins * kClasses; i += kWalk) s_cnt[i] = 0;
   for (int i = tid; i < kTab; i += kWalk) s_kmin[i] = a.kmin[arr * kTab + i];
   __syncthreads();
   if (!s_ok) {
@@ -977,7 +967,7 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
     __syncthreads();
     s_order[s_cnt[key] + rank] = (unsigned short)tid;
     __syncthreads();
-    for (int i = tid; i < kClasses; i += kWalk) s_cnt[i] = 0;  // (now the class histogram)
+    for (int i = tid; i < kWalkKeys; i += kWalk) s_cnt[i] = 0;  // (now the class histograms)
   }
   const int r = s_order[tid];  // the chunk this thread walks
   bool bad = false;
@@ -999,22 +989,24 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
     bad = !ok;
   }
   __syncthreads();
-  // the segment's list: its blocks that are not all zero, in class order,
-  // each entry the block's index in the segment (13 bits) over its bit
+  // the windows' lists: their blocks that are not all zero, in class order,
+  // each entry the block's index in the segment (12 bits) over its bit
   // offset in its chunk (15 bits: a chunk holds at most 640 words)
   const u32 B0 = c0 * kChunk, nblocks = min(rows * kChunk, a.nb - B0);
   for (u32 i = tid; i < nblocks; i += kWalk) {
     const unsigned q = s_cls[i >> 5][i & 31];
-    if (q) atomicAdd(&s_cnt[q], 1);
+    if (q) atomicAdd(&s_cnt[i / kWin * kClasses + q], 1);
   }
   __syncthreads();
-  {  // exclusive scan of the class counts, kPerT consecutive ones per thread
-    constexpr int kPerT = kClasses / kWalk;
-    const int lane = tid & 31, warp = tid >> 5;
+  const u64 seg = (u64)arr * a.nseg + blockIdx.x;
+  {  // exclusive scan of each window's class counts, a warp per window
+    constexpr int kPerT = kClasses / 32;
+    const int lane = tid & 31, w = tid >> 5;
+    int *cnt = s_cnt + w * kClasses + lane * kPerT;
     int x[kPerT], sum = 0;
 #pragma unroll
     for (int j = 0; j < kPerT; ++j) {
-      x[j] = s_cnt[tid * kPerT + j];
+      x[j] = cnt[j];
       sum += x[j];
     }
     int inc = sum;
@@ -1023,107 +1015,87 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
       const int y = __shfl_up_sync(0xffffffffu, inc, d);
       if (lane >= d) inc += y;
     }
-    if (lane == 31) s_wsum[warp] = inc;
-    __syncthreads();
     int run = inc - sum;
 #pragma unroll
-    for (int w = 0; w < kWalk / 32; ++w) run += w < warp ? s_wsum[w] : 0;
-#pragma unroll
     for (int j = 0; j < kPerT; ++j) {
-      s_cnt[tid * kPerT + j] = run;
+      cnt[j] = run;
       run += x[j];
     }
-    if (tid == kWalk - 1) s_nnz = (u32)run;
+    if (lane == 31) a.wincount[seg * kSegWins + w] = (u32)run;
   }
   __syncthreads();
-  const u64 seg = (u64)arr * a.nseg + blockIdx.x;
   u32 *list = a.list + seg * kSeg;
   for (u32 i = tid; i < nblocks; i += kWalk) {
     const unsigned q = s_cls[i >> 5][i & 31];
-    if (q) list[atomicAdd(&s_cnt[q], 1)] = (i << 15) | s_offs[i >> 5][i & 31];
-  }
-  if (tid == 0) a.segcount[seg] = s_nnz;
-  // the segment's all-zero blocks to the output, row by row: a warp per row,
-  // 32 consecutive floats per store
-  {
-    const u32 B1 = B0 + nblocks, bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
-    const u32 r1 = min(4 * bi1 + 4, (u32)a.n0), lane = tid & 31;
-    for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kWalk / 32) {
-      const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
-      const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
-      const u32 j1 = min(4 * (hi - rb), (u32)a.n1);
-      float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
-      for (u32 j = 4 * (lo - rb) + lane; j < j1; j += 32) {
-        const u32 l = rb + (j >> 2) - B0;  // the block's index in the segment
-        if (s_cls[l >> 5][l & 31] == 0) row[j] = 0.0f;
-      }
-    }
+    const u32 w = i / kWin;
+    if (q) list[w * kWin + atomicAdd(&s_cnt[w * kClasses + q], 1)] = (i << 15) | s_offs[i >> 5][i & 31];
   }
   if (bad) report_bad(a, arr);
 }
 
-// The 4 x 4 block b of array arr to the output (edge blocks clipped).
-__device__ __forceinline__ void store_block(const DecArgs &a, u32 arr, u32 b, const float (&x)[16]) {
-  const u32 bi = b / a.nb1, bj = b - bi * a.nb1;
-  float *p0 = a.out + ((long long)arr * a.n0 + 4ll * bi) * a.n1 + 4ll * bj;
-  if (4ll * bi + 3 < a.n0 && 4ll * bj + 3 < a.n1) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) p0[cc] = x[4 * r + cc];
-      p0 += a.n1;
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (4ll * bi + r < a.n0) {
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc)
-          if (4ll * bj + cc < a.n1) p0[cc] = x[4 * r + cc];
-      }
-      p0 += a.n1;
-    }
-  }
-}
-
-// Pass 2: decode the listed blocks of one mode, a CTA per segment (a
-// grid-stride loop over one resident wave of CTAs), a thread per entry in
-// list order, so that the lanes of a warp hold blocks of one class and run
-// the decode's loops for as many trips.  Each thread reads its block's bits
-// from global memory, bounded by its chunk.
+// Pass 2: decode the windows of one mode, a CTA per window (a grid-stride
+// loop over one resident wave of CTAs), a thread per list entry, so that the
+// lanes of a warp hold blocks of one class and run the decode's loops for as
+// many trips.  Each thread reads its block's bits from global memory, bounded
+// by its chunk, and leaves its 4 x 4 values in the window's shared memory; the
+// CTA then writes the window's rows, 32 consecutive floats a store (blocks
+// stored one by one in class order wrote half sectors, which cost the 64
+// images of 351 x 1701 490 MB of reads and 317 of writes for 76 and 153).
 template <bool LL>
-__global__ void __launch_bounds__(kDec) k_cz_decode(const __grid_constant__ DecArgs a) {
+__global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ DecArgs a) {
+  extern __shared__ __align__(16) float s_out[];  // [4][kOutPitch]: block l at columns 4 l .. 4 l + 3
   __shared__ unsigned char s_sfx[16][kDec];
-  __shared__ int s_q[LL ? 1 : 16][kDec];  // coefficient slots (fixed accuracy)
-  __shared__ u32 s_n;
-  const int tid = threadIdx.x;
-  const u64 nseg = (u64)a.count * a.nseg;
-  for (u64 seg = blockIdx.x; seg < nseg; seg += gridDim.x) {
-    const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg);
+  __shared__ int s_n;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const u64 nwin = (u64)a.count * a.nseg * kSegWins;
+  for (u64 win = blockIdx.x; win < nwin; win += gridDim.x) {
+    const u64 seg = win / kSegWins;
+    const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg), w = (u32)(win % kSegWins);
+    const u32 B0 = sj * kSeg + w * kWin;  // first block of the window
     const unsigned char *slot = a.in + (u64)arr * a.stride;
     if (tid == 0)
-      s_n = header_ok(a, slot) && (reinterpret_cast<const u32 *>(slot)[2] != 0) == LL
-                ? a.segcount[seg]
-                : 0u;
+      s_n = B0 < a.nb && header_ok(a, slot) && (reinterpret_cast<const u32 *>(slot)[2] != 0) == LL
+                ? (int)a.wincount[win]
+                : -1;
+    for (int i = tid; i < kOutPitch; i += kDec)
+      reinterpret_cast<float4 *>(s_out)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
-    const u32 n = s_n;
-    const u32 *list = a.list + seg * kSeg;
-    const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
-    for (u32 p = tid; p < n; p += kDec) {
-      const u32 e = list[p];
-      const u32 b = sj * kSeg + (e >> 15);
-      u32 start, next;
-      if (!chunk_words(a, slot, b / kChunk, start, next)) continue;  // (reported by the walk)
-      GReader rd;
-      rd.init_at(words + start, next - start, e & 0x7fffu);
-      float x[16];
-      const bool ok = decode_block<LL>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid],
-                                       &s_q[0][tid], kDec, x) &&
-                      !rd.overrun();
-      if (!ok) report_bad(a, arr);
-      store_block(a, arr, b, x);
+    const int n = s_n;
+    if (n >= 0) {
+      const u32 *list = a.list + seg * kSeg + w * kWin;
+      const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
+      for (int p = tid; p < n; p += kDec) {
+        const u32 e = list[p];
+        const u32 b = sj * kSeg + (e >> 15);
+        u32 start, next;
+        if (!chunk_words(a, slot, b / kChunk, start, next)) continue;  // (reported by the walk)
+        GReader rd;
+        rd.init_at(words + start, next - start, e & 0x7fffu);
+        float x[16];
+        float *place = s_out + 4 * (b - B0);
+        const bool ok = decode_block<LL>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid], kDec,
+                                         reinterpret_cast<int *>(place), x) &&
+                        !rd.overrun();
+        if (!ok) report_bad(a, arr);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          *reinterpret_cast<float4 *>(place + r * kOutPitch) =
+              make_float4(x[4 * r], x[4 * r + 1], x[4 * r + 2], x[4 * r + 3]);
+      }
+      __syncthreads();
+      // rows of the window, a warp per row (edge blocks clipped)
+      const u32 B1 = min(B0 + kWin, a.nb), bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
+      const u32 r1 = min(4 * bi1 + 4, (u32)a.n0);
+      for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kDec / 32) {
+        const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
+        const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
+        const u32 j0 = 4 * (lo - rb), j1 = min(4 * (hi - rb), (u32)a.n1);
+        float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
+        const float *src = s_out + (i & 3) * kOutPitch + 4 * (lo - B0);
+        for (u32 j = j0 + lane; j < j1; j += 32) row[j] = src[j - j0];
+      }
     }
-    __syncthreads();  // (s_n is set again for the next segment)
+    __syncthreads();  // (the window's memory is cleared for the next one)
   }
 }
 
@@ -1216,7 +1188,7 @@ u64 codec_decode_scratch_bytes(long long count, long long n0, long long n1) {
   long long nchunk = 0;
   if (!codec_shape(n0, n1, nullptr, nullptr, &nchunk, nullptr, nullptr)) return 0;
   const u64 nseg = (u64)((nchunk + kWalk - 1) / kWalk), G = (u64)decode_group(count, nchunk);
-  return 16 + ((u64)count * kTab + 15) / 16 * 16 + (4 * G * nseg + 15) / 16 * 16 +
+  return 16 + ((u64)count * kTab + 15) / 16 * 16 + (4 * G * nseg * kSegWins + 15) / 16 * 16 +
          4ull * kSeg * G * nseg;
 }
 
@@ -1232,10 +1204,15 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
   int dev = 0, nsm = 0, per_sm[2] = {0, 0};
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  constexpr int kSmem = 4 * kOutPitch * (int)sizeof(float);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_cz_decode<false>, kDec, 0);
+    e = cudaFuncSetAttribute(k_cz_decode<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_cz_decode<true>, kDec, 0);
+    e = cudaFuncSetAttribute(k_cz_decode<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_cz_decode<false>, kDec, kSmem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_cz_decode<true>, kDec, kSmem);
   if (e != cudaSuccess) return e;
   a.nb1 = (u32)nb1;
   a.nb = (u32)nb;
@@ -1247,8 +1224,8 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
   a.err = reinterpret_cast<int *>(scratch);
   unsigned char *tab = scratch + 16, *p = tab + ((u64)count * kTab + 15) / 16 * 16;
   const long long G = decode_group(count, nchunk);
-  a.segcount = reinterpret_cast<u32 *>(p);
-  a.list = reinterpret_cast<u32 *>(p + (4ull * G * a.nseg + 15) / 16 * 16);
+  a.wincount = reinterpret_cast<u32 *>(p);
+  a.list = reinterpret_cast<u32 *>(p + (4ull * G * a.nseg * kSegWins + 15) / 16 * 16);
   k_cz_kmin<<<(unsigned)count, kTab, 0, st>>>(in, stride, 0.0, tab);
   for (long long g0 = 0; g0 < count; g0 += G) {
     const long long g = std::min(G, count - g0);
@@ -1258,14 +1235,14 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
     a.out = out + (u64)g0 * (u64)n0 * (u64)n1;
     a.kmin = tab + (u64)g0 * kTab;
     const dim3 gwalk(a.nseg, (unsigned)g);
-    // the decode loops over the group's segments with one resident wave of CTAs
-    const u64 nseg = (u64)g * a.nseg;
-    const unsigned gd0 = (unsigned)std::min<u64>(nseg, (u64)std::max(1, per_sm[0]) * nsm);
-    const unsigned gd1 = (unsigned)std::min<u64>(nseg, (u64)std::max(1, per_sm[1]) * nsm);
+    // the decode loops over the group's windows with one resident wave of CTAs
+    const u64 nwin = (u64)g * a.nseg * kSegWins;
+    const unsigned gd0 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[0]) * nsm);
+    const unsigned gd1 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[1]) * nsm);
     k_cz_walk<false><<<gwalk, kWalk, 0, st>>>(a);
     k_cz_walk<true><<<gwalk, kWalk, 0, st>>>(a);
-    k_cz_decode<false><<<gd0, kDec, 0, st>>>(a);
-    k_cz_decode<true><<<gd1, kDec, 0, st>>>(a);
+    k_cz_decode<false><<<gd0, kDec, kSmem, st>>>(a);
+    k_cz_decode<true><<<gd1, kDec, kSmem, st>>>(a);
   }
   return cudaGetLastError();
 }
