@@ -316,10 +316,9 @@ int check_velocity(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d, long lo
                    cudaStream_t st) {
   DevBuf r;
   CU(r.alloc(ctx, 16, st));
-  // pageable copies: the H2D is staged before the call returns and the D2H
-  // completes before it returns, so stack arrays are safe here
-  const unsigned init[4] = {0u, 0x7f7fffffu, 0u, 0u};
-  CU(cudaMemcpyAsync(r.p, init, 16, cudaMemcpyHostToDevice, st));
+  // (the smallest value, which starts above all, is not used here; a pageable
+  // D2H copy completes before it returns, so the stack array is safe)
+  CU(cudaMemsetAsync(r.p, 0, 16, st));
   CU(launch_vrange(vel_d, n, r.as<unsigned>(), st));
   unsigned out[4];
   CU(cudaMemcpyAsync(out, r.p, 16, cudaMemcpyDeviceToHost, st));
@@ -448,11 +447,35 @@ struct Common {
   int l2_ahead = 0;  // RunConfig::l2_ahead of the call
   int pdl = 0;       // RunConfig::pdl of the call
   long long n_rent = 0, n_rext = 0, n_rcen = 0;  // receiver-table entries (debug index checks)
-  DevBuf c_all, gx, gz, src_rc, rptr, rent, rext_ptr, rext_ent, rcen_ptr, rcen_ent, wav, items, err;
+  DevBuf c_all, tables;
+  // the call's small tables, all in `tables`: sponge factors, source rows and
+  // columns, the receivers of the single-step and the two-step tiles, the wavelet,
+  // the items' samples and shots, the device flag, and the receivers sorted by
+  // row and strip (phases with the grid on chip)
+  const float *gx = nullptr, *gz = nullptr, *wav = nullptr;
+  const int *src_rc = nullptr, *rptr = nullptr, *rext_ptr = nullptr, *rcen_ptr = nullptr,
+            *items = nullptr;
+  const int2 *rent = nullptr, *rext_ent = nullptr, *rcen_ent = nullptr, *res_ent = nullptr;
+  int *err = nullptr;
   CUtensorMap mc;
-  ResPlan res;       // phases with the grid on chip (C = 0: not)
-  DevBuf res_ent;    // ... and their receivers, sorted by row and strip
+  ResPlan res;  // phases with the grid on chip (C = 0: not)
   int res_max_ent = 0;
+};
+
+// Host tables packed for one upload: a pageable copy synchronises its stream
+// before it starts, so one copy per table cost a small call most of its set-up.
+struct TablePack {
+  std::vector<unsigned char> h;
+  size_t add(const void *p, size_t bytes) {
+    const size_t o = (h.size() + 255) / 256 * 256;
+    h.resize(o + std::max<size_t>(bytes, 16), 0);
+    if (bytes) std::memcpy(h.data() + o, p, bytes);
+    return o;
+  }
+  template <class T>
+  size_t add(const std::vector<T> &v) {
+    return add(v.data(), v.size() * sizeof(T));
+  }
 };
 
 static double tile_step_us(double n, int tile_z);
@@ -543,23 +566,17 @@ static RunConfig resolve_config(RunConfig c, const Geo &g, int B) {
   return c;
 }
 
-// Chooses the resident form for B items in flight and uploads its receiver table.
-static int setup_resident(rtm_ctx *ctx, Common &C, const rtm_acq &acq, int B, cudaStream_t st) {
+// Chooses the resident form for B items in flight; ent: its receiver table.
+static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<int2> &ent) {
   const Geo &g = C.g;
   const int NS = (g.X0 + g.NX + 3) / 4;
-  std::vector<int2> ent(acq.nrec);
+  ent.resize(acq.nrec);
   for (int r = 0; r < acq.nrec; ++r) {
     const int row = acq.rec_iz[r] + g.nb, col = acq.rec_ix[r] + g.CP;
     ent[r] = make_int2(row * NS + col / 4, 4 * r + col % 4);
   }
   std::stable_sort(ent.begin(), ent.end(), [](const int2 &a, const int2 &b) { return a.x < b.x; });
   C.res = resident_plan(g, B, ent, &C.res_max_ent);
-  if (!C.res.C) return RTM_OK;
-  if (ent.empty()) ent.push_back(make_int2(0x7fffffff, 0));
-  CU(C.res_ent.alloc(ctx, ent.size() * sizeof(int2), st));
-  // (a pageable copy is staged before the call returns)
-  CU(cudaMemcpyAsync(C.res_ent.p, ent.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-  return RTM_OK;
 }
 
 // Receiver lists of the two-step tiles: every tile whose extended region
@@ -597,9 +614,11 @@ static void step2_receiver_lists(const Geo &g, const rtm_acq &acq, std::vector<i
   if (cent.empty()) cent.push_back(make_int2(0, 0));
 }
 
-// Upload the per-call tables shared by all items.
+// Choose the resident form, upload the per-call tables (one copy) and make c.
+// items: the items' samples, then their shots.
 static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_acq &acq,
-                        int nsample, const float *vel_d, cudaStream_t st, const RunConfig &cfg) {
+                        int nsample, const float *vel_d, cudaStream_t st, const RunConfig &cfg,
+                        int B, const std::vector<int> &items) {
   const int step_kernel = cfg.step_kernel;
   C.g = make_geo(gr, step_kernel >= 3 ? cfg.tile_z : 24);
   C.kernel = step_kernel;
@@ -608,6 +627,9 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
   C.k = make_coef(gr);
   C.nsample = nsample;
   const Geo &g = C.g;
+  std::vector<int2> res_ent;
+  if (cfg.resident) choose_resident(C, acq, B, res_ent);
+  const bool res = C.res.C > 0;
   std::vector<float> gz, gx;
   sponge_tables(g, gx, gz);
   // sources: memory (row, col); receivers: CSR over single-step tiles
@@ -616,49 +638,46 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
     src[s] = acq.src_iz[s] + g.nb;
     src[acq.nshot + s] = acq.src_ix[s] + g.CP;
   }
-  std::vector<int> rptr;
-  std::vector<int2> rent;
-  receiver_tiles(g, acq, rptr, rent);
-  std::vector<int> eptr, cptr;
-  std::vector<int2> eent, cent;
-  step2_receiver_lists(g, acq, eptr, eent, cptr, cent);
+  std::vector<int> rptr, eptr, cptr;
+  std::vector<int2> rent, eent, cent;
+  if (!res) {
+    receiver_tiles(g, acq, rptr, rent);
+    step2_receiver_lists(g, acq, eptr, eent, cptr, cent);
+  }
   C.n_rent = (long long)rent.size();
   C.n_rext = (long long)eent.size();
   C.n_rcen = (long long)cent.size();
+  TablePack t;
+  const size_t o_gx = t.add(gx), o_gz = t.add(gz), o_src = t.add(src), o_rptr = t.add(rptr),
+               o_rent = t.add(rent), o_eptr = t.add(eptr), o_eent = t.add(eent),
+               o_cptr = t.add(cptr), o_cent = t.add(cent),
+               o_wav = t.add(acq.wavelet, (size_t)gr.nt * 4), o_items = t.add(items),
+               o_res = t.add(res_ent), o_err = t.add(nullptr, 0);
   CU(C.c_all.alloc(ctx, (size_t)nsample * g.plane * 4, st));
-  CU(C.gx.alloc(ctx, gx.size() * 4, st));
-  CU(C.gz.alloc(ctx, gz.size() * 4, st));
-  CU(C.src_rc.alloc(ctx, src.size() * 4, st));
-  CU(C.rptr.alloc(ctx, rptr.size() * 4, st));
-  CU(C.rent.alloc(ctx, rent.size() * sizeof(int2), st));
-  CU(C.rext_ptr.alloc(ctx, eptr.size() * 4, st));
-  CU(C.rext_ent.alloc(ctx, eent.size() * sizeof(int2), st));
-  CU(C.rcen_ptr.alloc(ctx, cptr.size() * 4, st));
-  CU(C.rcen_ent.alloc(ctx, cent.size() * sizeof(int2), st));
-  CU(C.wav.alloc(ctx, (size_t)gr.nt * 4, st));
-  CU(C.err.alloc(ctx, 16, st));
-  CU(cudaMemcpyAsync(C.gx.p, gx.data(), gx.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.gz.p, gz.data(), gz.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.src_rc.p, src.data(), src.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.rptr.p, rptr.data(), rptr.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.rent.p, rent.data(), rent.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                     st));
-  CU(cudaMemcpyAsync(C.rext_ptr.p, eptr.data(), eptr.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.rext_ent.p, eent.data(), eent.size() * sizeof(int2),
-                     cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.rcen_ptr.p, cptr.data(), cptr.size() * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.rcen_ent.p, cent.data(), cent.size() * sizeof(int2),
-                     cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(C.wav.p, acq.wavelet, (size_t)gr.nt * 4, cudaMemcpyHostToDevice, st));
-  CU(cudaMemsetAsync(C.err.p, 0, 16, st));
+  CU(C.tables.alloc(ctx, t.h.size(), st));
+  CU(cudaMemcpyAsync(C.tables.p, t.h.data(), t.h.size(), cudaMemcpyHostToDevice, st));
+  unsigned char *base = C.tables.as<unsigned char>();
+  C.gx = reinterpret_cast<float *>(base + o_gx);
+  C.gz = reinterpret_cast<float *>(base + o_gz);
+  C.src_rc = reinterpret_cast<int *>(base + o_src);
+  C.rptr = reinterpret_cast<int *>(base + o_rptr);
+  C.rent = reinterpret_cast<int2 *>(base + o_rent);
+  C.rext_ptr = reinterpret_cast<int *>(base + o_eptr);
+  C.rext_ent = reinterpret_cast<int2 *>(base + o_eent);
+  C.rcen_ptr = reinterpret_cast<int *>(base + o_cptr);
+  C.rcen_ent = reinterpret_cast<int2 *>(base + o_cent);
+  C.wav = reinterpret_cast<float *>(base + o_wav);
+  C.items = reinterpret_cast<int *>(base + o_items);
+  C.res_ent = reinterpret_cast<int2 *>(base + o_res);
+  C.err = reinterpret_cast<int *>(base + o_err);
   CU(launch_prep_c(vel_d, C.c_all.as<float>(), g, gr.dt, nsample, st));
-  if (step_kernel >= 2) {
+  if (step_kernel >= 2 && !res) {
     const int H = step2_ext();
     int rc = make_map(ctx, &C.mc, C.c_all.as<float>(), g, nsample, step2_tile_x() + 2 * H,
                       g.tz2 + 2 * H);
     if (rc) return rc;
   }
-  // the host vectors above go out of scope: make the copies complete first
+  // the packed tables go out of scope: make their copy complete first
   CU(cudaStreamSynchronize(st));
   return RTM_OK;
 }
@@ -704,18 +723,18 @@ static void fill_args(StepArgs &A, const Common &C, const rtm_grid &gr, const rt
   std::memset(&A, 0, sizeof(A));
   A.g = C.g;
   A.k = C.k;
-  A.gx = C.gx.as<float>();
-  A.gz = C.gz.as<float>();
+  A.gx = C.gx;
+  A.gz = C.gz;
   A.c_all = C.c_all.as<float>();
-  A.src_row = C.src_rc.as<int>();
-  A.src_col = C.src_rc.as<int>() + acq.nshot;
-  A.wav = C.wav.as<float>();
+  A.src_row = C.src_rc;
+  A.src_col = C.src_rc + acq.nshot;
+  A.wav = C.wav;
   A.src_scale = (float)(1.0 / (gr.dx * gr.dz));
-  A.rtile_ptr = C.rptr.as<int>();
-  A.rtile_ent = C.rent.as<int2>();
+  A.rtile_ptr = C.rptr;
+  A.rtile_ent = C.rent;
   A.nrec = acq.nrec;
   A.nt = gr.nt;
-  A.err = C.err.as<int>();
+  A.err = C.err;
   A.len.nshot = acq.nshot;
   A.len.nsample = C.nsample;
   A.len.rent = C.n_rent;
@@ -736,10 +755,10 @@ static void fill_args2(Step2Args &A2, const StepArgs &A, const Common &C) {
   A2.src_col = A.src_col;
   A2.wav = A.wav;
   A2.src_scale = A.src_scale;
-  A2.rext_ptr = C.rext_ptr.as<int>();
-  A2.rext_ent = C.rext_ent.as<int2>();
-  A2.rcen_ptr = C.rcen_ptr.as<int>();
-  A2.rcen_ent = C.rcen_ent.as<int2>();
+  A2.rext_ptr = C.rext_ptr;
+  A2.rext_ent = C.rext_ent;
+  A2.rcen_ptr = C.rcen_ptr;
+  A2.rcen_ent = C.rcen_ent;
   A2.nrec = A.nrec;
   A2.nt = A.nt;
   A2.seis = A.seis;
@@ -751,7 +770,7 @@ static void fill_args2(Step2Args &A2, const StepArgs &A, const Common &C) {
   A2.num = A.num;
   A2.den = A.den;
   A2.dmax = A.dmax;
-  A2.err = C.err.as<int>();
+  A2.err = C.err;
   A2.refl = A.refl;
   A2.len = A.len;
   A2.len.rent = C.n_rext;
@@ -770,7 +789,7 @@ static void fill_args_res(ResArgs &R, const StepArgs &A, const Common &C) {
   R.src_col = A.src_col;
   R.wav = A.wav;
   R.src_scale = A.src_scale;
-  R.ent = C.res_ent.as<int2>();
+  R.ent = C.res_ent;
   R.nent = A.nrec;
   R.max_ent = C.res_max_ent;
   R.nrec = A.nrec;
@@ -795,7 +814,7 @@ static int maybe_inject_timeout(rtm_ctx *ctx, const Common &C, cudaStream_t st) 
   while (n > 0 && !ctx->inject_timeouts.compare_exchange_weak(n, n - 1)) {
   }
   static const int kRaised = 1;  // (a pageable copy is staged before the call returns)
-  if (n > 0) CU(cudaMemcpyAsync(C.err.p, &kRaised, 4, cudaMemcpyHostToDevice, st));
+  if (n > 0) CU(cudaMemcpyAsync(C.err, &kRaised, 4, cudaMemcpyHostToDevice, st));
   return RTM_OK;
 }
 
@@ -884,25 +903,22 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   if (B > nitems) B = (int)nitems;
   if (B < 1) B = 1;
   const RunConfig cfg = resolve_config(wanted, make_geo(gr), B);
-  {
-    PhaseRange ph("setup");
-    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg);
-  }
-  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
-  if (!rc && cfg.resident) rc = setup_resident(ctx, C, acq, B, st);
-  if (rc) return rc;
-  trace_mark("tables and model set up");
-  const Geo &g = C.g;
-  const bool res = C.res.C > 0;
-  const int nsnap = gr.nt / op.isnap;
   // items in (sample, shot) order
   std::vector<int> items(2 * nitems);
   for (long long q = 0; q < nitems; ++q) {
     items[q] = (int)(q / acq.nshot);
     items[nitems + q] = (int)(q % acq.nshot);
   }
-  CU(C.items.alloc(ctx, items.size() * 4, st));
-  CU(cudaMemcpyAsync(C.items.p, items.data(), items.size() * 4, cudaMemcpyHostToDevice, st));
+  {
+    PhaseRange ph("setup");
+    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg, B, items);
+  }
+  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
+  if (rc) return rc;
+  trace_mark("tables and model set up");
+  const Geo &g = C.g;
+  const bool res = C.res.C > 0;
+  const int nsnap = gr.nt / op.isnap;
   const size_t esz = snap_elem_bytes(op.snap_dtype);
   // checkpoint mode: the state every cpC steps instead of every snapshot;
   // each segment's snapshots are recomputed into a ring of `ring` slots
@@ -910,7 +926,9 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   const int nseg = cpC ? (gr.nt + cpC - 1) / cpC : 0;
   const int ring = cpC ? cpC / op.isnap + 1 : nsnap;
   Fields F, U;  // F: forward fields, then the receiver wavefield; U: recomputed forward
-  if ((rc = alloc_fields(ctx, F, g, B, st, cfg.step_kernel))) return rc;
+  // (phases with the grid on chip need fields only to hand states over)
+  const bool need_fields = !res || cpC;
+  if (need_fields && (rc = alloc_fields(ctx, F, g, B, st, cfg.step_kernel))) return rc;
   if (cpC && (rc = alloc_fields(ctx, U, g, B, st, cfg.step_kernel))) return rc;
   DevBuf snap, smax, num, den, dmax, stack, comp, cps;
   CU(snap.alloc(ctx, std::max<size_t>((size_t)B * ring * g.pplane * esz, 16), st));
@@ -1141,10 +1159,10 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
 
   for (long long q0 = 0; q0 < nitems; q0 += B) {
     nb = (int)std::min<long long>(B, nitems - q0);
-    A.item_sample = C.items.as<int>() + q0;
-    A.item_shot = C.items.as<int>() + nitems + q0;
+    A.item_sample = C.items + q0;
+    A.item_shot = C.items + nitems + q0;
     fill_args2(A2, A, C);
-    if ((rc = zero_fields(ctx, F, g, nb, st))) return rc;
+    if (need_fields && (rc = zero_fields(ctx, F, g, nb, st))) return rc;
     CU(cudaMemsetAsync(smax.p, 0, smax.bytes, st));
     CU(cudaMemsetAsync(dmax.p, 0, dmax.bytes, st));
     if (!cpC) {
@@ -1160,7 +1178,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
       if (born_refl) {
         // Born modelling: the perturbation field starts at rest; each step
         // adds c m S^{n+1} on imaging steps and records the receivers
-        if ((rc = zero_fields(ctx, F, g, nb, st))) return rc;
+        if (need_fields && (rc = zero_fields(ctx, F, g, nb, st))) return rc;
         A.refl = A2.refl = born_refl;
         A.rec_out = A2.rec_out = born_out + (size_t)q0 * nt * acq.nrec;
         A.len.rec_out = A2.len.rec_out = (nitems - q0) * (long long)nt * acq.nrec;
@@ -1198,7 +1216,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
         if ((rc = mark())) return rc;
         continue;
       }
-      if ((rc = zero_fields(ctx, F, g, nb, st))) return rc;
+      if (need_fields && (rc = zero_fields(ctx, F, g, nb, st))) return rc;
       if ((rc = issue_late(q0 / B))) return rc;
       if ((rc = mark())) return rc;
       {
@@ -1236,7 +1254,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
       if ((rc = mark())) return rc;
     }
     CU(launch_norm_stack(A.num, A.den, A.dmax, A.item_sample, nb, (float)op.eps, g.pplane,
-                         stack.as<float>(), comp.as<float>(), nsample, C.err.as<int>(), st));
+                         stack.as<float>(), comp.as<float>(), nsample, C.err, st));
     launches += 1;
   }
   launches += step_launches;
@@ -1248,7 +1266,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   }
   launches += 1;  // prep_c
   if (flag_slot >= 0)
-    CU(cudaMemcpyAsync(ctx->h_flags + 2 * flag_slot, C.err.p, 8, cudaMemcpyDeviceToHost, st));
+    CU(cudaMemcpyAsync(ctx->h_flags + 2 * flag_slot, C.err, 8, cudaMemcpyDeviceToHost, st));
   double ms_total = 0.0;
   if (ctx->prof) {
     CU(cudaStreamSynchronize(st));
@@ -1282,18 +1300,15 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
   const RunConfig cfg = resolve_config(ctx->defaults, make_geo(gr), B);
   const int sk = cfg.step_kernel;
   Common C;
-  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, cfg);
-  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
-  if (rc) return rc;
-  const Geo &g = C.g;
   std::vector<int> items(2 * (size_t)ns);
   for (int q = 0; q < ns; ++q) {
     items[q] = 0;
     items[ns + q] = s0 + q;
   }
-  CU(C.items.alloc(ctx, items.size() * 4, st));
-  CU(cudaMemcpyAsync(C.items.p, items.data(), items.size() * 4, cudaMemcpyHostToDevice, st));
-  if (ctx->defaults.resident && (rc = setup_resident(ctx, C, acq, B, st))) return rc;
+  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, cfg, B, items);
+  if (!rc) rc = maybe_inject_timeout(ctx, C, st);
+  if (rc) return rc;
+  const Geo &g = C.g;
   const bool res = C.res.C > 0;
   Fields F;
   if (!res && (rc = alloc_fields(ctx, F, g, B, st, sk))) return rc;
@@ -1305,8 +1320,8 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
   for (int q0 = 0; q0 < ns; q0 += B) {
     const int nb = std::min(B, ns - q0);
     if (!res && (rc = zero_fields(ctx, F, g, nb, st))) return rc;
-    A.item_sample = C.items.as<int>() + q0;
-    A.item_shot = C.items.as<int>() + ns + q0;
+    A.item_sample = C.items + q0;
+    A.item_shot = C.items + ns + q0;
     A.rec_out = seis_d + (size_t)q0 * gr.nt * acq.nrec;
     A.len.rec_out = (long long)(ns - q0) * gr.nt * acq.nrec;
     if (res) {  // the whole modelling in one launch
@@ -1340,7 +1355,7 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
     }
   }
   if (flag_slot >= 0)
-    CU(cudaMemcpyAsync(ctx->h_flags + 2 * flag_slot, C.err.p, 8, cudaMemcpyDeviceToHost, st));
+    CU(cudaMemcpyAsync(ctx->h_flags + 2 * flag_slot, C.err, 8, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));  // `items` lives on this stack frame
   std::lock_guard<std::mutex> lk(ctx->mu);
   ctx->stats.launches += launches + 1;
