@@ -54,6 +54,13 @@ struct Shape {
   static constexpr int R2 = R1 - 1;     // centre rows per thread at substep 2
   static constexpr int VZ = C2Z + 16;   // v^n tile rows (halo 8)
   static constexpr unsigned kTx = (VX * VZ + 2 * EX * EZ) * 4;  // bytes per stage
+  static constexpr unsigned kTxV = VX * VZ * 4;                 // of which v^n
+  // Whether a block of k_step2a starts on its Laplacians when v^n has arrived
+  // and waits for d^n and c behind them.  4 % faster with 16-row tiles (one item
+  // of 1701 x 351 3.67 -> 3.55 us a step, 4 of 851 x 176 3.89 -> 3.76) and 24-row
+  // ones (4 of 1701 x 351 8.95 -> 8.60); 32-row tiles would hold 20 more
+  // registers across the wait and lose 2.5 % (48 of 1701 x 351 77.1 -> 79.1).
+  static constexpr bool kSplit = R1 <= 4;
 };
 
 template <int R1>
@@ -105,10 +112,11 @@ __device__ __forceinline__ float &v1_at(Stage<R1> &S, int off) {
 }
 static_assert(EX == 128, "v1_at decodes offsets with EX = 128");
 
-// Issue tile t into stage S (all threads call; thread 0 issues the copies).
+// Issue tile t into stage S (all threads call; thread 0 issues the copies):
+// v^n completes on bar, d^n and c on bar_dc (which may be the same barrier).
 template <int R1>
 __device__ __forceinline__ void issue_tile(Stage<R1> &S, unsigned long long *bar,
-                                           const CUtensorMap *mv, const CUtensorMap *md,
+                                           unsigned long long *bar_dc, const CUtensorMap *mv, const CUtensorMap *md,
                                            const CUtensorMap *mc, const Step2Args &A, int t) {
   const Geo &g = A.g;
   const TileRef T = tile_at<R1>(g, t);
@@ -117,12 +125,17 @@ __device__ __forceinline__ void issue_tile(Stage<R1> &S, unsigned long long *bar
     const int smp = A.one_sample ? 0 : A.item_sample[T.b];
     (void)RTM_IN(smp, A.len.nsample, A.err);  // (the copy engine clips the box; a bad plane is
                                               // recorded, not read)
+    const bool one = bar == bar_dc;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(Shape<R1>::kTx)
+                 "r"(one ? Shape<R1>::kTx : Shape<R1>::kTxV)
                  : "memory");
     tma_load_3d(&S.v0[0][0], mv, T.x0 - 8, T.z0 - 8, T.b, bar);
-    tma_load_3d(&S.d[0][0], md, T.x0 - 4, T.z0 - 4, T.b, bar);
-    tma_load_3d(&S.c[0][0], mc, T.x0 - 4, T.z0 - 4, smp, bar);
+    if (!one)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar_dc)),
+                   "r"(Shape<R1>::kTx - Shape<R1>::kTxV)
+                   : "memory");
+    tma_load_3d(&S.d[0][0], md, T.x0 - 4, T.z0 - 4, T.b, bar_dc);
+    tma_load_3d(&S.c[0][0], mc, T.x0 - 4, T.z0 - 4, smp, bar_dc);
   }
   if (!tile_interior<R1>(g, T.x0, T.z0)) {  // edge-clamped sponge factors
     if (tid < EX) S.gxs[tid] = A.gx[min(max(T.x0 - 4 + tid, 0), g.P - 1)];
@@ -165,10 +178,12 @@ __device__ __forceinline__ void prefetch_imaging(const Step2Args &A, const Step2
 // Substep 1 on rows R1 ty .. R1 ty + R1 - 1, columns 4tx..4tx+3 of the
 // extended region: d^{n+1} into nd (Born source included) and S.d; v^n of the
 // same cells into ce.
-template <int MODE, bool SPONGE, bool ISO, int R1>
+// arrive(): waits for the d^n and c tiles, which the Laplacians do not need
+// (Shape::kSplit).
+template <int MODE, bool SPONGE, bool ISO, int R1, class Arrive>
 __device__ __forceinline__ void substep1p(Stage<R1> &S, const Step2Args &A, const Step2RT &rt,
                                           int b, int x0, int z0, float4 (&ce)[R1],
-                                          float4 (&nd)[R1]) {
+                                          float4 (&nd)[R1], Arrive arrive) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   const Geo &g = A.g;
   float4 zc[R1 + 8];
@@ -176,16 +191,29 @@ __device__ __forceinline__ void substep1p(Stage<R1> &S, const Step2Args &A, cons
   for (int q = 0; q < R1 + 8; ++q)
     zc[q] = *reinterpret_cast<const float4 *>(&S.v0[R1 * ty + q][4 + 4 * tx]);
   const float *gxs = &S.gxs[4 * tx];
+  float2 lap[Shape<R1>::kSplit ? R1 : 1][2];
 #pragma unroll
   for (int r = 0; r < R1; ++r) {
     const int er = R1 * ty + r;
     const float4 xl = *reinterpret_cast<const float4 *>(&S.v0[er + 4][4 * tx]);
     const float4 xr = *reinterpret_cast<const float4 *>(&S.v0[er + 4][8 + 4 * tx]);
-    const float4 dv = *reinterpret_cast<const float4 *>(&S.d[er][4 * tx]);
-    const float4 cv = *reinterpret_cast<const float4 *>(&S.c[er][4 * tx]);
-    const float gzr = SPONGE ? S.gzs[er] : 1.f;
-    nd[r] = update4<SPONGE, ISO>(&zc[r], xl, xr, dv, cv, A.k, gzr, gxs);
+    laplacian4<ISO>(&zc[r], xl, xr, A.k, lap[Shape<R1>::kSplit ? r : 0]);
     ce[r] = zc[r + 4];
+    if (!Shape<R1>::kSplit) {
+      const float4 dv = *reinterpret_cast<const float4 *>(&S.d[er][4 * tx]);
+      const float4 cv = *reinterpret_cast<const float4 *>(&S.c[er][4 * tx]);
+      nd[r] = difference4<SPONGE>(lap[0], ce[r], dv, cv, SPONGE ? S.gzs[er] : 1.f, gxs);
+    }
+  }
+  if (Shape<R1>::kSplit) {
+    arrive();
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const int er = R1 * ty + r;
+      const float4 dv = *reinterpret_cast<const float4 *>(&S.d[er][4 * tx]);
+      const float4 cv = *reinterpret_cast<const float4 *>(&S.c[er][4 * tx]);
+      nd[r] = difference4<SPONGE>(lap[Shape<R1>::kSplit ? r : 0], ce[r], dv, cv, SPONGE ? S.gzs[er] : 1.f, gxs);
+    }
   }
   if (MODE == MODE_BORN) {  // the Born source joins each row's new difference
     const int gcol = x0 - 4 + 4 * tx;
@@ -333,9 +361,11 @@ __device__ __forceinline__ void snap_f32(const Step2Args &A, int b, int idx, int
 // One tile: both substeps, the fused work of steps n+1 and n+2, the stores.
 // IN_IMG compiles in the imaging with the input field (rt.img_in_idx, dmax
 // flag 3); instances without it must not be launched with either set.
-template <int MODE, int R1, bool IN_IMG>
+// v^n has arrived; arrive(): waits for d^n and c, called by every thread.
+template <int MODE, int R1, bool IN_IMG, class Arrive>
 __device__ __forceinline__ void tile_body(Stage<R1> &S, float *red, const Step2Args &A,
-                                          const Step2RT &rt, int t, const InImg<R1> *pre) {
+                                          const Step2RT &rt, int t, const InImg<R1> *pre,
+                                          Arrive arrive) {
   constexpr int EZ = Shape<R1>::EZ, C2Z = Shape<R1>::C2Z, R2 = Shape<R1>::R2;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
   const Geo &g = A.g;
@@ -398,15 +428,17 @@ __device__ __forceinline__ void tile_body(Stage<R1> &S, float *red, const Step2A
   if (run1) {
     if (A.k.iso) {
       if (interior)
-        substep1p<MODE, false, true, R1>(S, A, rt, b, x0, z0, ce, nd);
+        substep1p<MODE, false, true, R1>(S, A, rt, b, x0, z0, ce, nd, arrive);
       else
-        substep1p<MODE, true, true, R1>(S, A, rt, b, x0, z0, ce, nd);
+        substep1p<MODE, true, true, R1>(S, A, rt, b, x0, z0, ce, nd, arrive);
     } else {
       if (interior)
-        substep1p<MODE, false, false, R1>(S, A, rt, b, x0, z0, ce, nd);
+        substep1p<MODE, false, false, R1>(S, A, rt, b, x0, z0, ce, nd, arrive);
       else
-        substep1p<MODE, true, false, R1>(S, A, rt, b, x0, z0, ce, nd);
+        substep1p<MODE, true, false, R1>(S, A, rt, b, x0, z0, ce, nd, arrive);
     }
+  } else if (Shape<R1>::kSplit) {
+    arrive();
   }
   __syncthreads();  // every read of v^n is done: the tile may take v^{n+1}
 
@@ -626,7 +658,7 @@ __global__ void __launch_bounds__(NTH, 2)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  issue_tile<R1>(S.st[0], &S.bar[0], &map_v, &map_d, &map_c, A, tile_index(0));
+  issue_tile<R1>(S.st[0], &S.bar[0], &S.bar[0], &map_v, &map_d, &map_c, A, tile_index(0));
   const bool imaging =
       MODE == MODE_BWD && (rt.img_mid_idx >= 0 || rt.img_out_idx >= 0 || rt.img_in_idx >= 0);
   if (imaging) prefetch_imaging<R1>(A, rt, tile_index(0));
@@ -635,7 +667,7 @@ __global__ void __launch_bounds__(NTH, 2)
     const bool has_next = (int)blockIdx.x + (k + 1) * G < ntiles;
     // stage s^1 was released by the barrier that ended tile k-1
     if (has_next) {
-      issue_tile<R1>(S.st[s ^ 1], &S.bar[s ^ 1], &map_v, &map_d, &map_c, A, tile_index(k + 1));
+      issue_tile<R1>(S.st[s ^ 1], &S.bar[s ^ 1], &S.bar[s ^ 1], &map_v, &map_d, &map_c, A, tile_index(k + 1));
       if (imaging) prefetch_imaging<R1>(A, rt, tile_index(k + 1));
     }
     const unsigned phase = (unsigned)(k >> 1) & 1u;
@@ -648,7 +680,7 @@ __global__ void __launch_bounds__(NTH, 2)
       if (has_next) mbar_wait_bounded(&S.bar[s ^ 1], (unsigned)((k + 1) >> 1) & 1u, kWaitNs);
       return;
     }
-    tile_body<MODE, R1, true>(S.st[s], S.red, A, rt, tile_index(k), nullptr);
+    tile_body<MODE, R1, true>(S.st[s], S.red, A, rt, tile_index(k), nullptr, [] {});
     // generic-proxy writes of this stage (d in place, v^{n+1}) are ordered
     // before the copy engine's next writes into it
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -663,7 +695,7 @@ __global__ void __launch_bounds__(NTH, 2)
 template <int R1>
 struct Smem1 {
   Stage<R1> st;
-  unsigned long long bar;
+  unsigned long long bar, bar_dc;  // v^n; d^n and c
   float red[NTH / 32];
 };
 
@@ -684,9 +716,12 @@ __global__ void __launch_bounds__(NTH, 3)
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&S.bar)), "r"(1)
                  : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&S.bar_dc)), "r"(1)
+                 : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   constexpr bool IN_IMG = (VAR & 1) != 0, PDL = (VAR & 2) != 0;
+  unsigned long long *const bar_dc = Shape<R1>::kSplit ? &S.bar_dc : &S.bar;
   __syncthreads();
   if constexpr (PDL) {
     // launched as a programmatic dependent: copy what the previous launch does
@@ -697,9 +732,13 @@ __global__ void __launch_bounds__(NTH, 3)
       const int smp = A.one_sample ? 0 : A.item_sample[T.b];
       (void)RTM_IN(smp, A.len.nsample, A.err);
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&S.bar)),
-                   "r"(Shape<R1>::kTx)
+                   "r"(Shape<R1>::kSplit ? Shape<R1>::kTxV : Shape<R1>::kTx)
                    : "memory");
-      tma_load_3d(&S.st.c[0][0], &map_c, T.x0 - 4, T.z0 - 4, smp, &S.bar);
+      if (Shape<R1>::kSplit)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar_dc)),
+                     "r"(Shape<R1>::kTx - Shape<R1>::kTxV)
+                     : "memory");
+      tma_load_3d(&S.st.c[0][0], &map_c, T.x0 - 4, T.z0 - 4, smp, bar_dc);
     }
     if (!tile_interior<R1>(A.g, T.x0, T.z0)) {
       if (tid < EX) S.st.gxs[tid] = A.gx[min(max(T.x0 - 4 + tid, 0), A.g.P - 1)];
@@ -711,10 +750,10 @@ __global__ void __launch_bounds__(NTH, 3)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
       tma_load_3d(&S.st.v0[0][0], &map_v, T.x0 - 8, T.z0 - 8, T.b, &S.bar);
-      tma_load_3d(&S.st.d[0][0], &map_d, T.x0 - 4, T.z0 - 4, T.b, &S.bar);
+      tma_load_3d(&S.st.d[0][0], &map_d, T.x0 - 4, T.z0 - 4, T.b, bar_dc);
     }
   } else {
-    issue_tile<R1>(S.st, &S.bar, &map_v, &map_d, &map_c, A, t);
+    issue_tile<R1>(S.st, &S.bar, bar_dc, &map_v, &map_d, &map_c, A, t);
   }
   if (MODE == MODE_BWD && (rt.img_mid_idx >= 0 || rt.img_out_idx >= 0))
     prefetch_imaging<R1>(A, rt, t);
@@ -725,10 +764,18 @@ __global__ void __launch_bounds__(NTH, 3)
   if (__syncthreads_or(!ok)) {  // (block-wide; also orders the staged sponge factors)
     if (tid == 0) atomicExch(A.err, 1);
     mbar_wait_bounded(&S.bar, 0, kWaitNs);  // let the copies in flight land (bounded)
+    mbar_wait_bounded(bar_dc, 0, kWaitNs);
     return;
   }
+  bool late = false;  // the wait for d^n and c gave up: flagged, the tile's result is void
   tile_body<MODE, R1, IN_IMG>(S.st, S.red, A, rt, t,
-                              IN_IMG && MODE == MODE_BWD && rt.img_in_idx >= 0 ? &pre : nullptr);
+                              IN_IMG && MODE == MODE_BWD && rt.img_in_idx >= 0 ? &pre : nullptr, [&] {
+                                if (!mbar_wait_bounded(bar_dc, 0, kWaitNs)) {
+                                  late = true;
+                                  atomicExch(A.err, 1);
+                                }
+                              });
+  if (late) mbar_wait_bounded(bar_dc, 0, kWaitNs);  // (as above)
 }
 
 size_t step2p_smem_bytes(int tile_z) {

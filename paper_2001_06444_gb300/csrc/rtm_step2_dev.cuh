@@ -196,13 +196,11 @@ __device__ __forceinline__ void laplacian4(const float4 *zc, const float4 &xl, c
   }
 }
 
-template <bool SPONGE, bool ISO>
-__device__ __forceinline__ float4 update4(const float4 *zc, const float4 &xl, const float4 &xr,
-                                          const float4 &dv, const float4 &cv, const Coef &k,
-                                          float gzr, const float *gxs) {
-  const float4 xc = zc[4];
-  float2 laps[2];
-  laplacian4<ISO>(zc, xl, xr, k, laps);
+// d^{n+1} of the strip from its Laplacian (laplacian4).
+template <bool SPONGE>
+__device__ __forceinline__ float4 difference4(const float2 (&laps)[2], const float4 &xc,
+                                              const float4 &dv, const float4 &cv, float gzr,
+                                              const float *gxs) {
   float out[4];
 #pragma unroll
   for (int l = 0; l < 4; l += 2) {
@@ -229,6 +227,15 @@ __device__ __forceinline__ float4 update4(const float4 *zc, const float4 &xl, co
     }
   }
   return make_float4(out[0], out[1], out[2], out[3]);
+}
+
+template <bool SPONGE, bool ISO>
+__device__ __forceinline__ float4 update4(const float4 *zc, const float4 &xl, const float4 &xr,
+                                          const float4 &dv, const float4 &cv, const Coef &k,
+                                          float gzr, const float *gxs) {
+  float2 laps[2];
+  laplacian4<ISO>(zc, xl, xr, k, laps);
+  return difference4<SPONGE>(laps, zc[4], dv, cv, gzr, gxs);
 }
 
 // Born modelling: d += (c m) S at the physical pixels of a 4-column strip
