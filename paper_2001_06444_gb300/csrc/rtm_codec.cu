@@ -1045,7 +1045,6 @@ template <bool LL>
 __global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ DecArgs a) {
   extern __shared__ __align__(16) float s_out[];  // [4][kOutPitch]: block l at columns 4 l .. 4 l + 3
   __shared__ unsigned char s_sfx[16][kDec];
-  __shared__ int s_n;
   const int tid = threadIdx.x, lane = tid & 31;
   const u64 nwin = (u64)a.count * a.nseg * kSegWins;
   for (u64 win = blockIdx.x; win < nwin; win += gridDim.x) {
@@ -1053,47 +1052,43 @@ __global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ D
     const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg), w = (u32)(win % kSegWins);
     const u32 B0 = sj * kSeg + w * kWin;  // first block of the window
     const unsigned char *slot = a.in + (u64)arr * a.stride;
-    if (tid == 0)
-      s_n = B0 < a.nb && header_ok(a, slot) && (reinterpret_cast<const u32 *>(slot)[2] != 0) == LL
-                ? (int)a.wincount[win]
-                : -1;
+    if (B0 >= a.nb || !header_ok(a, slot) || (reinterpret_cast<const u32 *>(slot)[2] != 0) != LL)
+      continue;  // (uniform: another mode's stream, or none)
+    const int n = (int)a.wincount[win];
     for (int i = tid; i < kOutPitch; i += kDec)
       reinterpret_cast<float4 *>(s_out)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
-    const int n = s_n;
-    if (n >= 0) {
-      const u32 *list = a.list + seg * kSeg + w * kWin;
-      const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
-      for (int p = tid; p < n; p += kDec) {
-        const u32 e = list[p];
-        const u32 b = sj * kSeg + (e >> 15);
-        u32 start, next;
-        if (!chunk_words(a, slot, b / kChunk, start, next)) continue;  // (reported by the walk)
-        GReader rd;
-        rd.init_at(words + start, next - start, e & 0x7fffu);
-        float x[16];
-        float *place = s_out + 4 * (b - B0);
-        const bool ok = decode_block<LL>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid], kDec,
-                                         reinterpret_cast<int *>(place), x) &&
-                        !rd.overrun();
-        if (!ok) report_bad(a, arr);
+    const u32 *list = a.list + seg * kSeg + w * kWin;
+    const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
+    for (int p = tid; p < n; p += kDec) {
+      const u32 e = list[p];
+      const u32 b = sj * kSeg + (e >> 15);
+      u32 start, next;
+      if (!chunk_words(a, slot, b / kChunk, start, next)) continue;  // (reported by the walk)
+      GReader rd;
+      rd.init_at(words + start, next - start, e & 0x7fffu);
+      float x[16];
+      float *place = s_out + 4 * (b - B0);
+      const bool ok = decode_block<LL>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid], kDec,
+                                       reinterpret_cast<int *>(place), x) &&
+                      !rd.overrun();
+      if (!ok) report_bad(a, arr);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          *reinterpret_cast<float4 *>(place + r * kOutPitch) =
-              make_float4(x[4 * r], x[4 * r + 1], x[4 * r + 2], x[4 * r + 3]);
-      }
-      __syncthreads();
-      // rows of the window, a warp per row (edge blocks clipped)
-      const u32 B1 = min(B0 + kWin, a.nb), bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
-      const u32 r1 = min(4 * bi1 + 4, (u32)a.n0);
-      for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kDec / 32) {
-        const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
-        const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
-        const u32 j0 = 4 * (lo - rb), j1 = min(4 * (hi - rb), (u32)a.n1);
-        float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
-        const float *src = s_out + (i & 3) * kOutPitch + 4 * (lo - B0);
-        for (u32 j = j0 + lane; j < j1; j += 32) row[j] = src[j - j0];
-      }
+      for (int r = 0; r < 4; ++r)
+        *reinterpret_cast<float4 *>(place + r * kOutPitch) =
+            make_float4(x[4 * r], x[4 * r + 1], x[4 * r + 2], x[4 * r + 3]);
+    }
+    __syncthreads();
+    // rows of the window, a warp per row (edge blocks clipped)
+    const u32 B1 = min(B0 + kWin, a.nb), bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
+    const u32 r1 = min(4 * bi1 + 4, (u32)a.n0);
+    for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kDec / 32) {
+      const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
+      const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
+      const u32 j0 = 4 * (lo - rb), j1 = min(4 * (hi - rb), (u32)a.n1);
+      float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
+      const float *src = s_out + (i & 3) * kOutPitch + 4 * (lo - B0);
+      for (u32 j = j0 + lane; j < j1; j += 32) row[j] = src[j - j0];
     }
     __syncthreads();  // (the window's memory is cleared for the next one)
   }
