@@ -193,7 +193,11 @@ int rtm_ctx_stats(rtm_ctx *ctx, rtm_stats *out, int reset);
  *   - whether each phase of a batch is captured and replayed as a CUDA graph.
  * The fastest is used by later rtm_migrate, rtm_migrate_ensemble and
  * request-loop calls with the same grid, nt, isnap and snapshot format.  All
- * candidates give bit-identical results.
+ * candidates give bit-identical results.  Whatever the choice, grids small
+ * enough run whole phases on chip where that is faster, and kernel-4 launches
+ * of up to about 6000 tiles are programmatic dependents of the one before.
+ * Without a tuned entry the library uses kernel 4 with the tile height (16, 24
+ * or 32) that suits the launch's size.
  * choice (nullable, 5 ints): {kernel 1 to 4, items cap (0 = memory), graph 0
  * or 1, tile height 16, 24 or 32, L2 prefetch 0 or 1}.  Synchronises the
  * stream. */
@@ -398,7 +402,8 @@ int rtm_compress(rtm_ctx *ctx, const float *data, long long count, long long n0,
  * stream that is malformed or was not made for n0 x n1 (the elements of its
  * damaged chunks are then unspecified).  Device scratch of 4 bytes per 4 x 4
  * block of up to 2^24 blocks at a time (the decode's block lists), plus 288
- * bytes per stream, is taken from the context's pool for the call. */
+ * bytes per stream and 4 per 1024 blocks, is taken from the context's pool for
+ * the call. */
 int rtm_decompress(rtm_ctx *ctx, const void *in, uint64_t in_stride, long long count,
                    long long n0, long long n1, float *data, void *stream);
 
@@ -411,14 +416,16 @@ int rtm_decompress(rtm_ctx *ctx, const void *in, uint64_t in_stride, long long c
  * horizontal neighbour times, ((T-a)^+/dz)^2 + ((T-b)^+/dx)^2 = (1/v)^2, and
  * T = 0 at the source node.  Its discrete solution is unique (the one fast
  * marching computes); the device reaches it by parallel fast sweeping, one
- * (sample, source) problem per CTA, in FP32.
+ * (sample, source) problem per CTA, in FP32.  Device scratch for the slowness
+ * and the work fields is taken from the context's pool for a group of problems
+ * at a time: 2 GB at most, or what one problem needs (about 30 bytes per node).
  * vel: [nsample][nz][nx] m/s, host or device, positive and finite
  * (RTM_ERR_ARG otherwise).  Sources and receivers: host arrays of node
  * indices.  times: [nsample][nsrc][nrec] s at the receivers, fields:
  * [nsample][nsrc][nz][nx] s, either may be NULL but not both; host or device.
  * flags: where each problem's work field lives.  0 chooses: in shared
- * memory (one problem per SM, the lowest latency per solve) when the
- * problems fit one per SM, else in an L2-resident device buffer (many
+ * memory (the lowest latency per solve) when all problems fit at once or
+ * enough of them fit an SM, else in an L2-resident device buffer (many
  * problems per SM, the highest throughput); RTM_EIK_OFFCHIP or RTM_EIK_SHARED
  * force one (fields larger than shared memory always stay off chip).
  * max_iter (<= 0: 64) caps the iterations of four sweeps; iters (host,

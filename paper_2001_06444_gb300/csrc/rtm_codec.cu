@@ -914,14 +914,15 @@ __device__ __forceinline__ int walk_key(u32 nw) {
 
 // Pass 1 of decoding: one thread per chunk, one segment (kWalk chunks) per
 // CTA.  The CTA's chunks are first ordered by size class (a counting sort in
-// shared memory), so that a warp walks chunks of similar length: the walk
-// moves one token per iteration and a warp takes as many iterations as its
-// longest chunk.  The bit offsets and cost classes of the blocks stay in
+// shared memory), so that a warp walks chunks of similar length: a trip skips a
+// run of zero blocks and walks one block, and a warp takes as many trips as its
+// longest chunk.  Bound by that chain of instructions (64 images of 351 x 1701 at
+// 1e-4: 139 us; 244 with a token a trip, every trip through the code of all
+// token kinds).  The bit offsets and cost classes of the blocks stay in
 // shared memory; the CTA then writes its windows' lists (the blocks that are
 // not all zero, ordered by class with a second counting sort per window) and
-// their counts.  One kernel per mode; each
-// skips the other mode's streams, and the fixed-accuracy one reports bad
-// headers.
+// their counts.  One kernel per mode; each skips the other mode's streams, and
+// the fixed-accuracy one reports bad headers.
 template <bool LL>
 __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecArgs a) {
   __shared__ unsigned short s_offs[kWalk][kChunk + 1];
@@ -1040,7 +1041,12 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
 // by its chunk, and leaves its 4 x 4 values in the window's shared memory; the
 // CTA then writes the window's rows, 32 consecutive floats a store (blocks
 // stored one by one in class order wrote half sectors, which cost the 64
-// images of 351 x 1701 490 MB of reads and 317 of writes for 76 and 153).
+// images of 351 x 1701 490 MB of reads and 317 of writes for 76 and 153).  Bound
+// by the bit coding's instructions and divergence: 270 us for those images.
+// Whole calls, 4 seismograms of 5000 x 1701 / those images, us: windows of 512
+// blocks with 256 threads 392 / 545, with 512 threads 501 / 612; 1024 with 256
+// 340 / 505 (but one 201 x 101 panel 188 against 173); 2048 with 512 373 / 559;
+// kept, 1024 with 512: 370 / 525 (same runs; blocks stored one by one 412 / 626).
 template <bool LL>
 __global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ DecArgs a) {
   extern __shared__ __align__(16) float s_out[];  // [4][kOutPitch]: block l at columns 4 l .. 4 l + 3

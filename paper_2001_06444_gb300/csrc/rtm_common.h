@@ -60,7 +60,7 @@ struct Geo {
   int nz, nx, SX, CP;     // physical grid and its memory column origin
   int ntx, ntz;           // tiles per grid (single-step kernel)
   int ntx2, ntz2;         // tiles per grid (two-step kernels)
-  int tz2;                // centre rows of a two-step tile (24, or 16 for the persistent kernel)
+  int tz2;                // centre rows of a two-step tile (16, 24 or 32)
   long long plane;        // NZ * P   (floats)
   long long pplane;       // nz * SX  (elements)
 };

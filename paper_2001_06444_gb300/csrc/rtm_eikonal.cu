@@ -520,6 +520,14 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
   }
 }
 
+// One problem per CTA.  64 models x 34 sources of 426 x 88 (R = 3, one warp,
+// fields off chip): 11.2 ms with k_eik_sweep, 2.5 ms here, bound by the fields'
+// stream (9.1 GB through L2 and DRAM at 3.6 TB/s) and the latency of its loads,
+// 4 to 5 problems a scheduler at 122 registers; ten problems' worth of L2
+// prefetch did not help (2.64 -> 2.78 ms), and keeping three tiles in turn
+// instead of moving registers costs residency (142 registers, 3.88 ms).  One
+// model x 34 sources (fields in shared memory): 4.26 -> 0.85 ms, bound by one
+// solve's chain of tile updates.
 template <int R, bool RES, bool ISO, bool W1>
 __global__ void __launch_bounds__(W1 ? 32 : 32 * kRowMaxWarps) k_eik_rows(const __grid_constant__ RowArgs A) {
   extern __shared__ __align__(16) unsigned char s_raw[];

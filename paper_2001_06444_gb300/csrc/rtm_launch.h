@@ -31,7 +31,7 @@ cudaError_t launch_step2p(int mode, int tile_z, const CUtensorMap &mv, const CUt
                           cudaStream_t st);
 size_t step2p_smem_bytes(int tile_z);
 // two-step kernel, one tile per block, v^{n+1} written over v^n (rtm_prop2p.cu):
-// tile_z = 24 or 32 centre rows, maps as for launch_step2p
+// tile_z = 16, 24 or 32 centre rows, maps as for launch_step2p
 cudaError_t launch_step2a(int mode, int tile_z, const CUtensorMap &mv, const CUtensorMap &md,
                           const CUtensorMap &mc, const Step2Args &A, const Step2RT &rt, int B,
                           cudaStream_t st);
