@@ -23,15 +23,14 @@
 // kmin is the largest k >= 1 with 16 2^k + 21.5 <= tol 2^(28-e), else 0.
 //
 // Encoding, in three passes with no device-side waiting:
-//   1. one CTA per tile of 128 blocks (4 chunks), one warp per chunk, one lane
-//      per block.  Each lane computes its block's coded length in closed form
+//   1. one warp per chunk, one lane per block.  Each lane computes its block's coded length in closed form
 //      (the events of the plane scan are the suffix maxima of the
 //      coefficients' top planes), a warp scan places the blocks, the lanes
-//      write their bits into shared memory, and the tile is copied to a
-//      staging slot of the maximum tile size;
-//   2. per array, an exclusive scan of the tiles' word counts, the header and
+//      write their bits into shared memory, and the chunk is copied to a
+//      staging slot of the maximum chunk size;
+//   2. per array, over tiles of 128 blocks (4 chunks), an exclusive scan of the tiles' word counts, the header and
 //      the stream's byte count;
-//   3. one CTA per tile copies its words to their offset and writes the
+//   3. one CTA per tile copies its chunks' words to their offset and writes the
 //      offsets of its chunks.
 // Decoding, per group of arrays, in two passes with no device-side waiting:
 //   1. the walk: one thread per chunk (a CTA's chunks ordered by size first)
@@ -65,6 +64,9 @@ constexpr int kTile = kChunk * kWarps;   // blocks per encoder tile (one CTA)
 constexpr int kBlockWords = 20;          // 640 bits bound one coded block
 constexpr int kChunkWords = kChunk * kBlockWords;
 constexpr int kTileWords = kTile * kBlockWords;
+constexpr int kEncWarps[2] = {1, 4};     // chunks of an encoder CTA: fixed accuracy, lossless
+static_assert(kWarps % kEncWarps[0] == 0 && kWarps % kEncWarps[1] == 0,
+              "an encoder CTA codes chunks of one tile");
 constexpr int kWalk = 128;               // decoder's walk: chunks per CTA, one per thread
 constexpr int kWalkKeys = 64;            // size classes the walk orders chunks by
 constexpr int kSeg = kWalk * kChunk;     // blocks of a walk CTA: a segment of the decode's list
@@ -105,7 +107,7 @@ struct EncArgs {
   unsigned char *out;
   u64 stride, index_bytes;
   u64 *sizes;             // [count] stream bytes
-  u32 *stage;             // [count * tiles][kTileWords] coded tiles
+  u32 *stage;             // [count * tiles * kWarps][kChunkWords] coded chunks
   u32 *chunk_words;       // [count * tiles][kWarps]
   u64 *tile_off;          // [count * tiles] word offset of each tile
   u32 *nonfinite;         // [count] array holds a NaN or an infinity
@@ -253,7 +255,7 @@ struct Block {
       nonfinite = mx >= 0x7f800000u;
       const u32 E = mx >> 23;
       e = E ? (int)E - 126 : (31 - __clz(mx)) - 148;
-      kmin = ktab[e + 150];
+      kmin = __ldg(ktab + e + 150);
       if (nonfinite) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) q[i] = 0;  // refused later; keep the length bounded
@@ -389,21 +391,27 @@ struct Block {
   }
 };
 
-// Pass 1: code one tile (128 blocks, 4 chunks) into its staging slot of
-// kTileWords words and record the words of each chunk.
+// Pass 1: a warp codes one chunk (32 blocks) into its staging slot of
+// kChunkWords words and records its length.  Bound by issue and by the warps in
+// flight to hide the coding's latencies.  No barrier: the chunks' lengths differ by
+// the data, and warps that met at a tile's barrier waited for its densest chunk
+// (2.6 of 12 stall cycles).  CTAs of one warp and 64 registers (32 warps an SM
+// instead of 24): 32 seismograms of 5000 x 1701 at 1e-4 1000 -> 857 us, 4 of them
+// 183 -> 170, 64 images of 351 x 1701 at 1e-4 297 -> 286; at 72 registers 939, at
+// 80 1004, CTAs of 4 warps 958.  Lossless, whose 105 registers leave 16 to 18
+// warps an SM: CTAs of 4 warps (32 seismograms 1513 -> 1475 us; of one warp 1747).
 template <bool LL>
-__global__ void __launch_bounds__(kTile, LL ? 4 : 6) k_cz_encode(const __grid_constant__ EncArgs a) {
-  __shared__ u32 sbuf[kWarps][kChunkWords];
-  __shared__ u32 s_words[kWarps];
-  __shared__ unsigned char s_kmin[kTab];
-  __shared__ unsigned char s_s[LL ? 1 : 16][kTile];  // entry planes (fixed accuracy)
-  __shared__ u32 s_m[LL ? 1 : 16][kTile];            // magnitudes (fixed accuracy)
+__global__ void __launch_bounds__(32 * kEncWarps[LL], LL ? 4 : 32)
+k_cz_encode(const __grid_constant__ EncArgs a) {
+  constexpr int NW = kEncWarps[LL], kEnc = 32 * NW;
+  __shared__ u32 sbuf[NW][kChunkWords];
+  __shared__ unsigned char s_s[LL ? 1 : 16][kEnc];  // entry planes (fixed accuracy)
+  __shared__ u32 s_m[LL ? 1 : 16][kEnc];            // magnitudes (fixed accuracy)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kTab; i += blockDim.x) s_kmin[i] = a.kmin[i];
-  __syncthreads();
-  const u64 T = blockIdx.x;  // tile over all arrays
+  const u64 G = (u64)blockIdx.x * NW + warp;  // chunk slot over all arrays
+  const u64 T = G / kWarps;                          // tile over all arrays
   const u32 arr = (u32)(T / a.tiles), lt = (u32)(T % a.tiles);
-  const u32 b = lt * kTile + threadIdx.x;
+  const u32 b = (lt * kWarps + (u32)(G % kWarps)) * kChunk + lane;
   const float *src = a.data + (long long)arr * a.n0 * a.n1;
 
   Block<LL> c;
@@ -419,7 +427,7 @@ __global__ void __launch_bounds__(kTile, LL ? 4 : 6) k_cz_encode(const __grid_co
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) bits[4 * r + cc] = __float_as_uint(row[col[cc]]);
     }
-    c.analyse(bits, s_kmin);
+    c.analyse(bits, a.kmin);
   } else {
     c.len = 0;
   }
@@ -434,7 +442,6 @@ __global__ void __launch_bounds__(kTile, LL ? 4 : 6) k_cz_encode(const __grid_co
   const u32 nw = (u32)(chunk_bits + 31) >> 5;
   u32 *buf = sbuf[warp];
   for (u32 i = lane; i < nw; i += 32) buf[i] = 0;
-  if (lane == 0) s_words[warp] = nw;
   __syncwarp();
   // fixed accuracy: warps of dense blocks keep the unrolled emission, the
   // others take the rolled loops (the vote is warp-uniform)
@@ -450,16 +457,17 @@ __global__ void __launch_bounds__(kTile, LL ? 4 : 6) k_cz_encode(const __grid_co
           s_m[i][threadIdx.x] = c.m[i];
         }
       }
-      c.emit_rolled(buf, (u32)(incl - c.len), &s_s[0][threadIdx.x], &s_m[0][threadIdx.x], kTile);
+      c.emit_rolled(buf, (u32)(incl - c.len), &s_s[0][threadIdx.x], &s_m[0][threadIdx.x], kEnc);
     }
   }
-  const int nf = __syncthreads_or(c.nonfinite);
-  u32 off = 0;
-  for (int w = 0; w < warp; ++w) off += s_words[w];
-  u32 *stage = a.stage + T * kTileWords;
-  for (u32 i = lane; i < nw; i += 32) stage[off + i] = buf[i];
-  if (lane == 0) a.chunk_words[T * kWarps + warp] = nw;
-  if (threadIdx.x == 0 && nf) atomicOr(a.nonfinite + arr, 1u);
+  __syncwarp();
+  const bool nf = __any_sync(0xffffffffu, c.nonfinite);
+  u32 *stage = a.stage + G * kChunkWords;
+  for (u32 i = lane; i < nw; i += 32) stage[i] = buf[i];
+  if (lane == 0) {
+    a.chunk_words[G] = nw;
+    if (nf) atomicOr(a.nonfinite + arr, 1u);
+  }
 }
 
 // Pass 2: per array, the word offset of every tile (exclusive scan of the
@@ -523,27 +531,32 @@ __global__ void __launch_bounds__(1024) k_cz_scan(const __grid_constant__ EncArg
   }
 }
 
-// Pass 3: copy each tile's words from its staging slot to its offset and
-// write the offsets of its chunks.
+// Pass 3: copy each tile's words from its chunks' staging slots to its offset
+// and write the offsets of its chunks.  The CTA's threads share the tile's words,
+// whatever their chunk (a warp per chunk waits for the longest one).
 __global__ void __launch_bounds__(kTile) k_cz_place(const __grid_constant__ EncArgs a) {
   const u64 T = blockIdx.x;
   const u32 arr = (u32)(T / a.tiles), lt = (u32)(T % a.tiles);
   const u32 *cw = a.chunk_words + T * kWarps;
-  u32 tw = 0;
+  u32 at[kWarps + 1];  // words before each chunk
+  at[0] = 0;
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) tw += cw[w];
+  for (int w = 0; w < kWarps; ++w) at[w + 1] = at[w] + cw[w];
   const u64 base = a.tile_off[T];
   unsigned char *slot = a.out + (u64)arr * a.stride;
   u32 *index = reinterpret_cast<u32 *>(slot + kHeader);
-  u32 *words = reinterpret_cast<u32 *>(slot + kHeader + a.index_bytes);
+  u32 *words = reinterpret_cast<u32 *>(slot + kHeader + a.index_bytes) + base;
   const u32 *stage = a.stage + T * kTileWords;
-  for (u32 i = threadIdx.x; i < tw; i += blockDim.x) words[base + i] = stage[i];
-  if (threadIdx.x < kWarps) {
-    const u32 chunk = lt * kWarps + threadIdx.x;
-    u32 off = 0;
-    for (int w = 0; w < (int)threadIdx.x; ++w) off += cw[w];
-    if (chunk < a.nchunk) index[chunk] = (u32)(base + off);
+  for (u32 i = threadIdx.x; i < at[kWarps]; i += blockDim.x) {
+    u32 from = i;  // word of the tile's staging slots
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w)
+      if (i >= at[w]) from = w * kChunkWords + (i - at[w]);
+    words[i] = stage[from];
   }
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if ((int)threadIdx.x == w && lt * kWarps + w < a.nchunk) index[lt * kWarps + w] = (u32)(base + at[w]);
 }
 
 // ---------------------------------------------------------------- decode --
@@ -1144,11 +1157,11 @@ cudaError_t launch_cz_encode(const float *data, long long count, long long n0, l
   a.n1 = n1;
   a.tiles = (u32)((nb + kTile - 1) / kTile);
   const u64 tiles = (u64)count * a.tiles;
-  if (tiles > 0x7fffffffull || count > 0xffffffffll) return cudaErrorInvalidValue;
+  if (tiles > 0x7fffffffull / kWarps || count > 0xffffffffll) return cudaErrorInvalidValue;
   a.out = out;
   a.stride = stride;
   a.sizes = sizes;
-  // scratch: stage | tile_off | chunk_words | nonfinite | kmin; every word but
+  // scratch: stage (a slot per chunk) | tile_off | chunk_words | nonfinite | kmin; every word but
   // the non-finite flags is written before it is read
   a.stage = reinterpret_cast<u32 *>(scratch);
   a.tile_off = reinterpret_cast<u64 *>(scratch + tiles * 4ull * kTileWords);
@@ -1161,10 +1174,10 @@ cudaError_t launch_cz_encode(const float *data, long long count, long long n0, l
   if (e != cudaSuccess) return e;
   k_cz_kmin<<<1, kTab, 0, st>>>(nullptr, 0, tol, tab);
   if (tol > 0) {
-    k_cz_encode<false><<<(unsigned)tiles, kTile, 0, st>>>(a);
+    k_cz_encode<false><<<(unsigned)(tiles * (kWarps / kEncWarps[0])), 32 * kEncWarps[0], 0, st>>>(a);
     k_cz_scan<false><<<(unsigned)count, 1024, 0, st>>>(a);
   } else {
-    k_cz_encode<true><<<(unsigned)tiles, kTile, 0, st>>>(a);
+    k_cz_encode<true><<<(unsigned)(tiles * (kWarps / kEncWarps[1])), 32 * kEncWarps[1], 0, st>>>(a);
     k_cz_scan<true><<<(unsigned)count, 1024, 0, st>>>(a);
   }
   k_cz_place<<<(unsigned)tiles, kTile, 0, st>>>(a);
