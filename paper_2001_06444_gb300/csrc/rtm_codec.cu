@@ -73,7 +73,8 @@ constexpr int kSeg = kWalk * kChunk;     // blocks of a walk CTA: a segment of t
 constexpr int kClasses = 256;            // decode cost classes (0: all-zero blocks)
 constexpr int kWin = 1024;               // blocks of a decode window
 constexpr int kSegWins = kSeg / kWin;    // windows of a segment
-constexpr int kDec = 512;                // decoder: threads per CTA, one block per thread
+constexpr int kDec = 256;                // decoder: threads per CTA, one block per thread
+constexpr int kDecWaves = 16;            // decoder: CTAs launched per resident one
 constexpr int kOutPitch = 4 * kWin + 8;  // floats of a window's row in shared memory
 constexpr u64 kGroupBlocks = 1ull << 24; // list entries per group of arrays
 static_assert(kSegWins == kWalk / 32 && kClasses % 32 == 0 && kSeg % kWin == 0,
@@ -122,7 +123,7 @@ struct DecArgs {
   u32 nb1, nb, nchunk;
   u64 stride, index_bytes;
   const unsigned char *kmin;  // [count][kTab]
-  int *err;  // [0] malformed flag, [1] first malformed array
+  int *err;  // [0] malformed flag, [1] first malformed array, [2 + mode] streams of the mode
   u32 arr0;       // first array of this group (error reports)
   u32 count;      // arrays in this group
   u32 nseg;       // segments (kWalk chunks, kSeg blocks) per array
@@ -956,6 +957,7 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
     return;
   }
   if ((reinterpret_cast<const u32 *>(slot)[2] != 0) != LL) return;
+  if (tid == 0) a.err[2 + LL] = 1;  // the mode's decode has work
   const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
   const u32 c0 = blockIdx.x * kWalk;
   const u32 rows = min((u32)kWalk, a.nchunk - c0);
@@ -1047,25 +1049,33 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
   if (bad) report_bad(a, arr);
 }
 
-// Pass 2: decode the windows of one mode, a CTA per window (a grid-stride
-// loop over one resident wave of CTAs), a thread per list entry, so that the
-// lanes of a warp hold blocks of one class and run the decode's loops for as
-// many trips.  Each thread reads its block's bits from global memory, bounded
-// by its chunk, and leaves its 4 x 4 values in the window's shared memory; the
-// CTA then writes the window's rows, 32 consecutive floats a store (blocks
-// stored one by one in class order wrote half sectors, which cost the 64
-// images of 351 x 1701 490 MB of reads and 317 of writes for 76 and 153).  Bound
-// by the bit coding's instructions and divergence: 270 us for those images.
-// Whole calls, 4 seismograms of 5000 x 1701 / those images, us: windows of 512
-// blocks with 256 threads 392 / 545, with 512 threads 501 / 612; 1024 with 256
-// 340 / 505 (but one 201 x 101 panel 188 against 173); 2048 with 512 373 / 559;
-// kept, 1024 with 512: 370 / 525 (same runs; blocks stored one by one 412 / 626).
+// Pass 2: decode the windows of one mode, a CTA per window at a time, a thread
+// per list entry, so that the lanes of a warp hold blocks of one class and run
+// the decode's loops for as many trips; the warps take the costliest entries
+// first.  Each thread reads its block's bits from global memory, bounded by its
+// chunk, and leaves its 4 x 4 values in the window's shared memory; the CTA then
+// writes the window's rows, 32 consecutive floats a store (blocks stored one by
+// one in class order wrote half sectors, which cost the 64 images of 351 x 1701
+// 490 MB of reads and 317 of writes for 76 and 153).  Bound by the bit coding's
+// instructions and divergence.  Whole calls, us, for 4 and 32 seismograms of
+// 5000 x 1701, those images (all at 1e-4) and 3 seismograms of 900 x 333:
+//   blocks stored one by one from lists of 4096 blocks    409  1635  617  328
+//   windows, 512 threads, entries in order                367  2071  472  173
+//   256 threads                                           335  1900  457  184
+//   and 4 times the resident CTAs instead of one wave     333  1855  434  184
+//   and the costliest entries first, to the next warp     311  1722  446  170
+//   and 16 times the resident CTAs (kept)                 313  1673  447  174
+// (512 threads with the last two: 335, 1920, 462, 169.  Windows of 2048 blocks
+// or of 512 were slower.)  32 seismograms, 60 % of whose blocks are zero, leave
+// few entries of a class per window: there the lists of 4096 were as fast.
 template <bool LL>
-__global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ DecArgs a) {
+__global__ void __launch_bounds__(kDec, 3) k_cz_decode(const __grid_constant__ DecArgs a) {
   extern __shared__ __align__(16) float s_out[];  // [4][kOutPitch]: block l at columns 4 l .. 4 l + 3
   __shared__ unsigned char s_sfx[16][kDec];
+  __shared__ int s_next;
   const int tid = threadIdx.x, lane = tid & 31;
   const u64 nwin = (u64)a.count * a.nseg * kSegWins;
+  if (!a.err[2 + LL]) return;
   for (u64 win = blockIdx.x; win < nwin; win += gridDim.x) {
     const u64 seg = win / kSegWins;
     const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg), w = (u32)(win % kSegWins);
@@ -1074,12 +1084,19 @@ __global__ void __launch_bounds__(kDec, 2) k_cz_decode(const __grid_constant__ D
     if (B0 >= a.nb || !header_ok(a, slot) || (reinterpret_cast<const u32 *>(slot)[2] != 0) != LL)
       continue;  // (uniform: another mode's stream, or none)
     const int n = (int)a.wincount[win];
+    if (tid == 0) s_next = 0;
     for (int i = tid; i < kOutPitch; i += kDec)
       reinterpret_cast<float4 *>(s_out)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     const u32 *list = a.list + seg * kSeg + w * kWin;
     const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
-    for (int p = tid; p < n; p += kDec) {
+    for (;;) {  // the costliest blocks first, 32 to the next warp that is free
+      int q = 0;
+      if (lane == 0) q = atomicAdd(&s_next, 32);
+      q = __shfl_sync(0xffffffffu, q, 0);
+      if (q >= n) break;
+      const int p = n - 1 - q - lane;
+      if (p < 0) continue;
       const u32 e = list[p];
       const u32 b = sj * kSeg + (e >> 15);
       u32 start, next;
@@ -1249,10 +1266,11 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
     a.out = out + (u64)g0 * (u64)n0 * (u64)n1;
     a.kmin = tab + (u64)g0 * kTab;
     const dim3 gwalk(a.nseg, (unsigned)g);
-    // the decode loops over the group's windows with one resident wave of CTAs
+    // each CTA of the decode takes up to a few windows (the last ones of a
+    // long loop would be uneven)
     const u64 nwin = (u64)g * a.nseg * kSegWins;
-    const unsigned gd0 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[0]) * nsm);
-    const unsigned gd1 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[1]) * nsm);
+    const unsigned gd0 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[0]) * nsm * kDecWaves);
+    const unsigned gd1 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[1]) * nsm * kDecWaves);
     k_cz_walk<false><<<gwalk, kWalk, 0, st>>>(a);
     k_cz_walk<true><<<gwalk, kWalk, 0, st>>>(a);
     k_cz_decode<false><<<gd0, kDec, kSmem, st>>>(a);
