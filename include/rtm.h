@@ -418,7 +418,8 @@ int rtm_decompress(rtm_ctx *ctx, const void *in, uint64_t in_stride, long long c
  * marching computes); the device reaches it by parallel fast sweeping, one
  * (sample, source) problem per CTA, in FP32.  Device scratch for the slowness
  * and the work fields is taken from the context's pool for a group of problems
- * at a time: 2 GB at most, or what one problem needs (about 30 bytes per node).
+ * at a time: 2 GB at most, or what one problem needs (16 bytes per node and the
+ * padding of the skewed layout).
  * vel: [nsample][nz][nx] m/s, host or device, positive and finite
  * (RTM_ERR_ARG otherwise).  Sources and receivers: host arrays of node
  * indices.  times: [nsample][nsrc][nrec] s at the receivers, fields:

@@ -218,7 +218,7 @@ constexpr int kRowGap = 4;    // tiles between the barriers of a CTA of several 
 constexpr int kRowRing = 16;  // tiles of a seam's ring (> kRowGap + 1 in flight)
 constexpr int kRowMap = 64 << 10;  // largest tile map (bytes)
 constexpr int kRowMaxWarps = 12;   // of a CTA: 1536 rows
-constexpr int kRowWarps = 8;  // resident warps an SM needs for shared-memory fields to win
+constexpr int kRowWarps = 8;  // resident warps an SM for shared-memory fields to win: row_plan
 
 // False: too large (k_eik_sweep solves it).
 bool row_geo(int nz, int nx, RowGeo &g) {
@@ -659,6 +659,13 @@ struct RowPlan {
 // Off-chip fields and slowness stay within about this much scratch.
 constexpr size_t kRowScratch = size_t(2) << 30;
 
+// Where the fields live: in shared memory if every problem is resident at once
+// (nothing is gained by more of them an SM), or if 8 warps an SM are, enough to
+// hide each other's latencies; else off chip.  Kernel ms, shared / off chip, nodes
+// from 1500 to 4500 m/s at random: 152 problems of 88 x 426 3.31 / 3.45, of 176 x
+// 176 2.27 / 2.94; 4800 problems of 20 x 40 0.35 / 0.53, of 64 x 64 (about 10 an SM)
+// 1.56 / 1.66, of 40 x 100 (fewer than 8) 1.81 / 1.66, of 64 x 200 7.09 / 5.35,
+// of 88 x 426 (one an SM) 78.6 / 26.6.
 static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
                      int smem_cta, int smem_sm) {
   if (!row_geo(nz, nx, p.g)) return false;
