@@ -422,7 +422,8 @@ int rtm_decompress(rtm_ctx *ctx, const void *in, uint64_t in_stride, long long c
  * padding of the skewed layout).
  * vel: [nsample][nz][nx] m/s, host or device, positive and finite
  * (RTM_ERR_ARG otherwise).  Sources and receivers: host arrays of node
- * indices.  times: [nsample][nsrc][nrec] s at the receivers, fields:
+ * indices; at most 2^31 - 1 (sample, source) problems (RTM_ERR_ARG beyond).
+ * times: [nsample][nsrc][nrec] s at the receivers, fields:
  * [nsample][nsrc][nz][nx] s, either may be NULL but not both; host or device.
  * flags: where each problem's work field lives.  0 chooses: in shared
  * memory (the lowest latency per solve) when all problems fit at once or

@@ -748,7 +748,6 @@ static cudaError_t launch_eikonal(EikArgs A, const float *slow, int nsample, boo
   A.slow = slow;
   const int nz = A.nz, nx = A.nx, nsrc = A.nsrc;
   const long long problems = (long long)nsample * nsrc;
-  if (problems > 0x7fffffffll) return cudaErrorInvalidValue;
   // tile shape: 2 x 2 (a short chain of dependent updates per thread, half
   // the diagonals of single nodes); RTM_EIK_TILE=TZxTX overrides it (one of
   // 1x1 2x2 2x4 4x2), for measurements
@@ -820,6 +819,10 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
     if (rec_iz[r] < 0 || rec_iz[r] >= nz || rec_ix[r] < 0 || rec_ix[r] >= nx)
       return fail(ctx, RTM_ERR_ARG, "receiver %d at (%d, %d) is outside the grid", r, rec_iz[r],
                   rec_ix[r]);
+  // the kernels, on either path, count problems in 32 bits
+  if ((long long)nsample * nsrc > 0x7fffffffll)
+    return fail(ctx, RTM_ERR_ARG, "%d samples x %d sources are more than 2^31 - 1 problems", nsample,
+                nsrc);
   if (max_iter <= 0) max_iter = 64;
   if ((flags & ~(RTM_EIK_OFFCHIP | RTM_EIK_SHARED)) || flags == (RTM_EIK_OFFCHIP | RTM_EIK_SHARED))
     return fail(ctx, RTM_ERR_ARG, "bad flags %d", flags);
