@@ -698,8 +698,7 @@ static cudaError_t launch_eik_rows(const RowPlan &P, const float *vel, int nsamp
   A.slow_b = slow + (size_t)P.group * P.g.quads;
   A.work = work;
   auto run = [&](auto kernel, unsigned n) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         P.smem);
+    const cudaError_t e = allow_shared_memory(kernel);
     if (e != cudaSuccess) return e;
     kernel<<<n, 32 * P.g.W, P.smem, st>>>(A);
     return cudaGetLastError();
@@ -766,8 +765,7 @@ static cudaError_t launch_eikonal(EikArgs A, const float *slow, int nsample, boo
   const size_t smem = resident ? (size_t)nz * nx * 4 : 0;
   auto go = [&](auto kernel) -> cudaError_t {
     if (resident) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+      const cudaError_t e = allow_shared_memory(kernel);
       if (e != cudaSuccess) return e;
     }
     kernel<<<(unsigned)problems, threads, smem, st>>>(A);

@@ -38,6 +38,19 @@ cudaError_t launch_step2a(int mode, int tile_z, const CUtensorMap &mv, const CUt
 size_t step2a_smem_bytes(int tile_z);
 // bounded-wait self-test: raises *flag after waiting `ns` for bytes that never arrive
 cudaError_t launch_wait_probe(int *flag, unsigned long long ns, cudaStream_t st);
+// Allows a kernel without static shared memory all the dynamic shared memory of
+// the device.  The limit belongs to the kernel, not to the launch: a call that
+// set it to its own size could lower it under another thread's larger launch.
+template <class K>
+cudaError_t allow_shared_memory(K kernel) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e == cudaSuccess
+             ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+             : e;
+}
 // whole phases with the grid on chip, one cluster of blocks per item
 // (rtm_resident.cu): C blocks of H rows; a thread owns R rows x 4 columns
 constexpr int kResRows = 6;

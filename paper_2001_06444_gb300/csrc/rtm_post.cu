@@ -367,8 +367,7 @@ cudaError_t launch_ens_stats(const float *images, int n, long long npix, double 
   const long long blocks = (npix + PB - 1) / PB;
   auto go = [&](auto kernel, int threads) -> cudaError_t {
     if (smem > 48 * 1024) {
-      cudaError_t e =
-          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = allow_shared_memory(kernel);
       if (e != cudaSuccess) return e;
     }
     kernel<<<(unsigned)blocks, threads, smem, st>>>(images, n, npad, PB, npix, mean, std_, q05, q95);
