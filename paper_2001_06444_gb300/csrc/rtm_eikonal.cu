@@ -14,7 +14,8 @@
 // sequential row-by-row sweep does (updated in this sweep, or from the
 // previous one) gives the sequential sweep's result bit for bit.
 //
-// k_eik_rows (every grid whose tile map fits, about 0.7 M nodes): each lane
+// k_eik_rows (grids whose tile map fits, about 0.7 M nodes, but not thousands of
+// tall ones: row_plan): each lane
 // owns R <= 4 consecutive rows, a warp up to 32 R rows, and walks tiles of R x
 // 4 nodes along them, one tile behind the lane of the rows before.  A tile's
 // neighbours above, below and beside come from the lane's registers and from
@@ -25,7 +26,7 @@
 // (they could not change), and a problem ends once no tile is left to
 // evaluate, instead of sweeping once more to find that nothing changes.
 //
-// k_eik_sweep (larger grids, and RTM_EIK_TILE): one CTA per problem, tiles on
+// k_eik_sweep (the others, and RTM_EIK_TILE): one CTA per problem, tiles on
 // one diagonal in parallel, a barrier per diagonal (Detrixhe, Gibou and Min
 // 2013).
 //
@@ -659,6 +660,9 @@ struct RowPlan {
 // Off-chip fields and slowness stay within about this much scratch.
 constexpr size_t kRowScratch = size_t(2) << 30;
 
+// Beyond this much of padded off-chip fields in all, tall grids go to k_eik_sweep.
+constexpr size_t kRowMost = size_t(4) << 30;
+
 // Where the fields live: in shared memory if every problem is resident at once
 // (nothing is gained by more of them an SM), or if 8 warps an SM are, enough to
 // hide each other's latencies; else off chip.  Kernel ms, shared / off chip, nodes
@@ -666,6 +670,18 @@ constexpr size_t kRowScratch = size_t(2) << 30;
 // 176 2.27 / 2.94; 4800 problems of 20 x 40 0.35 / 0.53, of 64 x 64 (about 10 an SM)
 // 1.56 / 1.66, of 40 x 100 (fewer than 8) 1.81 / 1.66, of 64 x 200 7.09 / 5.35,
 // of 88 x 426 (one an SM) 78.6 / 26.6.
+//
+// False, too, for many problems of tall grids: the skewed copies pad every tile
+// row by the lanes' offsets (1500 x 40: 50 times its nodes, 24 MB a problem), and
+// every sweep streams them, at a cost a quad that grows with the warps of a
+// problem, while k_eik_sweep costs about the same a node whatever the shape.
+// Whole calls, ms, rows / sweeps: while all copies stay within 2 GB the rows win
+// everywhere (1500 x 40 x 100: 9.0 / 10.2); beyond 4 GB by pad (quads x 4 / nodes)
+// times warps: 600 x 200 x 4800 (27) 45.2 / 60.0, 500 x 100 x 4800 (30) 24.5 / 25.5,
+// 400 x 120 x 4800 (32) 21.5 / 22.4, 300 x 60 x 4800 (34) 9.1 / 8.3, 1000 x 300 x
+// 1600 (43) 70.8 / 63.3, 400 x 60 x 4800 (59) 18.0 / 11.7, 1000 x 100 x 1600 (113)
+// 58.1 / 18.3, 1500 x 40 x 4800 (600) 460 / 33.  Problems of two warps never lose
+// (129 x 8 x 4800: 1.37 / 1.75).
 static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
                      int smem_cta, int smem_sm) {
   if (!row_geo(nz, nx, p.g)) return false;
@@ -679,6 +695,9 @@ static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flag
   }
   p.smem = base + (p.resident ? g.field_bytes : 0);
   const size_t per = 2 * (size_t)g.quads * sizeof(float4);  // both copies
+  if (!p.resident && g.W > 2 && (size_t)problems > kRowMost / per &&
+      4ll * g.quads * g.W > 33ll * nz * nx)
+    return false;
   const size_t per_sample = per + (p.resident ? 0 : per * nsrc);
   p.group = (int)std::max<size_t>(1, std::min<size_t>(nsample, kRowScratch / per_sample));
   p.chunk = (long long)p.group * nsrc;
