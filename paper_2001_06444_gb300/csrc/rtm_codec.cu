@@ -40,7 +40,8 @@
 //   2. the decode: a CTA per window, one block per thread in list order, so
 //      that the lanes of a warp run the same loops for as many trips; the
 //      window's values come together in shared memory and are written row by
-//      row.
+//      row.  Large groups: a CTA per segment of 4 windows, blocks written one by
+//      one over rows of zeros.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -76,8 +77,9 @@ constexpr int kSegWins = kSeg / kWin;    // windows of a segment
 constexpr int kDec = 256;                // decoder: threads per CTA, one block per thread
 constexpr int kDecWaves = 16;            // decoder: CTAs launched per resident one
 constexpr int kOutPitch = 4 * kWin + 8;  // floats of a window's row in shared memory
+constexpr int kDirPitch = 4 * kDec + 8;  // ... of the CTA's blocks, one per thread (DIRECT)
 constexpr u64 kGroupBlocks = 1ull << 24; // list entries per group of arrays
-static_assert(kSegWins == kWalk / 32 && kClasses % 32 == 0 && kSeg % kWin == 0,
+static_assert(kSegWins == 4 && kSegWins == kWalk / 32 && kClasses % 32 == 0 && kSeg % kWin == 0,
               "a warp of the walk scans the class counts of one window");
 static_assert(kSeg <= (1 << 13), "a segment's block index takes 13 bits of a list entry");
 constexpr int kHeader = 64;
@@ -762,7 +764,7 @@ __device__ bool walk_chunk(GReader &rd, u32 nblk, const unsigned char *ktab, uns
 }
 
 // Decode one block into x (the decode).  Returns false on a malformed block.
-template <bool LL, class R>
+template <bool LL, int PITCH, class R>
 __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
                                              unsigned char *sfx, int sstride, int *qs,
                                              float (&x)[16]) {
@@ -783,9 +785,8 @@ __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
   // refinement: magnitudes and signs, in coding order, each at the midpoint
   // of its kept interval.  Fixed accuracy takes a rolled loop over the
   // members (one trip per member, so lanes with as many members stay in
-  // step), the coefficients through the block's place in the window's shared
-  // memory, qs[(j / 4) kOutPitch + j % 4], j in block order (it comes zeroed);
-  // lossless keeps the unrolled register form (64-bit coefficients).
+  // step), the coefficients through the block's place in shared memory, qs[(j /
+  // 4) PITCH + j % 4], j in block order (it comes zeroed); lossless keeps the unrolled register form (64-bit coefficients).
   using S = typename std::conditional<LL, long long, int>::type;
   S q[16];
   long long qw[16];
@@ -801,12 +802,12 @@ __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
       if (t) {
         const long long v = (long long)((t << kmin) + half);
         const int j = perm_rt(i);
-        qs[(j >> 2) * kOutPitch + (j & 3)] = (int)((fs >> w) ? -v : v);
+        qs[(j >> 2) * PITCH + (j & 3)] = (int)((fs >> w) ? -v : v);
       }
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int4 t = *reinterpret_cast<const int4 *>(qs + r * kOutPitch);
+      const int4 t = *reinterpret_cast<const int4 *>(qs + r * PITCH);
       const int u[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
       for (int l = 0; l < 4; ++l) {
@@ -1049,16 +1050,18 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
   if (bad) report_bad(a, arr);
 }
 
-// Pass 2: decode the windows of one mode, a CTA per window at a time, a thread
-// per list entry, so that the lanes of a warp hold blocks of one class and run
-// the decode's loops for as many trips; the warps take the costliest entries
-// first.  Each thread reads its block's bits from global memory, bounded by its
-// chunk, and leaves its 4 x 4 values in the window's shared memory; the CTA then
-// writes the window's rows, 32 consecutive floats a store (blocks stored one by
-// one in class order wrote half sectors, which cost the 64 images of 351 x 1701
-// 490 MB of reads and 317 of writes for 76 and 153).  Bound by the bit coding's
-// instructions and divergence.  Whole calls, us, for 4 and 32 seismograms of
-// 5000 x 1701, those images (all at 1e-4) and 3 seismograms of 900 x 333:
+// Pass 2: decode the listed blocks of one mode, a thread per list entry, so that
+// the lanes of a warp hold blocks of one class and run the decode's loops for as
+// many trips; the warps take the costliest entries first.  Each thread reads its
+// block's bits from global memory, bounded by its chunk.  Bound by the bit coding's
+// instructions and divergence, and by the warps in flight to hide its chains.
+//
+// Windows (DIRECT false): a CTA takes a window at a time, gathers its 4 x 4 values
+// in shared memory and writes its rows, 32 consecutive floats a store (blocks
+// stored one by one in class order write half sectors, which cost 64 images of 351
+// x 1701 490 MB of reads and 317 of writes for 76 and 153).  Whole calls, us, for 4
+// and 32 seismograms of 5000 x 1701, those images (all at 1e-4) and 3 seismograms
+// of 900 x 333:
 //   blocks stored one by one from lists of 4096 blocks    409  1635  617  328
 //   windows, 512 threads, entries in order                367  2071  472  173
 //   256 threads                                           335  1900  457  184
@@ -1066,67 +1069,114 @@ __global__ void __launch_bounds__(kWalk) k_cz_walk(const __grid_constant__ DecAr
 //   and the costliest entries first, to the next warp     311  1722  446  170
 //   and 16 times the resident CTAs (kept)                 313  1673  447  174
 // (512 threads with the last two: 335, 1920, 462, 169.  Windows of 2048 blocks
-// or of 512 were slower.)  32 seismograms, 60 % of whose blocks are zero, leave
-// few entries of a class per window: there the lists of 4096 were as fast.
-template <bool LL>
-__global__ void __launch_bounds__(kDec, 3) k_cz_decode(const __grid_constant__ DecArgs a) {
-  extern __shared__ __align__(16) float s_out[];  // [4][kOutPitch]: block l at columns 4 l .. 4 l + 3
+// or of 512 were slower.)
+//
+// Segments (DIRECT): a CTA takes the 4 windows of a segment as one list, writes the
+// segment's rows as zeros and then each block over them.  Four times the entries
+// between two barriers, and 16 KB of shared memory instead of 64: 32 warps an SM
+// instead of 24.  For calls of many segments (kDirectSegs): a few of them leave the
+// device uneven.
+template <bool LL, bool DIRECT>
+__global__ void __launch_bounds__(kDec, DIRECT ? 4 : 3)
+k_cz_decode(const __grid_constant__ DecArgs a) {
+  // windows: [4][kOutPitch], block l at columns 4 l .. 4 l + 3; DIRECT: [4][kDirPitch],
+  // the block of thread t at columns 4 t .. 4 t + 3
+  extern __shared__ __align__(16) float s_out[];
   __shared__ unsigned char s_sfx[16][kDec];
   __shared__ int s_next;
+  constexpr int PITCH = DIRECT ? kDirPitch : kOutPitch;
+  constexpr u32 kUnit = DIRECT ? kSeg : kWin, kUnits = kSeg / kUnit;  // blocks of a unit, units of a segment
   const int tid = threadIdx.x, lane = tid & 31;
-  const u64 nwin = (u64)a.count * a.nseg * kSegWins;
+  const u64 nunit = (u64)a.count * a.nseg * kUnits;
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   if (!a.err[2 + LL]) return;
-  for (u64 win = blockIdx.x; win < nwin; win += gridDim.x) {
-    const u64 seg = win / kSegWins;
-    const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg), w = (u32)(win % kSegWins);
-    const u32 B0 = sj * kSeg + w * kWin;  // first block of the window
+  for (u64 unit = blockIdx.x; unit < nunit; unit += gridDim.x) {
+    const u64 seg = unit / kUnits;
+    const u32 arr = (u32)(seg / a.nseg), sj = (u32)(seg - (u64)arr * a.nseg), w = (u32)(unit % kUnits);
+    const u32 B0 = sj * kSeg + w * kUnit;  // first block of the unit
     const unsigned char *slot = a.in + (u64)arr * a.stride;
     if (B0 >= a.nb || !header_ok(a, slot) || (reinterpret_cast<const u32 *>(slot)[2] != 0) != LL)
       continue;  // (uniform: another mode's stream, or none)
-    const int n = (int)a.wincount[win];
+    u32 cnt[kSegWins];  // entries of the unit's windows (one: cnt[0])
+#pragma unroll
+    for (int k = 0; k < kSegWins; ++k) cnt[k] = k < (DIRECT ? kSegWins : 1) ? a.wincount[seg * kSegWins + w + k] : 0u;
+    const int n = (int)(cnt[0] + cnt[1] + cnt[2] + cnt[3]);
     if (tid == 0) s_next = 0;
-    for (int i = tid; i < kOutPitch; i += kDec)
-      reinterpret_cast<float4 *>(s_out)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // rows of the unit, a warp per row (edge blocks clipped)
+    const u32 B1 = min(B0 + kUnit, a.nb), bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
+    const u32 r1 = min(4 * bi1 + 4, (u32)a.n0);
+    auto rows = [&](auto value) {
+      for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kDec / 32) {
+        const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
+        const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
+        const u32 j0 = 4 * (lo - rb), j1 = min(4 * (hi - rb), (u32)a.n1);
+        float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
+        const float *src = s_out + (i & 3) * kOutPitch + 4 * (lo - B0);
+        for (u32 j = j0 + lane; j < j1; j += 32) row[j] = value(src + (j - j0));
+      }
+    };
+    if (DIRECT) {
+      rows([](const float *) { return 0.f; });
+    } else {
+      for (int i = tid; i < kOutPitch; i += kDec) reinterpret_cast<float4 *>(s_out)[i] = zero4;
+    }
     __syncthreads();
-    const u32 *list = a.list + seg * kSeg + w * kWin;
+    const u32 *list = a.list + seg * kSeg + w * kUnit;
     const u32 *words = reinterpret_cast<const u32 *>(slot + kHeader + a.index_bytes);
-    for (;;) {  // the costliest blocks first, 32 to the next warp that is free
+    for (;;) {  // the costliest blocks of a window first, 32 to the next warp that is free
       int q = 0;
       if (lane == 0) q = atomicAdd(&s_next, 32);
       q = __shfl_sync(0xffffffffu, q, 0);
       if (q >= n) break;
-      const int p = n - 1 - q - lane;
-      if (p < 0) continue;
-      const u32 e = list[p];
+      u32 p = (u32)(q + lane), first = 0, c = cnt[0];
+      if (p >= (u32)n) continue;
+#pragma unroll
+      for (int k = 1; k < (DIRECT ? kSegWins : 1); ++k)
+        if (first == (u32)(k - 1) * kWin && p >= c) {
+          p -= c;
+          first = k * kWin;
+          c = cnt[k];
+        }
+      const u32 e = list[first + c - 1 - p];
       const u32 b = sj * kSeg + (e >> 15);
       u32 start, next;
       if (!chunk_words(a, slot, b / kChunk, start, next)) continue;  // (reported by the walk)
       GReader rd;
       rd.init_at(words + start, next - start, e & 0x7fffu);
       float x[16];
-      float *place = s_out + 4 * (b - B0);
-      const bool ok = decode_block<LL>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid], kDec,
-                                       reinterpret_cast<int *>(place), x) &&
+      float *place = s_out + 4 * (DIRECT ? (u32)tid : b - B0);
+      if (DIRECT) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) *reinterpret_cast<float4 *>(place + r * PITCH) = zero4;
+      }
+      const bool ok = decode_block<LL, PITCH>(rd, a.kmin + (u64)arr * kTab, &s_sfx[0][tid], kDec,
+                                              reinterpret_cast<int *>(place), x) &&
                       !rd.overrun();
       if (!ok) report_bad(a, arr);
+      if (!DIRECT) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-        *reinterpret_cast<float4 *>(place + r * kOutPitch) =
-            make_float4(x[4 * r], x[4 * r + 1], x[4 * r + 2], x[4 * r + 3]);
+        for (int r = 0; r < 4; ++r)
+          *reinterpret_cast<float4 *>(place + r * PITCH) =
+              make_float4(x[4 * r], x[4 * r + 1], x[4 * r + 2], x[4 * r + 3]);
+      } else {
+        const u32 bi = b / a.nb1, bj = b - bi * a.nb1;
+        float *o = a.out + ((u64)arr * a.n0 + 4ull * bi) * a.n1 + 4ull * bj;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (4ll * bi + r < a.n0) {
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+              if (4ll * bj + l < a.n1) o[l] = x[4 * r + l];
+          }
+          o += a.n1;
+        }
+      }
     }
     __syncthreads();
-    // rows of the window, a warp per row (edge blocks clipped)
-    const u32 B1 = min(B0 + kWin, a.nb), bi0 = B0 / a.nb1, bi1 = (B1 - 1) / a.nb1;
-    const u32 r1 = min(4 * bi1 + 4, (u32)a.n0);
-    for (u32 i = 4 * bi0 + (tid >> 5); i < r1; i += kDec / 32) {
-      const u32 rb = (i >> 2) * a.nb1;  // first block of this row's block row
-      const u32 lo = max(B0, rb), hi = min(B1, rb + a.nb1);
-      const u32 j0 = 4 * (lo - rb), j1 = min(4 * (hi - rb), (u32)a.n1);
-      float *row = a.out + ((u64)arr * a.n0 + i) * a.n1;
-      const float *src = s_out + (i & 3) * kOutPitch + 4 * (lo - B0);
-      for (u32 j = j0 + lane; j < j1; j += 32) row[j] = src[j - j0];
+    if (!DIRECT) {
+      rows([](const float *v) { return *v; });
+      __syncthreads();  // (the window's memory is cleared for the next one)
     }
-    __syncthreads();  // (the window's memory is cleared for the next one)
   }
 }
 
@@ -1223,6 +1273,19 @@ u64 codec_decode_scratch_bytes(long long count, long long n0, long long n1) {
          4ull * kSeg * G * nseg;
 }
 
+// Segments of a group of arrays from which the decode takes whole segments
+// (k_cz_decode<., true>).  Whole calls, us, segments / windows, of n segments:
+//   seismograms of 5000 x 1701, n = 524 (4), 1e-4      335 /  323
+//   n = 1048 (8), 1e-4, 0.1, lossless                  458 /  473, 238 / 271, 487 /  513
+//   n = 2096 (16), 0.1                                 369 /  438
+//   n = 4192 (32), lossless                           1710 / 1843
+//   images of 351 x 1701 at 1e-4, n = 640 (64)         586 /  457
+//   n = 1000, 1500, 2000                               682 /  646, 892 / 889, 1249 / 1271
+//   images of 101 x 201 at 1e-4, n = 2000 (one each)   564 /  604
+// (blocks one by one from segments' lists, zero blocks in the walk, one wave of
+// CTAs: 420; 556, 253, 618; 371; 1753; 632; 772, 1007, 1313; 617.)
+constexpr u64 kDirectSegs = 1024;
+
 // scratch: codec_decode_scratch_bytes(count, n0, n1) bytes, 16-byte aligned;
 // its first 8 bytes must hold {0, 0x7fffffff} (the error record)
 cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long count, long long n0,
@@ -1232,29 +1295,35 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
   if (!codec_shape(n0, n1, &nb1, &nb, &nchunk, &a.index_bytes, nullptr))
     return cudaErrorInvalidValue;
   if (count < 1 || count > 65535) return cudaErrorInvalidValue;
-  int dev = 0, nsm = 0, per_sm[2] = {0, 0};
+  int dev = 0, nsm = 0, per_sm[2][2];  // [DIRECT][mode]
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  constexpr int kSmem = 4 * kOutPitch * (int)sizeof(float);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cz_decode<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cz_decode<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_cz_decode<false>, kDec, kSmem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_cz_decode<true>, kDec, kSmem);
+  constexpr int kSmem[2] = {4 * kOutPitch * (int)sizeof(float), 4 * kDirPitch * (int)sizeof(float)};
+  auto prepare = [&](auto kernel, int direct, int mode) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem[direct]);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[direct][mode], kernel, kDec, kSmem[direct]);
+  };
+  a.nseg = (u32)((nchunk + kWalk - 1) / kWalk);
+  const long long G = decode_group(count, nchunk);
+  const bool direct = (u64)G * a.nseg >= kDirectSegs;
+  if (direct) {
+    prepare(k_cz_decode<false, true>, 1, 0);
+    prepare(k_cz_decode<true, true>, 1, 1);
+  } else {
+    prepare(k_cz_decode<false, false>, 0, 0);
+    prepare(k_cz_decode<true, false>, 0, 1);
+  }
   if (e != cudaSuccess) return e;
   a.nb1 = (u32)nb1;
   a.nb = (u32)nb;
   a.nchunk = (u32)nchunk;
-  a.nseg = (u32)((nchunk + kWalk - 1) / kWalk);
   a.n0 = n0;
   a.n1 = n1;
   a.stride = stride;
   a.err = reinterpret_cast<int *>(scratch);
   unsigned char *tab = scratch + 16, *p = tab + ((u64)count * kTab + 15) / 16 * 16;
-  const long long G = decode_group(count, nchunk);
   a.wincount = reinterpret_cast<u32 *>(p);
   a.list = reinterpret_cast<u32 *>(p + (4ull * G * a.nseg * kSegWins + 15) / 16 * 16);
   k_cz_kmin<<<(unsigned)count, kTab, 0, st>>>(in, stride, 0.0, tab);
@@ -1266,15 +1335,21 @@ cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long coun
     a.out = out + (u64)g0 * (u64)n0 * (u64)n1;
     a.kmin = tab + (u64)g0 * kTab;
     const dim3 gwalk(a.nseg, (unsigned)g);
-    // each CTA of the decode takes up to a few windows (the last ones of a
-    // long loop would be uneven)
-    const u64 nwin = (u64)g * a.nseg * kSegWins;
-    const unsigned gd0 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[0]) * nsm * kDecWaves);
-    const unsigned gd1 = (unsigned)std::min<u64>(nwin, (u64)std::max(1, per_sm[1]) * nsm * kDecWaves);
+    // each CTA of the decode takes up to a few units (the last ones of a long
+    // loop would be uneven)
+    auto grid = [&](int mode) {
+      const u64 units = (u64)g * a.nseg * (direct ? 1 : kSegWins);
+      return (unsigned)std::min<u64>(units, (u64)std::max(1, per_sm[direct][mode]) * nsm * kDecWaves);
+    };
     k_cz_walk<false><<<gwalk, kWalk, 0, st>>>(a);
     k_cz_walk<true><<<gwalk, kWalk, 0, st>>>(a);
-    k_cz_decode<false><<<gd0, kDec, kSmem, st>>>(a);
-    k_cz_decode<true><<<gd1, kDec, kSmem, st>>>(a);
+    if (direct) {
+      k_cz_decode<false, true><<<grid(0), kDec, kSmem[1], st>>>(a);
+      k_cz_decode<true, true><<<grid(1), kDec, kSmem[1], st>>>(a);
+    } else {
+      k_cz_decode<false, false><<<grid(0), kDec, kSmem[0], st>>>(a);
+      k_cz_decode<true, false><<<grid(1), kDec, kSmem[0], st>>>(a);
+    }
   }
   return cudaGetLastError();
 }
