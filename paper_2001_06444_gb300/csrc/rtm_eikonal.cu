@@ -693,6 +693,10 @@ static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flag
     const long long per_sm = std::min(32 / g.W, smem_sm / (base + g.field_bytes + 1024));
     p.resident = (flags & RTM_EIK_SHARED) || problems <= per_sm * sms || per_sm * g.W >= kRowWarps;
   }
+  // forced into shared memory, but too large with its padding: k_eik_sweep keeps
+  // the bare field there
+  if ((flags & RTM_EIK_SHARED) && !p.resident && (size_t)nz * nx * 4 <= eik_resident_limit())
+    return false;
   p.smem = base + (p.resident ? g.field_bytes : 0);
   const size_t per = 2 * (size_t)g.quads * sizeof(float4);  // both copies
   if (!p.resident && g.W > 2 && (size_t)problems > kRowMost / per &&
