@@ -419,7 +419,8 @@ int rtm_decompress(rtm_ctx *ctx, const void *in, uint64_t in_stride, long long c
  * (sample, source) problem per CTA, in FP32.  Device scratch for the slowness
  * and the work fields is taken from the context's pool for a group of problems
  * at a time: 2 GB at most, or what one problem needs (16 bytes per node and the
- * padding of the skewed layout).
+ * padding of the skewed layout), and in smaller groups where the device has less
+ * left.
  * vel: [nsample][nz][nx] m/s, host or device, positive and finite
  * (RTM_ERR_ARG otherwise).  Sources and receivers: host arrays of node
  * indices; at most 2^31 - 1 (sample, source) problems (RTM_ERR_ARG beyond).

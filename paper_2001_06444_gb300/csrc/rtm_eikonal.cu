@@ -657,7 +657,8 @@ struct RowPlan {
   size_t slow_bytes = 0, work_bytes = 0;
 };
 
-// Off-chip fields and slowness stay within about this much scratch.
+// Off-chip fields and slowness stay within about this much scratch, and within
+// less where the device has less (rtm_eikonal).
 constexpr size_t kRowScratch = size_t(2) << 30;
 
 // Beyond this much of padded off-chip fields in all, tall grids go to k_eik_sweep.
@@ -683,7 +684,7 @@ constexpr size_t kRowMost = size_t(4) << 30;
 // 58.1 / 18.3, 1500 x 40 x 4800 (600) 460 / 33.  Problems of two warps never lose
 // (129 x 8 x 4800: 1.37 / 1.75).
 static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
-                     int smem_cta, int smem_sm) {
+                     int smem_cta, int smem_sm, size_t scratch) {
   if (!row_geo(nz, nx, p.g)) return false;
   const RowGeo &g = p.g;
   const int base = g.map_bytes + g.ring_bytes;
@@ -703,10 +704,10 @@ static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flag
       4ll * g.quads * g.W > 33ll * nz * nx)
     return false;
   const size_t per_sample = per + (p.resident ? 0 : per * nsrc);
-  p.group = (int)std::max<size_t>(1, std::min<size_t>(nsample, kRowScratch / per_sample));
+  p.group = (int)std::max<size_t>(1, std::min<size_t>(nsample, scratch / per_sample));
   p.chunk = (long long)p.group * nsrc;
   if (!p.resident)
-    p.chunk = std::max<long long>(1, std::min<long long>(p.chunk, (long long)(kRowScratch / per)));
+    p.chunk = std::max<long long>(1, std::min<long long>(p.chunk, (long long)(scratch / per)));
   p.slow_bytes = per * p.group;
   p.work_bytes = p.resident ? 16 : per * (size_t)p.chunk;
   return true;
@@ -885,9 +886,6 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   cudaDeviceGetAttribute(&smem_cta, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
-  RowPlan plan;
-  const bool rows = !getenv("RTM_EIK_TILE") && row_plan(plan, nz, nx, nsample, nsrc, flags, sms,
-                                                        smem_cta, smem_sm);
   const bool fits = (size_t)N * 4 <= eik_resident_limit();
   const bool resident = fits && !(flags & RTM_EIK_OFFCHIP) &&
                         ((flags & RTM_EIK_SHARED) || problems <= (long long)sms);
@@ -898,15 +896,36 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
     dt = dtimes.as<float>();
   }
   float *df = fields;
-  if ((fields && !is_device_ptr(fields)) || (!fields && !rows && !resident)) {
-    EIK_CU(dfields.alloc(ctx, fbytes, st));  // output staging, or the off-chip work fields
+  if (fields && !is_device_ptr(fields)) {
+    EIK_CU(dfields.alloc(ctx, fbytes, st));
     df = dfields.as<float>();
   }
   EIK_CU(diters.alloc(ctx, (size_t)problems * 4, st));
-  if (rows) {
-    EIK_CU(dslow.alloc(ctx, plan.slow_bytes, st));
-    EIK_CU(dwork.alloc(ctx, plan.work_bytes, st));
-  } else {
+  // the row-owning solver's scratch; where the device is too full for it, groups of
+  // half as many problems, down to one, and then the diagonal sweeps, which need none
+  // but the bare fields
+  RowPlan plan;
+  bool rows = false;
+  for (size_t scratch = kRowScratch; !getenv("RTM_EIK_TILE");) {
+    if (!row_plan(plan, nz, nx, nsample, nsrc, flags, sms, smem_cta, smem_sm, scratch)) break;
+    cudaError_t e = dslow.alloc(ctx, plan.slow_bytes, st);
+    if (e == cudaSuccess) e = dwork.alloc(ctx, plan.work_bytes, st);
+    if (e == cudaSuccess) {
+      rows = true;
+      break;
+    }
+    cudaGetLastError();
+    dslow.release();
+    dwork.release();
+    if (e != cudaErrorMemoryAllocation) EIK_CU(e);
+    if (plan.group == 1 && (plan.resident || plan.chunk == 1)) break;
+    scratch = std::min(scratch, plan.slow_bytes + plan.work_bytes) / 2;
+  }
+  if (!rows) {
+    if (!fields && !resident) {  // the off-chip work fields
+      EIK_CU(dfields.alloc(ctx, fbytes, st));
+      df = dfields.as<float>();
+    }
     EIK_CU(dslow.alloc(ctx, vbytes, st));
     EIK_CU(launch_eik_slowness(v, (long long)nsample * N, dslow.as<float>(), st));
   }
