@@ -298,7 +298,8 @@ struct RowProblem {
 
 // update() without branches, for a chain of dependent updates: the expressions
 // are the same, so are the bits (the root's argument is at least 1e-30, where
-// the flushing reciprocal square root equals the plain one).  ISO: dz == dx.
+// the flushing reciprocal square root equals the plain one).  ISO: dz == dx and
+// wz == wx.
 template <bool ISO>
 __device__ __forceinline__ float update_flat(float a, float b, float s, const EikArgs &A) {
   const float u1 = fminf(a, b), u2 = fmaxf(a, b);
@@ -727,7 +728,8 @@ static cudaError_t launch_eik_rows(const RowPlan &P, const float *vel, int nsamp
     kernel<<<n, 32 * P.g.W, P.smem, st>>>(A);
     return cudaGetLastError();
   };
-  const bool iso = E.dz == E.dx;
+  // (spacings that only round to the same float differ in their squares)
+  const bool iso = E.dz == E.dx && E.wz == E.wx;
   auto go = [&](auto rows, unsigned n) -> cudaError_t {
     constexpr int R = decltype(rows)::value;
     auto one = [&](auto res, auto same) -> cudaError_t {
