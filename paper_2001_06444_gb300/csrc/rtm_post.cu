@@ -98,8 +98,8 @@ __global__ void k_filter(const float *stack_all, const float *comp_all, int nz, 
 // 0.70 ms for 64 x 597,051.  The other (n <= kFastN, every value of the block
 // finite) takes one pixel per thread and no FP64 operation per value:
 //   - each value becomes an integer X on a grid 2^55 below the pixel's largest
-//     power of two (exact unless the value is 2^31 times smaller than the
-//     largest), so sum X is exact in 64 bits;
+//     power of two, so sum X is exact in 64 bits (a pixel with a value more than
+//     2^31 times smaller than its largest, which the grid would cut, sums in FP64);
 //   - with M the rounded mean of the X, sum (X - M)^2 is exact in three 64-bit
 //     sums of products of 28-bit digits, and sum (X - mean)^2 = sum (X - M)^2 -
 //     R^2 / n with R = sum X - n M: no cancellation, at most one rounding each
@@ -189,6 +189,22 @@ __device__ __forceinline__ void fast_stats(const float *col, int n, int PB, int 
   q95 = interpolate(c, d, f95);
 }
 
+// Mean and standard deviation of one column in FP64, two passes, as sorted_stats
+// takes them.
+__device__ __forceinline__ void column_moments(const float *col, int n, int PB, double &mean,
+                                               double &sd) {
+  double s = 0.0;
+  for (int k = 0; k < n; ++k) s += (double)col[k * PB];
+  const double m = s / n;
+  double q = 0.0;
+  for (int k = 0; k < n; ++k) {
+    const double d = (double)col[k * PB] - m;
+    q += d * d;
+  }
+  mean = m;
+  sd = n > 1 ? sqrt(q / (n - 1)) : 0.0;
+}
+
 // The general form on the column block in shared memory [npad][PB]: sums in FP64,
 // two passes, and a bitonic sort of each column.
 __device__ __forceinline__ void sorted_stats(float *sv, int n, int npad, int PB, long long p0,
@@ -269,14 +285,16 @@ __global__ void k_ens_stats_fast(const float *images, int n, int npad, int PB, l
   const long long p0 = (long long)blockIdx.x * PB;
   const int p = threadIdx.x;
   const bool in = p < PB && p0 + p < npix;
-  unsigned top = 0;  // largest magnitude's bits
+  unsigned top = 0, low = 0xffffffffu;  // bits of the largest magnitude, of the smallest but 0 (less 1)
   if (p < PB) {
     const float *src = images + p0 + p;
 #pragma unroll 8
     for (int k = 0; k < n; ++k) {
       const float v = in ? __ldcs(src + (long long)k * npix) : 0.f;
       sv[k * PB + p] = v;
-      top = max(top, __float_as_uint(v) & 0x7fffffffu);
+      const unsigned mag = __float_as_uint(v) & 0x7fffffffu;
+      top = max(top, mag);
+      low = min(low, mag - 1u);  // (0 becomes the largest)
     }
   }
   if (!__syncthreads_or(top >= 0x7f800000u)) {  // all finite
@@ -285,8 +303,13 @@ __global__ void k_ens_stats_fast(const float *images, int n, int npad, int PB, l
     const int lo5 = (int)floor(h5), lo95 = (int)floor(h95);
     double m, s;
     float a, b;
-    fast_stats<L>(sv + p, n, PB, max((int)(top >> 23), 1), 1.0 / n, n > 1 ? 1.0 / (n - 1) : 0.0, lo5,
-                  lo95, h5 - lo5, h95 - lo95, m, s, a, b);
+    const int emax = max((int)(top >> 23), 1);
+    fast_stats<L>(sv + p, n, PB, emax, 1.0 / n, n > 1 ? 1.0 / (n - 1) : 0.0, lo5, lo95, h5 - lo5,
+                  h95 - lo95, m, s, a, b);
+    // a value too small for the pixel's grid was cut: where the large ones cancel,
+    // it is the mean
+    if (emax - max((int)((low + 1u) >> 23), 1) > 31 && low != 0xffffffffu)
+      column_moments(sv + p, n, PB, m, s);
     mean[p0 + p] = m;
     std_[p0 + p] = s;
     q05[p0 + p] = a;
