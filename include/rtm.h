@@ -187,17 +187,19 @@ int rtm_ctx_stats(rtm_ctx *ctx, rtm_stats *out, int reset);
  *     list, the copies of the next tile overlapping the current one) with
  *     120 x 24 or 120 x 16 centre tiles; the two-step kernel with one tile
  *     per block that writes v^{n+1} over v^n in shared memory (kernel 4),
- *     which fits 120 x 24 or 120 x 32 tiles at 3 blocks per SM; or the
- *     single-step kernel (kernel 1);
+ *     which fits 120 x 16, 120 x 24 or 120 x 32 tiles at 3 blocks per SM; or
+ *     the single-step kernel (kernel 1);
  *   - the number of migrations in flight;
  *   - whether each phase of a batch is captured and replayed as a CUDA graph.
- * The fastest is used by later rtm_migrate, rtm_migrate_ensemble and
- * request-loop calls with the same grid, nt, isnap and snapshot format.  All
- * candidates give bit-identical results.  Whatever the choice, grids small
- * enough run whole phases on chip where that is faster, and kernel-4 launches
- * of up to about 6000 tiles are programmatic dependents of the one before.
- * Without a tuned entry the library uses kernel 4 with the tile height (16, 24
- * or 32) that suits the launch's size.
+ * All candidates give bit-identical results.  Without a tuned entry the
+ * library uses kernel 4 with the tile height (16, 24 or 32) that suits each
+ * launch's size, and all items that fit; that rule is a candidate too, and
+ * replaced only by one that is more than 2 % faster.  What is chosen is used by
+ * later rtm_migrate, rtm_migrate_ensemble and request-loop calls with the same
+ * grid, nt, isnap and snapshot format.  Whatever the choice, grids small enough
+ * run whole phases on chip where that is faster (for these only the last two
+ * points are tried; kernel 4 and 24 rows are reported), and kernel-4 launches of
+ * up to about 6000 tiles are programmatic dependents of the one before.
  * choice (nullable, 5 ints): {kernel 1 to 4, items cap (0 = memory), graph 0
  * or 1, tile height 16, 24 or 32, L2 prefetch 0 or 1}.  Synchronises the
  * stream. */

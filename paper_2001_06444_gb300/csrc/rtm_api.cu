@@ -579,6 +579,17 @@ static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<in
   C.res = resident_plan(g, B, ent, &C.res_max_ent);
 }
 
+// Whether B items of a call run their phases on chip.
+static bool runs_on_chip(const rtm_grid &gr, const rtm_acq &acq, int B) {
+  Common C;
+  std::vector<int2> ent;
+  C.g = make_geo(gr);
+  choose_resident(C, acq, B, ent);
+  return C.res.C > 0;
+}
+
+constexpr double kTuneMargin = 1.02;  // of rtm_autotune
+
 // Receiver lists of the two-step tiles: every tile whose extended region
 // (tile plus a 4-point ring) holds the receiver, and the one tile whose centre
 // does; offsets are r * EX + c within the extended region.
@@ -916,6 +927,12 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   if (rc) return rc;
   trace_mark("tables and model set up");
+  if (trace_enabled()) {
+    char how[96];
+    std::snprintf(how, sizeof how, "launches: on chip %d, kernel %d, rows %d, dependent %d, items %d",
+                  C.res.C > 0, cfg.step_kernel, cfg.tile_z, cfg.pdl, B);
+    trace_mark(how);
+  }
   const Geo &g = C.g;
   const bool res = C.res.C > 0;
   const int nsnap = gr.nt / op.isnap;
@@ -1545,6 +1562,7 @@ int rtm_ctx_set_batch(rtm_ctx *ctx, int max_items) {
 int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const rtm_opts *opts,
                  int trial_steps, int *choice, void *stream) {
   if (!ctx) return RTM_ERR_ARG;
+  CallTrace trace("rtm_autotune");
   int rc;
   if ((rc = check_grid(ctx, grid)) || (rc = check_acq(ctx, grid, acq, true)) ||
       (rc = check_opts(ctx, opts)))
@@ -1583,15 +1601,20 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
       1, std::min<long long>(nitems, (long long)((got - plan.shared_bytes - io) / plan.item_bytes)));
   DevBuf vel, seis, img;
   int best = -1;
-  double best_t = 1e300;
+  double best_t = 1e300, rule_t = 1e300;  // of all candidates, of the rule with every item in flight
   std::vector<RunConfig> cand;
-  // (kernel, tile height, L2 prefetch of later tiles): one tile per block
-  // without and with the prefetch, one tile per block with v^{n+1} over v^n
-  // (24 and 32 rows), persistent (24 and 16 rows), single step
-  const int kinds[7][3] = {{2, 24, 0}, {2, 24, 1}, {4, 24, 0}, {4, 32, 0},
-                           {3, 24, 0}, {3, 16, 0}, {1, 24, 0}};
-  for (const auto &kd : kinds)
-    for (int graph : {0, 1})
+  // (kernel, tile height, L2 prefetch of later tiles): the library's own rule
+  // (kernel 0), which a later call applies to its own number of items; one tile per
+  // block with v^{n+1} over v^n (16, 24 and 32 rows), one tile per block without and
+  // with the prefetch, persistent (24 and 16 rows), single step
+  const int kinds[9][3] = {{0, 24, 0}, {4, 16, 0}, {4, 24, 0}, {4, 32, 0}, {2, 24, 0},
+                           {2, 24, 1}, {3, 24, 0}, {3, 16, 0}, {1, 24, 0}};
+  // where the phases run on chip, every kernel's trial would run the same code
+  const bool on_chip = ctx->defaults.resident && runs_on_chip(tg, *acq, (int)bmax);
+  const int rule_z = resolve_config(RunConfig{}, make_geo(tg), (int)bmax).tile_z;
+  for (const auto &kd : kinds) {
+    if ((on_chip && kd[0]) || (kd[0] == 4 && kd[1] == rule_z)) continue;  // (as the rule's own)
+    for (int graph : {ctx->defaults.graph, 1 - ctx->defaults.graph})
       for (long long items : {bmax, (bmax + 1) / 2}) {
         RunConfig c;
         c.step_kernel = kd[0];
@@ -1606,6 +1629,7 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
                  o.l2_ahead == c.l2_ahead && o.graph == c.graph && o.max_items == c.max_items;
         if (!dup) cand.push_back(c);
       }
+  }
   rc = RTM_OK;
   do {
     if ((rc = vel.alloc(ctx, vbytes, st)) || (rc = seis.alloc(ctx, sbytes, st)) ||
@@ -1656,6 +1680,7 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
         if (!rc && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
           best_ms = std::min(best_ms, ms);
       }
+      if (i == 0) rule_t = best_ms;
       if (!rc && best_ms < best_t) {
         best_t = best_ms;
         best = (int)i;
@@ -1668,16 +1693,27 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
   if (!rc && cudaStreamSynchronize(st) != cudaSuccess) rc = fail(ctx, RTM_ERR_CUDA, "sync");
   unreserve(ctx, got);
   if (rc) return rc;
+  // two runs of one candidate differ by up to 2 %: only what is faster by more
+  // replaces the rule (a tuned entry pins its tile and cap for every later call)
+  if (rule_t <= kTuneMargin * best_t) best = 0;
+  RunConfig reported = cand[best];
+  if (reported.step_kernel == 0) {
+    if (on_chip)
+      reported.step_kernel = 4;  // (of phases that leave the chip; no tile was chosen)
+    else
+      reported = resolve_config(reported, make_geo(tg),
+                                reported.max_items > 0 ? reported.max_items : (int)bmax);
+  }
   {
     std::lock_guard<std::mutex> lk(ctx->mu);
     ctx->tuned[TuneKey{grid->nx, grid->nz, grid->nb, grid->nt, opts->isnap, opts->snap_dtype}] = cand[best];
   }
   if (choice) {
-    choice[0] = cand[best].step_kernel;
-    choice[1] = cand[best].max_items;
-    choice[2] = cand[best].graph;
-    choice[3] = cand[best].tile_z;
-    choice[4] = cand[best].l2_ahead;
+    choice[0] = reported.step_kernel;
+    choice[1] = reported.max_items;
+    choice[2] = reported.graph;
+    choice[3] = reported.tile_z;
+    choice[4] = reported.l2_ahead;
   }
   return RTM_OK;
 }
