@@ -1622,6 +1622,7 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
         c.l2_ahead = kd[2];
         c.graph = graph;
         c.resident = ctx->defaults.resident;
+        c.pdl = ctx->defaults.pdl;
         c.max_items = items >= nitems ? 0 : (int)items;
         bool dup = false;
         for (auto &o : cand)

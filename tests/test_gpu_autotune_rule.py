@@ -81,3 +81,11 @@ def test_phases_on_chip_are_not_told_apart_by_kernel():
     assert len({t[4] for t in trials}) <= 2 and len(trials) <= 12  # 2 graphs x 2 caps x 3 runs
     assert choice["max_items"] == 0
     assert after == before
+
+
+@pytest.mark.parametrize("pdl", [0, 1])
+def test_dependent_launches_stay_as_asked(pdl):
+    # RTM_PDL holds in the trials and after tuning
+    _, trials, before, after = _run(851, 176, 2, 120, 6, RTM_PDL=str(pdl))
+    lines = [t for t in trials + before + after if t[1] == 4]
+    assert len(lines) >= 6 and all(t[3] == pdl for t in lines), lines
