@@ -569,6 +569,11 @@ static RunConfig resolve_config(RunConfig c, const Geo &g, int B) {
 // Chooses the resident form for B items in flight; ent: its receiver table.
 static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<int2> &ent) {
   const Geo &g = C.g;
+  // (most grids are larger than any cluster holds: no table is sorted for them)
+  bool fits = false;
+  ResPlan p;
+  for (int c = 16; c >= 1 && !fits; c /= 2) fits = resident_shape(g, c, 0, p);
+  if (!fits) return;
   const int NS = (g.X0 + g.NX + 3) / 4;
   ent.resize(acq.nrec);
   for (int r = 0; r < acq.nrec; ++r) {
@@ -577,6 +582,7 @@ static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<in
   }
   std::stable_sort(ent.begin(), ent.end(), [](const int2 &a, const int2 &b) { return a.x < b.x; });
   C.res = resident_plan(g, B, ent, &C.res_max_ent);
+  if (C.res.C == 0) ent.clear();  // (nothing to upload)
 }
 
 // Whether B items of a call run their phases on chip.
