@@ -464,17 +464,46 @@ struct Common {
 
 // Host tables packed for one upload: a pageable copy synchronises its stream
 // before it starts, so one copy per table cost a small call most of its set-up.
+// Tables of more than kTableCopy bytes go up by themselves, from where they are (a
+// second host copy of 600,500 receivers' 14 MB took 2 ms); they have to live until
+// the stream is synchronised.
+constexpr size_t kTableCopy = 64 << 10;
 struct TablePack {
-  std::vector<unsigned char> h;
-  size_t add(const void *p, size_t bytes) {
-    const size_t o = (h.size() + 255) / 256 * 256;
-    h.resize(o + std::max<size_t>(bytes, 16), 0);
-    if (bytes) std::memcpy(h.data() + o, p, bytes);
-    return o;
+  struct Part {
+    const void *p;
+    size_t bytes, at;  // at: offset on the device (lay_out)
+  };
+  std::vector<Part> parts;
+  std::vector<unsigned char> h;  // the small tables, which lie first
+  int add(const void *p, size_t bytes) {
+    parts.push_back({p, bytes, 0});
+    return (int)parts.size() - 1;
   }
   template <class T>
-  size_t add(const std::vector<T> &v) {
+  int add(const std::vector<T> &v) {
     return add(v.data(), v.size() * sizeof(T));
+  }
+  // Places every table (an empty one holds 16 zero bytes); returns the bytes in all.
+  size_t lay_out() {
+    size_t size = 0;
+    for (int large : {0, 1}) {
+      for (Part &t : parts)
+        if ((t.bytes > kTableCopy) == (large != 0)) {
+          t.at = (size + 255) / 256 * 256;
+          size = t.at + std::max<size_t>(t.bytes, 16);
+        }
+      if (!large) h.resize(size, 0);
+    }
+    for (const Part &t : parts)
+      if (t.bytes && t.bytes <= kTableCopy) std::memcpy(h.data() + t.at, t.p, t.bytes);
+    return size;
+  }
+  cudaError_t upload(unsigned char *d, cudaStream_t st) const {
+    cudaError_t e = cudaMemcpyAsync(d, h.data(), h.size(), cudaMemcpyHostToDevice, st);
+    for (const Part &t : parts)
+      if (e == cudaSuccess && t.bytes > kTableCopy)
+        e = cudaMemcpyAsync(d + t.at, t.p, t.bytes, cudaMemcpyHostToDevice, st);
+    return e;
   }
 };
 
@@ -631,7 +660,7 @@ static void step2_receiver_lists(const Geo &g, const rtm_acq &acq, std::vector<i
   if (cent.empty()) cent.push_back(make_int2(0, 0));
 }
 
-// Choose the resident form, upload the per-call tables (one copy) and make c.
+// Choose the resident form, upload the per-call tables and make c.
 // items: the items' samples, then their shots.
 static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_acq &acq,
                         int nsample, const float *vel_d, cudaStream_t st, const RunConfig &cfg,
@@ -665,28 +694,28 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
   C.n_rext = (long long)eent.size();
   C.n_rcen = (long long)cent.size();
   TablePack t;
-  const size_t o_gx = t.add(gx), o_gz = t.add(gz), o_src = t.add(src), o_rptr = t.add(rptr),
-               o_rent = t.add(rent), o_eptr = t.add(eptr), o_eent = t.add(eent),
-               o_cptr = t.add(cptr), o_cent = t.add(cent),
-               o_wav = t.add(acq.wavelet, (size_t)gr.nt * 4), o_items = t.add(items),
-               o_res = t.add(res_ent), o_err = t.add(nullptr, 0);
+  const int i_gx = t.add(gx), i_gz = t.add(gz), i_src = t.add(src), i_rptr = t.add(rptr),
+            i_rent = t.add(rent), i_eptr = t.add(eptr), i_eent = t.add(eent), i_cptr = t.add(cptr),
+            i_cent = t.add(cent), i_wav = t.add(acq.wavelet, (size_t)gr.nt * 4),
+            i_items = t.add(items), i_res = t.add(res_ent), i_err = t.add(nullptr, 0);
+  const size_t table_bytes = t.lay_out();
   CU(C.c_all.alloc(ctx, (size_t)nsample * g.plane * 4, st));
-  CU(C.tables.alloc(ctx, t.h.size(), st));
-  CU(cudaMemcpyAsync(C.tables.p, t.h.data(), t.h.size(), cudaMemcpyHostToDevice, st));
-  unsigned char *base = C.tables.as<unsigned char>();
-  C.gx = reinterpret_cast<float *>(base + o_gx);
-  C.gz = reinterpret_cast<float *>(base + o_gz);
-  C.src_rc = reinterpret_cast<int *>(base + o_src);
-  C.rptr = reinterpret_cast<int *>(base + o_rptr);
-  C.rent = reinterpret_cast<int2 *>(base + o_rent);
-  C.rext_ptr = reinterpret_cast<int *>(base + o_eptr);
-  C.rext_ent = reinterpret_cast<int2 *>(base + o_eent);
-  C.rcen_ptr = reinterpret_cast<int *>(base + o_cptr);
-  C.rcen_ent = reinterpret_cast<int2 *>(base + o_cent);
-  C.wav = reinterpret_cast<float *>(base + o_wav);
-  C.items = reinterpret_cast<int *>(base + o_items);
-  C.res_ent = reinterpret_cast<int2 *>(base + o_res);
-  C.err = reinterpret_cast<int *>(base + o_err);
+  CU(C.tables.alloc(ctx, table_bytes, st));
+  CU(t.upload(C.tables.as<unsigned char>(), st));
+  auto table = [&](int i) { return C.tables.as<unsigned char>() + t.parts[i].at; };
+  C.gx = reinterpret_cast<float *>(table(i_gx));
+  C.gz = reinterpret_cast<float *>(table(i_gz));
+  C.src_rc = reinterpret_cast<int *>(table(i_src));
+  C.rptr = reinterpret_cast<int *>(table(i_rptr));
+  C.rent = reinterpret_cast<int2 *>(table(i_rent));
+  C.rext_ptr = reinterpret_cast<int *>(table(i_eptr));
+  C.rext_ent = reinterpret_cast<int2 *>(table(i_eent));
+  C.rcen_ptr = reinterpret_cast<int *>(table(i_cptr));
+  C.rcen_ent = reinterpret_cast<int2 *>(table(i_cent));
+  C.wav = reinterpret_cast<float *>(table(i_wav));
+  C.items = reinterpret_cast<int *>(table(i_items));
+  C.res_ent = reinterpret_cast<int2 *>(table(i_res));
+  C.err = reinterpret_cast<int *>(table(i_err));
   CU(launch_prep_c(vel_d, C.c_all.as<float>(), g, gr.dt, nsample, st));
   if (step_kernel >= 2 && !res) {
     const int H = step2_ext();
@@ -694,7 +723,7 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
                       g.tz2 + 2 * H);
     if (rc) return rc;
   }
-  // the packed tables go out of scope: make their copy complete first
+  // the tables go out of scope: make their copies complete first
   CU(cudaStreamSynchronize(st));
   return RTM_OK;
 }
