@@ -511,6 +511,24 @@ static double tile_step_us(double n, int tile_z);
 static double tiles_of(const Geo &g, int B, int tile_z);
 static int best_tile(const Geo &g, int B);
 
+// What more than one round of a tile's 256 threads over its receivers adds to a
+// step (us) that records: ten rows of receivers 1.1 (1.0), every cell 2.8 to 4 (1.8
+// to 3.5); one that injects takes twice that (both substeps, the tile's ring
+// included, by atomics): ten rows 2.3.
+static double tile_receivers_us(const Geo &g, int tile_z, const std::vector<ResCell> &cells) {
+  const int tx = step2_tile_x();
+  std::vector<int> n(g.ntx2 + 1, 0);  // of the present row of tiles
+  int end = 0, most = 0;
+  for (const ResCell &c : cells) {
+    if (c.row >= end) {
+      end = (c.row / tile_z + 1) * tile_z;
+      std::fill(n.begin(), n.end(), 0);
+    }
+    most = std::max(most, n[4 * c.strip / tx] += c.n);
+  }
+  return 0.25 * std::max(0, (most + 255) / 256 - 1);
+}
+
 // How B items' phases run with the grid on chip (k_resident), or C = 0 if the
 // tile kernels are the faster form or the grid does not fit.
 // Measured on a GB300 (600-step phases, FP32 and FP16 snapshots every 4 steps):
@@ -520,28 +538,38 @@ static int best_tile(const Geo &g, int B);
 //   1.0-1.2 us, in 4 blocks 2.3-2.9 us, 401 x 111 in 16 blocks 1.7 us, 501 x 181
 //   2.9-3.7 us; clusters beyond those that run at once take further rounds;
 //   a tile-kernel step as tile_step_us.
+// Receivers add resident_receivers_us or tile_receivers_us in the phases that record
+// or inject (rec_share of a call's steps).  30 items of 301 x 151 modelled over 200
+// steps, ms, on chip / tiles: a row 1.11 / 1.43, two rows 1.59 / 1.46, a well 1.76 /
+// 1.38, ten rows 3.03 / 1.66; one of 201 x 101: a row 0.28 / 0.50, ten 0.59 / 0.68.
 // Both sides near the line: 64 items of 201 x 101 4.8-6.4 us against 7.7, 7 of
 // 501 x 181 3.0-3.8 against 4.7, one of them 3.0-3.6 against 2.6; 851 x 176 does
 // not fit.
 // RTM_RESIDENT=C or C,R forces a cluster size (and rows a thread), 0 none.
-static ResPlan resident_plan(const Geo &g, int B, const std::vector<int2> &ent, int *max_ent) {
+static ResPlan resident_plan(const Geo &g, int B, const std::vector<ResCell> &cells,
+                             double rec_share, bool inject, int *max_ent) {
   const char *env = std::getenv("RTM_RESIDENT");
   int fc = 0, fr = 0;
   if (env) std::sscanf(env, "%d,%d", &fc, &fr);
   if (env && fc <= 0) return ResPlan{};
   const int tz = best_tile(g, B);
-  double best_t = fc > 0 ? 1e300 : tile_step_us(tiles_of(g, B, tz), tz);
+  double best_t = fc > 0 ? 1e300
+                         : tile_step_us(tiles_of(g, B, tz), tz) +
+                               (inject ? 2.0 : 1.0) * rec_share * tile_receivers_us(g, tz, cells);
   ResPlan best, p;
   for (int C : {16, 8, 4, 2, 1}) {
     if (fc > 0 && C != fc) continue;
     if (!resident_shape(g, C, fr, p)) continue;
-    const int ents = resident_max_ent(p, ent);
+    const int ents = resident_max_ent(p, cells);
     if (!resident_fits(p, ents)) continue;
     const int n = resident_clusters(p, ents);
     if (n < 1) continue;
-    const double t = ((B + n - 1) / n) *
-                     (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0) +
-                      (p.threads > 384 ? 0.4 : 0.0));
+    const int rounds = (B + n - 1) / n;
+    double t = rounds * (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0) +
+                         (p.threads > 384 ? 0.4 : 0.0));
+    if (t >= best_t) continue;
+    const double per_us = rounds * rec_share;
+    t += per_us * resident_receivers_us(p, cells, (best_t - t) / per_us);
     if (t < best_t) {
       best_t = t;
       best = p;
@@ -596,7 +624,8 @@ static RunConfig resolve_config(RunConfig c, const Geo &g, int B) {
 }
 
 // Chooses the resident form for B items in flight; ent: its receiver table.
-static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<int2> &ent) {
+static void choose_resident(Common &C, const rtm_acq &acq, int B, double rec_share, bool inject,
+                            std::vector<int2> &ent) {
   const Geo &g = C.g;
   // (most grids are larger than any cluster holds: no table is sorted for them)
   bool fits = false;
@@ -609,17 +638,18 @@ static void choose_resident(Common &C, const rtm_acq &acq, int B, std::vector<in
     const int row = acq.rec_iz[r] + g.nb, col = acq.rec_ix[r] + g.CP;
     ent[r] = make_int2(row * NS + col / 4, 4 * r + col % 4);
   }
-  std::stable_sort(ent.begin(), ent.end(), [](const int2 &a, const int2 &b) { return a.x < b.x; });
-  C.res = resident_plan(g, B, ent, &C.res_max_ent);
+  auto before = [](const int2 &a, const int2 &b) { return a.x < b.x; };
+  if (!std::is_sorted(ent.begin(), ent.end(), before)) std::stable_sort(ent.begin(), ent.end(), before);
+  C.res = resident_plan(g, B, resident_cells(ent, NS), rec_share, inject, &C.res_max_ent);
   if (C.res.C == 0) ent.clear();  // (nothing to upload)
 }
 
-// Whether B items of a call run their phases on chip.
+// Whether B items of a migration run their phases on chip.
 static bool runs_on_chip(const rtm_grid &gr, const rtm_acq &acq, int B) {
   Common C;
   std::vector<int2> ent;
   C.g = make_geo(gr);
-  choose_resident(C, acq, B, ent);
+  choose_resident(C, acq, B, 0.5, true, ent);
   return C.res.C > 0;
 }
 
@@ -661,10 +691,11 @@ static void step2_receiver_lists(const Geo &g, const rtm_acq &acq, std::vector<i
 }
 
 // Choose the resident form, upload the per-call tables and make c.
-// items: the items' samples, then their shots.
+// items: the items' samples, then their shots; rec_share: the part of the call's
+// steps that record or (inject) inject at the receivers.
 static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_acq &acq,
                         int nsample, const float *vel_d, cudaStream_t st, const RunConfig &cfg,
-                        int B, const std::vector<int> &items) {
+                        int B, double rec_share, bool inject, const std::vector<int> &items) {
   const int step_kernel = cfg.step_kernel;
   C.g = make_geo(gr, step_kernel >= 3 ? cfg.tile_z : 24);
   C.kernel = step_kernel;
@@ -674,7 +705,7 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
   C.nsample = nsample;
   const Geo &g = C.g;
   std::vector<int2> res_ent;
-  if (cfg.resident) choose_resident(C, acq, B, res_ent);
+  if (cfg.resident) choose_resident(C, acq, B, rec_share, inject, res_ent);
   const bool res = C.res.C > 0;
   std::vector<float> gz, gx;
   sponge_tables(g, gx, gz);
@@ -957,7 +988,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   }
   {
     PhaseRange ph("setup");
-    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg, B, items);
+    rc = setup_common(ctx, C, gr, acq, nsample, vel_d, st, cfg, B, 0.5, !born_refl, items);
   }
   if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   if (rc) return rc;
@@ -1357,7 +1388,7 @@ static int model_device(rtm_ctx *ctx, const rtm_grid &gr, const float *vel_d,
     items[q] = 0;
     items[ns + q] = s0 + q;
   }
-  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, cfg, B, items);
+  int rc = setup_common(ctx, C, gr, acq, 1, vel_d, st, cfg, B, 1.0, false, items);
   if (!rc) rc = maybe_inject_timeout(ctx, C, st);
   if (rc) return rc;
   const Geo &g = C.g;

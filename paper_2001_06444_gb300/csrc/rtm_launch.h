@@ -59,8 +59,18 @@ struct ResPlan {
 };
 // The shape with C blocks (R = 0: the fewest rows a thread that fit); false if it does not fit.
 bool resident_shape(const Geo &g, int C, int R, ResPlan &p);
-int resident_max_ent(const ResPlan &p, const std::vector<int2> &ent);
+// A strip of 4 columns of one row that holds receivers: n entries of the sorted
+// table from `first`; fast: one per column, in order.
+struct ResCell {
+  int row, strip, first, n;
+  bool fast;
+};
+std::vector<ResCell> resident_cells(const std::vector<int2> &ent, int NS);
+int resident_max_ent(const ResPlan &p, const std::vector<ResCell> &cells);
 bool resident_fits(const ResPlan &p, int max_ent);
+// What recording or injecting at the receivers adds to a step (us), or a value
+// beyond limit.
+double resident_receivers_us(const ResPlan &p, const std::vector<ResCell> &cells, double limit);
 int resident_clusters(const ResPlan &p, int max_ent);
 cudaError_t launch_resident(int mode, const ResPlan &p, ResArgs A, int B, cudaStream_t st);
 int step2_tile_x();

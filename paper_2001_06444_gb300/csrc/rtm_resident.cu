@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <array>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -784,11 +785,83 @@ bool resident_shape(const Geo &g, int C, int R, ResPlan &p) {
   return res_smem(p, 0) <= kResSmem;
 }
 
+// The block waits for the thread with the most receivers.  One row of them costs
+// little beside the step (a strip's 4 columns in order nothing); otherwise a thread
+// takes its entries one by one, about 0.1 us each, and looks up each row but its
+// first, 0.2 us and 0.02 a halving of the block's table.  Measured against this
+// (added us a step; 201 x 101 with 2 and with 6 rows a thread): four receivers a
+// cell 1.8 (1.6), a well 0.5 / 2.0 (0.5 / 1.9), ten rows 1.5 / 5.1 (1.2 / 4.5), every
+// cell 3.4 / 7.8, its traces' stores included (1.3 / 4.7).
+// Stops at `limit`, where the tile kernels are the faster form.
+double resident_receivers_us(const ResPlan &p, const std::vector<ResCell> &cells, double limit) {
+  const size_t n = cells.size();
+  if (n == 0) return 0.0;
+  bool plain = cells[0].row == cells[n - 1].row;  // one row, 4 entries a strip at most
+  for (size_t i = 0; plain && i < n; ++i) plain = cells[i].n <= 4;
+  if (plain) return 0.0;
+  std::vector<float> us(p.NS, 0.f);  // of the strips' threads in the present band of R rows
+  std::vector<char> rows(p.NS, 0);
+  float search = 0.f, most = 0.f;
+  int block = -1, block_end = 0, band_end = 0;  // rows behind the present block and band
+  for (size_t i = 0; i < n && most < limit; ++i) {
+    const ResCell &c = cells[i];
+    if (c.row >= block_end) {  // the block's table: the entries up to the next block
+      block = c.row / p.H;
+      block_end = (block + 1) * p.H;
+      band_end = 0;
+      const auto e = std::lower_bound(cells.begin() + i, cells.end(), block_end,
+                                      [](const ResCell &a, int x) { return a.row < x; });
+      const int last = e == cells.end() ? cells[n - 1].first + cells[n - 1].n : e->first;
+      search = 0.2f + 0.02f * std::log2((float)(last - c.first));
+    }
+    if (c.row >= band_end) {
+      band_end = block * p.H + ((c.row - block * p.H) / p.R + 1) * p.R;
+      std::fill(us.begin(), us.end(), 0.f);
+      std::fill(rows.begin(), rows.end(), 0);
+    }
+    float &t = us[c.strip];
+    char &seen = rows[c.strip];
+    if (seen == 0) {
+      t = c.fast ? 0.f : 0.1f * c.n;
+      seen = c.fast ? 1 : 2;
+    } else {
+      if (seen == 1) t = 0.4f;  // its first row is not its only one
+      t += 0.1f * c.n + search;
+      seen = 2;
+    }
+    most = std::max(most, t);
+  }
+  return most;
+}
+
+// The strips of 4 columns with receivers, in the order of ent (sorted by row and strip).
+std::vector<ResCell> resident_cells(const std::vector<int2> &ent, int NS) {
+  std::vector<ResCell> cells;
+  cells.reserve(ent.size() / 2 + 16);
+  int row = 0;
+  for (size_t i = 0, k; i < ent.size(); i += k) {
+    const int key = ent[i].x;
+    bool fast = (ent[i].y & 3) == 0;
+    for (k = 1; i + k < ent.size() && ent[i + k].x == key; ++k)
+      fast &= ent[i + k].y == ent[i].y + 5 * (int)k;
+    while (key >= (row + 1) * NS) ++row;
+    cells.push_back({row, key - row * NS, (int)i, (int)k, fast && k == 4});
+  }
+  return cells;
+}
+
 // The receivers of one block at most (for the shared-memory tables).
-int resident_max_ent(const ResPlan &p, const std::vector<int2> &ent) {
-  std::vector<int> n(p.C, 0);
-  for (const int2 &e : ent) n[std::min(e.x / p.NS / p.H, p.C - 1)]++;
-  return *std::max_element(n.begin(), n.end());
+int resident_max_ent(const ResPlan &p, const std::vector<ResCell> &cells) {
+  int most = 0, n = 0, end = 0;  // the last block takes what lies behind it, too
+  for (const ResCell &c : cells) {
+    if (c.row >= end && end < p.C * p.H) {
+      n = 0;
+      end = std::min(c.row / p.H + 1, p.C) * p.H;
+    }
+    n += c.n;
+    most = std::max(most, n);
+  }
+  return most;
 }
 
 bool resident_fits(const ResPlan &p, int max_ent) { return res_smem(p, max_ent) <= kResSmem; }

@@ -1,5 +1,6 @@
-"""Host tables of large receiver sets: a grid that no cluster of blocks holds does
-not pay for the tables of the phases on chip."""
+"""Receiver sets other than one row: a grid that no cluster of blocks holds does not
+pay for the tables of the phases on chip, and phases run on chip only where their
+receivers do not make that the slower form."""
 import time
 
 import numpy as np
@@ -42,3 +43,20 @@ def test_tables_of_a_grid_off_chip(monkeypatch):
     got, b = _model_time(monkeypatch, None, nx, nz, 4, rec_ix, rec_iz)
     assert torch.equal(a, b)
     assert got < 1.25 * want, (got, want)  # (22 ms against 14)
+
+
+@pytest.mark.parametrize("what", ["row", "ten rows", "well", "four wells", "every cell"])
+def test_receivers_that_suit_the_tiles_better(what, monkeypatch):
+    # 30 items: a row is faster on chip, the others with tiles
+    nx, nz = 301, 151
+    cells = {"row": [(i, 1) for i in range(nx)], "ten rows": [(i, k) for k in range(10) for i in range(nx)],
+             "well": [(nx // 2, k) for k in range(nz)],
+             "four wells": [(i, k) for i in (5, 50, 70, nx - 3) for k in range(nz)],
+             "every cell": [(i, k) for k in range(nz) for i in range(nx)]}[what]
+    rec_ix, rec_iz = np.array(cells, np.int64).T
+    tiles, a = _model_time(monkeypatch, "0", nx, nz, 200, rec_ix, rec_iz, nshot=30, reps=5)
+    default, b = _model_time(monkeypatch, None, nx, nz, 200, rec_ix, rec_iz, nshot=30, reps=5)
+    assert torch.equal(a, b)
+    assert default < 1.15 * tiles, (default, tiles)
+    if what == "row":
+        assert default < 0.9 * tiles, (default, tiles)
