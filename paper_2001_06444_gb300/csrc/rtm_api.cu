@@ -545,13 +545,17 @@ static double tile_receivers_us(const Geo &g, int tile_z, const std::vector<ResC
 // Both sides near the line: 64 items of 201 x 101 4.8-6.4 us against 7.7, 7 of
 // 501 x 181 3.0-3.8 against 4.7, one of them 3.0-3.6 against 2.6; 851 x 176 does
 // not fit.
+// With work of `beside` items more on other streams (the request loop) all of it
+// counts, and clusters of several launches pack less well (a quarter: 8 requests of
+// 12 shots of 401 x 111 on 8 blocks each 14.4 ms, the rounds of one launch 11.5).
 // RTM_RESIDENT=C or C,R forces a cluster size (and rows a thread), 0 none.
-static ResPlan resident_plan(const Geo &g, int B, const std::vector<ResCell> &cells,
+static ResPlan resident_plan(const Geo &g, int B, int beside, const std::vector<ResCell> &cells,
                              double rec_share, bool inject, int *max_ent) {
   const char *env = std::getenv("RTM_RESIDENT");
   int fc = 0, fr = 0;
   if (env) std::sscanf(env, "%d,%d", &fc, &fr);
   if (env && fc <= 0) return ResPlan{};
+  B += beside;
   const int tz = best_tile(g, B);
   double best_t = fc > 0 ? 1e300
                          : tile_step_us(tiles_of(g, B, tz), tz) +
@@ -567,6 +571,7 @@ static ResPlan resident_plan(const Geo &g, int B, const std::vector<ResCell> &ce
     const int rounds = (B + n - 1) / n;
     double t = rounds * (0.55 + 0.1 * p.R * (p.threads / 128.0) + (p.R > 4 ? 0.15 : 0.0) +
                          (p.threads > 384 ? 0.4 : 0.0));
+    if (beside) t *= 1.25;
     if (t >= best_t) continue;
     const double per_us = rounds * rec_share;
     t += per_us * resident_receivers_us(p, cells, (best_t - t) / per_us);
@@ -624,8 +629,8 @@ static RunConfig resolve_config(RunConfig c, const Geo &g, int B) {
 }
 
 // Chooses the resident form for B items in flight; ent: its receiver table.
-static void choose_resident(Common &C, const rtm_acq &acq, int B, double rec_share, bool inject,
-                            std::vector<int2> &ent) {
+static void choose_resident(Common &C, const rtm_acq &acq, int B, int beside, double rec_share,
+                            bool inject, std::vector<int2> &ent) {
   const Geo &g = C.g;
   // (most grids are larger than any cluster holds: no table is sorted for them)
   bool fits = false;
@@ -640,7 +645,7 @@ static void choose_resident(Common &C, const rtm_acq &acq, int B, double rec_sha
   }
   auto before = [](const int2 &a, const int2 &b) { return a.x < b.x; };
   if (!std::is_sorted(ent.begin(), ent.end(), before)) std::stable_sort(ent.begin(), ent.end(), before);
-  C.res = resident_plan(g, B, resident_cells(ent, NS), rec_share, inject, &C.res_max_ent);
+  C.res = resident_plan(g, B, beside, resident_cells(ent, NS), rec_share, inject, &C.res_max_ent);
   if (C.res.C == 0) ent.clear();  // (nothing to upload)
 }
 
@@ -649,7 +654,7 @@ static bool runs_on_chip(const rtm_grid &gr, const rtm_acq &acq, int B) {
   Common C;
   std::vector<int2> ent;
   C.g = make_geo(gr);
-  choose_resident(C, acq, B, 0.5, true, ent);
+  choose_resident(C, acq, B, 0, 0.5, true, ent);
   return C.res.C > 0;
 }
 
@@ -705,7 +710,7 @@ static int setup_common(rtm_ctx *ctx, Common &C, const rtm_grid &gr, const rtm_a
   C.nsample = nsample;
   const Geo &g = C.g;
   std::vector<int2> res_ent;
-  if (cfg.resident) choose_resident(C, acq, B, rec_share, inject, res_ent);
+  if (cfg.resident) choose_resident(C, acq, B, cfg.beside, rec_share, inject, res_ent);
   const bool res = C.res.C > 0;
   std::vector<float> gz, gx;
   sponge_tables(g, gx, gz);
@@ -979,7 +984,7 @@ int migrate_device(rtm_ctx *ctx, const rtm_grid &gr, int nsample, const float *v
   const long long nitems = (long long)nsample * acq.nshot;
   if (B > nitems) B = (int)nitems;
   if (B < 1) B = 1;
-  const RunConfig cfg = resolve_config(wanted, make_geo(gr), B);
+  const RunConfig cfg = resolve_config(wanted, make_geo(gr), B + wanted.beside);
   // items in (sample, shot) order
   std::vector<int> items(2 * nitems);
   for (long long q = 0; q < nitems; ++q) {

@@ -34,6 +34,7 @@ struct RunConfig {
   int pdl = -1;         // step_kernel 4: programmatic dependent launches (griddepcontrol);
                         // -1: chosen by the launch's size
   int resident = 1;     // run phases with the grid on chip where that is faster (resident_plan)
+  int beside = 0;       // other work on the device meanwhile, in items of this grid
 };
 // Shape key of the autotuner cache.
 struct TuneKey {

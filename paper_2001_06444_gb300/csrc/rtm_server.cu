@@ -36,6 +36,7 @@ struct rtm_req_state {
   MigrationPlan plan;
   size_t need1 = 0, want = 0, reserved = 0;
   int overtaken = 0;  // later requests admitted while this one headed the queue
+  double points = 0;  // of its grid, padded, times the shots in flight
   int state = RTM_REQ_QUEUED;
   int rc = RTM_OK;
   std::string err;
@@ -50,6 +51,7 @@ struct rtm_server {
   bool stop = false;
   uint64_t next = 1;
   int running = 0;
+  double points_running = 0;  // of the running requests
   int peak_running = 0;  // most requests running at once
   long long backfilled = 0;  // requests admitted past a waiting head
   bool log = false;          // RTM_SERVER_LOG=1: admissions and completions to stderr
@@ -59,6 +61,28 @@ struct rtm_server {
   static constexpr int kMaxOvertake = 16;    // backfill admissions past one waiting head
   static constexpr int kBackfillWindow = 64;  // queued requests looked at behind the head
 };
+
+// The work that runs beside request q, or will soon, in items of q's grid, for the
+// choice of its launches: small tiles or clusters of 16 blocks are the fastest for
+// one request alone, but not for the device.  8 requests of 12 shots of 401 x 111 and
+// 300 steps each planned alone took 14.3 ms (13.0 with the kernels before), planned
+// for all of them 11.9; 4 of 4 shots of 851 x 176 6.3 (5.5), 5.3; 24 of one shot
+// of 201 x 101 and 400 steps take 5.8 to 6.1.
+// A request starts about every 0.2 ms, and a step takes at least 1.5 us: of many short
+// requests only the first few overlap.
+static int work_beside(rtm_server *S, const rtm_req_state &q) {
+  constexpr double kStartUs = 200.0, kStepUs = 1.5;
+  std::lock_guard<std::mutex> lk(S->mu);
+  double points = S->points_running - q.points;
+  int others = S->running - 1;
+  for (auto it = S->queue.begin(); it != S->queue.end() && others + 1 < rtm_server::kMaxRunning; ++it) {
+    points += (*it)->points;
+    ++others;
+  }
+  if (others < 1) return 0;
+  const double overlap = std::min(1.0, 2.0 * q.r.grid.nt * kStepUs / kStartUs / others);
+  return (int)std::min(std::max(points * overlap / (double)q.plan.g.plane, 0.0), 1e6);
+}
 
 static void run_request(rtm_ctx *ctx, rtm_server *S, std::shared_ptr<rtm_req_state> q, int B) {
   int rc = RTM_OK;
@@ -73,10 +97,12 @@ static void run_request(rtm_ctx *ctx, rtm_server *S, std::shared_ptr<rtm_req_sta
   // threads share the context's)
   const int slot = rc ? -1 : flag_acquire(ctx);
   if (!rc) rc = check_velocity(ctx, q->r.grid, q->r.vel, (long long)q->r.grid.nx * q->r.grid.nz, st);
-  if (!rc)
+  if (!rc) {
+    RunConfig cfg = config_for(ctx, q->r.grid, q->r.opts);
+    cfg.beside = work_beside(S, *q);
     rc = migrate_device(ctx, q->r.grid, 1, q->r.vel, q->r.acq, q->r.seis, q->r.opts, q->r.image,
-                        B, st, config_for(ctx, q->r.grid, q->r.opts), nullptr, nullptr, nullptr,
-                        slot);
+                        B, st, cfg, nullptr, nullptr, nullptr, slot);
+  }
   if (rc && err.empty()) err = thread_error();
   if (st) {
     cudaError_t e = cudaStreamSynchronize(st);
@@ -99,6 +125,7 @@ static void run_request(rtm_ctx *ctx, rtm_server *S, std::shared_ptr<rtm_req_sta
     q->err = err;
     q->state = rc ? RTM_REQ_FAILED : RTM_REQ_DONE;
     S->running--;
+    S->points_running -= q->points;
     if (S->log)
       std::fprintf(stderr, "rtm-server %.3f done id=%llu rc=%d running=%d\n",
                    std::chrono::duration<double>(Clock::now() - S->t0).count(),
@@ -117,6 +144,8 @@ static void admit(rtm_ctx *ctx, rtm_server *S, const std::shared_ptr<rtm_req_sta
   const long long nitems = q->r.acq.nshot;
   long long B = (long long)((got - q->plan.shared_bytes) / q->plan.item_bytes);
   B = std::max<long long>(1, std::min<long long>(B, nitems));
+  q->points = (double)B * (double)q->plan.g.plane;
+  S->points_running += q->points;
   if (S->log)
     std::fprintf(stderr,
                  "rtm-server %.3f admit id=%llu grid=%dx%d shots=%d nt=%d B=%lld got=%.2fGB "
@@ -222,6 +251,7 @@ int rtm_server_submit(rtm_ctx *ctx, const rtm_request *req, uint64_t *ticket) {
   const int cap = ctx->max_batch > 0 ? ctx->max_batch : cfg.max_items;
   if (cap > 0 && nb > cap) nb = cap;
   q->want = q->plan.shared_bytes + (size_t)nb * q->plan.item_bytes;
+  q->points = (double)nb * (double)q->plan.g.plane;
   if (q->need1 > ctx->budget)
     return fail(ctx, RTM_ERR_NOMEM, "request needs %.3f GB, budget is %.3f GB", q->need1 / 1e9,
                 ctx->budget / 1e9);
