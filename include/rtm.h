@@ -193,14 +193,15 @@ int rtm_ctx_stats(rtm_ctx *ctx, rtm_stats *out, int reset);
  *   - whether each phase of a batch is captured and replayed as a CUDA graph.
  * All candidates give bit-identical results.  Without a tuned entry the
  * library uses kernel 4 with the tile height (16, 24 or 32) that suits each
- * launch's size, and all items that fit; that rule is a candidate too, and
- * replaced only by one that is more than 2 % faster.  What is chosen is used by
- * later rtm_migrate, rtm_migrate_ensemble and request-loop calls with the same
- * grid, nt, isnap and snapshot format.  Whatever the choice, grids small enough
- * run whole phases on chip where that is faster (for these only the last two
- * points are tried; kernel 4 and 24 rows are reported), and kernel-4 launches of
- * up to about 6000 tiles are programmatic dependents of the one before (all or
- * none of them with RTM_PDL=1 or 0 in the environment at rtm_ctx_create).
+ * launch's size, and all items that fit; that rule is a candidate too, with and
+ * without graphs, and replaced only by one that is more than 2 % faster.  What
+ * is chosen is used by later rtm_migrate, rtm_migrate_ensemble and request-loop
+ * calls with the same grid, nt, isnap and snapshot format.  Whatever the choice,
+ * grids small enough run whole phases on chip where that is faster (for these
+ * only the last two points are tried; kernel 4 and 24 rows are reported), and
+ * kernel-4 launches of up to about 6000 tiles are programmatic dependents of the
+ * one before (all or none of them with RTM_PDL=1 or 0 in the environment at
+ * rtm_ctx_create).
  * choice (nullable, 5 ints): {kernel 1 to 4, items cap (0 = memory), graph 0
  * or 1, tile height 16, 24 or 32, L2 prefetch 0 or 1}.  Synchronises the
  * stream. */

@@ -1671,8 +1671,8 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
   const long long bmax = std::max<long long>(
       1, std::min<long long>(nitems, (long long)((got - plan.shared_bytes - io) / plan.item_bytes)));
   DevBuf vel, seis, img;
-  int best = -1;
-  double best_t = 1e300, rule_t = 1e300;  // of all candidates, of the rule with every item in flight
+  int best = -1, rule = -1;  // of all candidates, of the rule with every item in flight
+  double best_t = 1e300, rule_t = 1e300;
   std::vector<RunConfig> cand;
   // (kernel, tile height, L2 prefetch of later tiles): the library's own rule
   // (kernel 0), which a later call applies to its own number of items; one tile per
@@ -1752,7 +1752,10 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
         if (!rc && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
           best_ms = std::min(best_ms, ms);
       }
-      if (i == 0) rule_t = best_ms;
+      if (!rc && c.step_kernel == 0 && c.max_items == cand[0].max_items && best_ms < rule_t) {
+        rule_t = best_ms;
+        rule = (int)i;
+      }
       if (!rc && best_ms < best_t) {
         best_t = best_ms;
         best = (int)i;
@@ -1766,8 +1769,9 @@ int rtm_autotune(rtm_ctx *ctx, const rtm_grid *grid, const rtm_acq *acq, const r
   unreserve(ctx, got);
   if (rc) return rc;
   // two runs of one candidate differ by up to 2 %: only what is faster by more
-  // replaces the rule (a tuned entry pins its tile and cap for every later call)
-  if (rule_t <= kTuneMargin * best_t) best = 0;
+  // replaces the rule, with or without graphs as it was the faster (a tuned entry
+  // pins its tile and cap for every later call)
+  if (rule >= 0 && rule_t <= kTuneMargin * best_t) best = rule;
   RunConfig reported = cand[best];
   if (reported.step_kernel == 0) {
     if (on_chip)
