@@ -23,13 +23,13 @@
 // kmin is the largest k >= 1 with 16 2^k + 21.5 <= tol 2^(28-e), else 0.
 //
 // Encoding, in three passes with no device-side waiting:
-//   1. one warp per chunk, one lane per block.  Each lane computes its block's coded length in closed form
-//      (the events of the plane scan are the suffix maxima of the
-//      coefficients' top planes), a warp scan places the blocks, the lanes
-//      write their bits into shared memory, and the chunk is copied to a
-//      staging slot of the maximum chunk size;
-//   2. per array, over tiles of 128 blocks (4 chunks), an exclusive scan of the tiles' word counts, the header and
-//      the stream's byte count;
+//   1. one warp per chunk, one lane per block.  Each lane computes its block's
+//      coded length in closed form (the events of the plane scan are the suffix
+//      maxima of the coefficients' top planes), a warp scan places the blocks,
+//      the lanes write their bits into shared memory, and the chunk is copied to
+//      a staging slot of the maximum chunk size;
+//   2. per array, over tiles of 128 blocks (4 chunks), an exclusive scan of the
+//      tiles' word counts, the header and the stream's byte count;
 //   3. one CTA per tile copies its chunks' words to their offset and writes the
 //      offsets of its chunks.
 // Decoding, per group of arrays, in two passes with no device-side waiting:
@@ -81,7 +81,7 @@ constexpr int kDirPitch = 4 * kDec + 8;  // ... of the CTA's blocks, one per thr
 constexpr u64 kGroupBlocks = 1ull << 24; // list entries per group of arrays
 static_assert(kSegWins == 4 && kSegWins == kWalk / 32 && kClasses % 32 == 0 && kSeg % kWin == 0,
               "a warp of the walk scans the class counts of one window");
-static_assert(kSeg <= (1 << 13), "a segment's block index takes 13 bits of a list entry");
+static_assert(kSeg <= (1 << 12), "a segment's block index takes 12 bits of a list entry");
 constexpr int kHeader = 64;
 constexpr u32 kMagic = 0x5A4D5452u;
 constexpr u32 kVersion = 3;
@@ -1263,7 +1263,7 @@ static long long decode_group(long long count, long long nchunk) {
 
 // device scratch of one decompression, in bytes: the 16-byte error record,
 // the kmin tables (count x kTab bytes, padded to 16), then for a group of
-// arrays the segment counts (4 bytes per segment, padded to 16) and lists
+// arrays the windows' counts (4 bytes per window, padded to 16) and lists
 // (4 bytes per block slot)
 u64 codec_decode_scratch_bytes(long long count, long long n0, long long n1) {
   long long nchunk = 0;
@@ -1287,7 +1287,8 @@ u64 codec_decode_scratch_bytes(long long count, long long n0, long long n1) {
 constexpr u64 kDirectSegs = 1024;
 
 // scratch: codec_decode_scratch_bytes(count, n0, n1) bytes, 16-byte aligned;
-// its first 8 bytes must hold {0, 0x7fffffff} (the error record)
+// its first 16 bytes must hold {0, 0x7fffffff, 0, 0} (the error record and the
+// modes met)
 cudaError_t launch_cz_decode(const unsigned char *in, u64 stride, long long count, long long n0,
                              long long n1, float *out, unsigned char *scratch, cudaStream_t st) {
   DecArgs a{};

@@ -523,7 +523,7 @@ __device__ __forceinline__ void row_sweep(const RowProblem &Q, const RowGeo &g, 
 }
 
 // One problem per CTA.  64 models x 34 sources of 426 x 88 (R = 3, one warp,
-// fields off chip): 11.2 ms with k_eik_sweep, 2.5 ms here, bound by the fields'
+// fields off chip): 11.2 ms with k_eik_sweep, 2.3 ms here, bound by the fields'
 // stream (9.1 GB through L2 and DRAM at 3.6 TB/s) and the latency of its loads,
 // 4 to 5 problems a scheduler at 122 registers; ten problems' worth of L2
 // prefetch did not help (2.64 -> 2.78 ms), and keeping three tiles in turn

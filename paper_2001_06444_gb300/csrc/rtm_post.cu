@@ -95,8 +95,8 @@ __global__ void k_filter(const float *stack_all, const float *comp_all, int nz, 
 // Two forms.  The general one sums in FP64, two passes, and sorts each pixel's
 // column (bitonic).  It is bound by FP64 arithmetic, which this device runs at
 // about 1/64 of the FP32 rate (5 FP64 operations a value), and by the sort:
-// 0.70 ms for 64 x 597,051.  The other (n <= kFastN, every value of the block
-// finite) takes one pixel per thread and no FP64 operation per value:
+// 0.70 ms for 64 x 597,051.  The other (3 to kFastN images, every value of the
+// block finite) takes one pixel per thread and no FP64 operation per value:
 //   - each value becomes an integer X on a grid 2^55 below the pixel's largest
 //     power of two, so sum X is exact in 64 bits (a pixel with a value more than
 //     2^31 times smaller than its largest, which the grid would cut, sums in FP64);

@@ -165,9 +165,11 @@ __device__ __forceinline__ float4 update4_pre(const float4 *zc, const float4 &xl
 // What stays in registers depends on R: up to 3 rows a thread keep the sponge's
 // products (PRE), up to 4 keep num, den and the next snapshot (HOLD); beyond,
 // the sponge is evaluated from its factors and num and den go through L2 at
-// imaging steps.  T: threads at most, 384 (168 registers each) or, for grids that
-// do not fit them, 512 (128 registers, some of them spilled: a 32-item phase of
-// 201 x 101 in 4 blocks takes 2.9-3.7 us a step with 512 threads, 2.6-3.2 with 384).
+// imaging steps.  T: threads at most, 384 (168 registers each; backward phases of 3,
+// 4 and 6 rows spill 120, 96 and 8 bytes) or, for grids that do not fit them, 512
+// (128 registers; every phase spills, backward 232 bytes with 5 rows and 500 with 6:
+// a 32-item phase of 201 x 101 in 4 blocks takes 2.9-3.7 us a step with 512 threads,
+// 2.6-3.2 with 384).
 template <int MODE, int R, int T>
 __global__ void __launch_bounds__(T, 1) k_resident(const __grid_constant__ ResArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
