@@ -673,10 +673,11 @@ constexpr size_t kRowMost = size_t(4) << 30;
 // 1.56 / 1.66, of 40 x 100 (fewer than 8) 1.81 / 1.66, of 64 x 200 7.09 / 5.35,
 // of 88 x 426 (one an SM) 78.6 / 26.6.
 //
-// False, too, for many problems of tall grids: the skewed copies pad every tile
-// row by the lanes' offsets (1500 x 40: 50 times its nodes, 24 MB a problem), and
-// every sweep streams them, at a cost a quad that grows with the warps of a
-// problem, while k_eik_sweep costs about the same a node whatever the shape.
+// False, too, for many problems of tall grids (unless any_shape): the skewed
+// copies pad every tile row by the lanes' offsets (1500 x 40: 50 times its nodes,
+// 24 MB a problem), and every sweep streams them, at a cost a quad that grows with
+// the warps of a problem, while k_eik_sweep costs about the same a node whatever
+// the shape.
 // Whole calls, ms, rows / sweeps: while all copies stay within 2 GB the rows win
 // everywhere (1500 x 40 x 100: 9.0 / 10.2); beyond 4 GB by pad (quads x 4 / nodes)
 // times warps: 600 x 200 x 4800 (27) 45.2 / 60.0, 500 x 100 x 4800 (30) 24.5 / 25.5,
@@ -685,7 +686,7 @@ constexpr size_t kRowMost = size_t(4) << 30;
 // 58.1 / 18.3, 1500 x 40 x 4800 (600) 460 / 33.  Problems of two warps never lose
 // (129 x 8 x 4800: 1.37 / 1.75).
 static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flags, int sms,
-                     int smem_cta, int smem_sm, size_t scratch) {
+                     int smem_cta, int smem_sm, size_t scratch, bool any_shape) {
   if (!row_geo(nz, nx, p.g)) return false;
   const RowGeo &g = p.g;
   const int base = g.map_bytes + g.ring_bytes;
@@ -701,7 +702,7 @@ static bool row_plan(RowPlan &p, int nz, int nx, int nsample, int nsrc, int flag
     return false;
   p.smem = base + (p.resident ? g.field_bytes : 0);
   const size_t per = 2 * (size_t)g.quads * sizeof(float4);  // both copies
-  if (!p.resident && g.W > 2 && (size_t)problems > kRowMost / per &&
+  if (!any_shape && !p.resident && g.W > 2 && (size_t)problems > kRowMost / per &&
       4ll * g.quads * g.W > 33ll * nz * nx)
     return false;
   const size_t per_sample = per + (p.resident ? 0 : per * nsrc);
@@ -907,27 +908,33 @@ extern "C" int rtm_eikonal(rtm_ctx *ctx, int nz, int nx, double dz, double dx, i
   // half as many problems, down to one, and then the diagonal sweeps, which need none
   // but the bare fields
   RowPlan plan;
-  bool rows = false;
-  for (size_t scratch = kRowScratch; !getenv("RTM_EIK_TILE");) {
-    if (!row_plan(plan, nz, nx, nsample, nsrc, flags, sms, smem_cta, smem_sm, scratch)) break;
-    cudaError_t e = dslow.alloc(ctx, plan.slow_bytes, st);
-    if (e == cudaSuccess) e = dwork.alloc(ctx, plan.work_bytes, st);
-    if (e == cudaSuccess) {
-      rows = true;
-      break;
+  auto take_rows = [&](bool any_shape) -> bool {
+    for (size_t scratch = kRowScratch; !getenv("RTM_EIK_TILE");) {
+      if (!row_plan(plan, nz, nx, nsample, nsrc, flags, sms, smem_cta, smem_sm, scratch, any_shape))
+        break;
+      if (dslow.alloc(ctx, plan.slow_bytes, st) == cudaSuccess &&
+          dwork.alloc(ctx, plan.work_bytes, st) == cudaSuccess)
+        return true;
+      cudaGetLastError();
+      dslow.release();
+      dwork.release();
+      if (plan.group == 1 && (plan.resident || plan.chunk == 1)) break;
+      scratch = std::min(scratch, plan.slow_bytes + plan.work_bytes) / 2;
     }
-    cudaGetLastError();
-    dslow.release();
-    dwork.release();
-    if (e != cudaErrorMemoryAllocation) EIK_CU(e);
-    if (plan.group == 1 && (plan.resident || plan.chunk == 1)) break;
-    scratch = std::min(scratch, plan.slow_bytes + plan.work_bytes) / 2;
+    return false;
+  };
+  bool rows = take_rows(false);
+  if (!rows && !fields && !resident) {  // the off-chip work fields of all problems
+    const cudaError_t e = dfields.alloc(ctx, fbytes, st);
+    if (e == cudaSuccess) {
+      df = dfields.as<float>();
+    } else {  // more than the device has: groups of the row-owning solver, whatever the grid
+      cudaGetLastError();
+      rows = take_rows(true);
+      if (!rows) EIK_CU(e);
+    }
   }
   if (!rows) {
-    if (!fields && !resident) {  // the off-chip work fields
-      EIK_CU(dfields.alloc(ctx, fbytes, st));
-      df = dfields.as<float>();
-    }
     EIK_CU(dslow.alloc(ctx, vbytes, st));
     EIK_CU(launch_eik_slowness(v, (long long)nsample * N, dslow.as<float>(), st));
   }

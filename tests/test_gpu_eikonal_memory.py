@@ -55,3 +55,22 @@ def test_a_nearly_full_device():
             del hog
             torch.cuda.empty_cache()
     assert torch.equal(got, want) and it2 == it
+
+
+def test_a_nearly_full_device_and_a_tall_grid():
+    # 1600 problems of 1500 x 40 go to the diagonal sweeps, whose fields are 384 MB; with
+    # less left they come in groups to the row-owning solver
+    vel = _models(1, 1500, 40)
+    with rtm.Context(0) as ctx:
+        want, _, it = _solve(ctx, vel, 1600)
+    with rtm.Context(0) as ctx:
+        _solve(ctx, vel, 2)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - (300 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            got, _, it2 = _solve(ctx, vel, 1600)
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+    assert torch.equal(got, want) and it2 == it
