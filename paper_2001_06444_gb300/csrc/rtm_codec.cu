@@ -786,7 +786,8 @@ __device__ __forceinline__ bool decode_block(R &rd, const unsigned char *ktab,
   // of its kept interval.  Fixed accuracy takes a rolled loop over the
   // members (one trip per member, so lanes with as many members stay in
   // step), the coefficients through the block's place in shared memory, qs[(j /
-  // 4) PITCH + j % 4], j in block order (it comes zeroed); lossless keeps the unrolled register form (64-bit coefficients).
+  // 4) PITCH + j % 4], j in block order (it comes zeroed); lossless keeps the
+  // unrolled register form (64-bit coefficients).
   using S = typename std::conditional<LL, long long, int>::type;
   S q[16];
   long long qw[16];
@@ -1085,7 +1086,8 @@ k_cz_decode(const __grid_constant__ DecArgs a) {
   __shared__ unsigned char s_sfx[16][kDec];
   __shared__ int s_next;
   constexpr int PITCH = DIRECT ? kDirPitch : kOutPitch;
-  constexpr u32 kUnit = DIRECT ? kSeg : kWin, kUnits = kSeg / kUnit;  // blocks of a unit, units of a segment
+  // blocks of a unit (a segment or a window), units of a segment
+  constexpr u32 kUnit = DIRECT ? kSeg : kWin, kUnits = kSeg / kUnit;
   const int tid = threadIdx.x, lane = tid & 31;
   const u64 nunit = (u64)a.count * a.nseg * kUnits;
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1099,7 +1101,8 @@ k_cz_decode(const __grid_constant__ DecArgs a) {
       continue;  // (uniform: another mode's stream, or none)
     u32 cnt[kSegWins];  // entries of the unit's windows (one: cnt[0])
 #pragma unroll
-    for (int k = 0; k < kSegWins; ++k) cnt[k] = k < (DIRECT ? kSegWins : 1) ? a.wincount[seg * kSegWins + w + k] : 0u;
+    for (int k = 0; k < kSegWins; ++k)
+      cnt[k] = k < (DIRECT ? kSegWins : 1) ? a.wincount[seg * kSegWins + w + k] : 0u;
     const int n = (int)(cnt[0] + cnt[1] + cnt[2] + cnt[3]);
     if (tid == 0) s_next = 0;
     // rows of the unit, a warp per row (edge blocks clipped)
